@@ -277,11 +277,13 @@ int mc_get_info(mc_job *job, mc_info *info);
 
 /* Choose how chains map to the GPU (placement 0 = lattice rows in
  * registers, L <= 32; 1 = shared memory; 2 = global memory with the rows
- * streamed through registers, L = 96, 100, 128 -- the default at L = 96,
- * where the threshold table then fits in shared memory, and with more than
- * 8 chains a warp at L = 100, 128; the joint's replays of such a job use
- * shared memory), chains per warp 1..32, warps per block 1..4.  The
- * dynamics and all results are independent of this choice. */
+ * streamed through registers, L = 96, 100, 128; the joint's replays of such
+ * a job use shared memory), chains per warp 1..32, warps per block 1..4.
+ * Placement 1 with one chain a warp resolves the 32 sites of a lattice word
+ * together, a site a lane (the default unless there are several chains a
+ * scheduler; the blocks are then sized by the library, whatever
+ * warps_per_block says).  The dynamics and all results are independent of
+ * this choice. */
 int mc_set_launch_shape(mc_job *job, int placement, int chains_per_warp, int warps_per_block);
 
 /* `iterations` weight iterations (round of n_sweeps sweeps, joint, weight
@@ -347,8 +349,8 @@ int mc_sync(mc_job *job);
  *             so that round r of a job started at t0 = 0 uses t0 = r*M.
  * Work is queued on cuda_stream (NULL = legacy default stream); returns
  * without waiting.  The launch shape is the library's default for L and
- * n_chains (see mc_set_launch_shape; at L = 96, and at L = 100, 128 with
- * more than 8 chains a warp, the lattices are swept in place in d_spins).
+ * n_chains (see mc_set_launch_shape; with placement 2 the lattices are
+ * swept in place in d_spins).
  * Scratch: the threshold table lives in one fixed
  * 320 KiB device array (L <= 128) that the library holds on every device
  * until the process exits; L > 128 is rejected with MC_EINVAL.  The first

@@ -195,6 +195,8 @@ MC_CHAIN_UNIT(chain_kernels_smem_L96);
 MC_CHAIN_UNIT(chain_kernels_smem_L100);
 MC_CHAIN_UNIT(chain_kernels_smem_L128);
 #undef MC_CHAIN_UNIT
+// generation with one chain per warp (any L; shape kPlaceSmem with one chain a warp)
+cudaError_t chain_kernels_warp(const DevJob& j, uint64_t t0, int64_t S, bool trace, cudaStream_t st);
 // the joint of a recorded round (any L): kernels without lattices or table
 cudaError_t chain_kernels_record(const DevJob& j, uint64_t t0, int64_t S, uint32_t r, cudaStream_t st);
 

@@ -8,6 +8,7 @@
 
 #include "mc_chain_kernels.cuh"
 #include "mc_scan_fsm.cuh"
+#include "mc_warp_chain.cuh"
 
 namespace mcgpu {
 
@@ -866,7 +867,8 @@ bool shape_supported(int L, const LaunchShape& s) {
   return plan_bytes(L, s, false, true) <= kMaxSmem;
 }
 
-LaunchShape default_shape(int L, int p, int num_sms) {
+// One chain a lane: the shape when there are too many chains for one a warp.
+static LaunchShape lane_shape(int L, int p, int num_sms) {
   LaunchShape s;
   // lattice rows in registers for L <= 32, except L = 24 and 32, whose
   // compile-time shared-memory bodies measured faster (L = 32, 16384 chains:
@@ -886,6 +888,11 @@ LaunchShape default_shape(int L, int p, int num_sms) {
   return s;
 }
 
+LaunchShape default_shape(int L, int p, int num_sms) {
+  if (warp_chain_better(L, p, num_sms)) return LaunchShape{kPlaceSmem, 1, 4};   // one chain a warp
+  return lane_shape(L, p, num_sms);
+}
+
 // Densest shape for L and p: as many chains per warp as there are (up to 32),
 // keeping the threshold table in shared memory if the default shape has it
 // there.  The time of a round is set by the latency of one chain, which a
@@ -893,7 +900,7 @@ LaunchShape default_shape(int L, int p, int num_sms) {
 // a job shaped this way takes the same time on far fewer warps -- the rest
 // of the GPU stays free for other jobs (the server uses it).
 LaunchShape dense_shape(int L, int p, int num_sms) {
-  LaunchShape def = default_shape(L, p, num_sms);
+  LaunchShape def = lane_shape(L, p, num_sms);
   // full warps at L = 100, 128 keep their lattices in global memory: a block
   // of 128 chains then needs only the histogram's shared memory, so blocks
   // of other jobs fit beside it
@@ -925,6 +932,7 @@ static bool replay_fits(int L, const LaunchShape& s) {
 static LaunchShape join_shape(int L, const LaunchShape& gen_shape) {
   LaunchShape gen = gen_shape;
   if (gen.placement == kPlaceGlobal) gen.placement = kPlaceSmem;   // replays restore into shared memory
+  if (gen.cpw == 1 && L <= 32 && L != 24 && L != 32) gen.placement = kPlaceReg;   // (one chain a warp)
   LaunchShape best = gen;
   int best_lanes = 0;
   bool best_ts = false;
@@ -1069,6 +1077,7 @@ cudaError_t join_finalize(const DevJob& j, int64_t S, cudaStream_t st) {
 
 static cudaError_t dispatch(const DevJob& j, const LaunchShape& s, bool gen, uint64_t t0, int64_t S, bool trace,
                             uint32_t r, cudaStream_t st) {
+  if (gen && s.placement == kPlaceSmem && s.cpw == 1) return chain_kernels_warp(j, t0, S, trace, st);
   if (s.placement == kPlaceReg) {
     if (j.L <= 16) return chain_kernels_reg_a(j, s, gen, t0, S, trace, r, st);
     if (j.L <= 28) return chain_kernels_reg_b(j, s, gen, t0, S, trace, r, st);
