@@ -7,6 +7,7 @@
 #include <type_traits>
 
 #include "mc_chain.cuh"
+#include "mc_height.cuh"
 #include "mc_internal.h"
 
 namespace mcgpu {
@@ -512,11 +513,6 @@ __global__ void __launch_bounds__(128) summary_kernel(const DevJob j, const int 
   const long long items = static_cast<long long>(nchains) * j.ck_K;
   const SmemPlan sp = smem_plan(j.L, Factory::kPlacement, cpw, blockDim.x >> 5, TSMEM, false);
   BlockCtx b = block_setup<TSMEM>(j, sp, cpw, 0, false);
-  // a recorded round: every lane keeps a window of levels in shared memory
-  constexpr int W = IsRec<Factory>::value ? 64 : 0;
-  __shared__ uint32_t s_win[W > 0 ? W * kWinStride : 1];
-  if constexpr (W > 0)
-    for (int q = threadIdx.x; q < W * kWinStride; q += blockDim.x) s_win[q] = 0xFFFFFFFFu;
   __syncthreads();
   unsigned long long* queue = reinterpret_cast<unsigned long long*>(&j.stats[kStatQueueSearch]);
   long long searched = 0;
@@ -529,8 +525,7 @@ __global__ void __launch_bounds__(128) summary_kernel(const DevJob j, const int 
     if (b.lane < cpw && item < items) {
       const int seg = static_cast<int>(item / nchains);
       const int i = j.perm[f + static_cast<int>(item % nchains)];
-      SummaryHook<W> hk;
-      if constexpr (W > 0) hk.win = s_win + threadIdx.x;
+      SummaryHook<0> hk;
       hk.umin = j.tj + static_cast<size_t>(i) * j.np1;
       hk.k = static_cast<int64_t>(seg) * j.seg_len;
       hk.chain = static_cast<uint32_t>(i);
@@ -544,13 +539,99 @@ __global__ void __launch_bounds__(128) summary_kernel(const DevJob j, const int 
       hk.flag = false;
       hk.done = false;
       const int64_t k_begin = hk.k;
-      if constexpr (IsRec<Factory>::value) record_segment(j, i, seg, S, hk);
-      else replay_segment<Factory>(j, b, i, seg, t0, S, hk);
+      replay_segment<Factory>(j, b, i, seg, t0, S, hk);
       hk.flush();
-      hk.drain();
       atomicMin(&j.summ[i], hk.lo);
       atomicMax(&j.summ[j.p + i], hk.hi);
       if (hk.flag) atomicOr(&j.summ[2 * j.p + i], 1);
+      searched += hk.k - k_begin;
+    }
+    __syncwarp();
+  }
+  if (searched)
+    atomicAdd(reinterpret_cast<unsigned long long*>(&j.stats[kStatSearched]), static_cast<unsigned long long>(searched));
+}
+
+// A lower bound of every chain's second-best v before the pass over its
+// samples, so that the pass's filter is tight from the start (without it each
+// segment's first samples pass: 15 of 2048 a lane, a quarter of the warps'
+// iterations): the second best of up to 1024 samples spread over the chain,
+// one warp a chain.
+__device__ __forceinline__ void height_top2(float v, float& best, float& second) {
+  second = fmaxf(second, fminf(best, v));
+  best = fmaxf(best, v);
+}
+template <class Factory>
+__global__ void __launch_bounds__(128) height_seed_kernel(const DevJob j, const int64_t S, const uint32_t r) {
+  if (j.stats[kStatPending] == 0) return;
+  const int f = static_cast<int>(j.stats[kStatFirstPending]);
+  const float* wl = reinterpret_cast<const float*>(j.lvcnt);
+  const int lane = threadIdx.x & 31;
+  const int64_t M = S * j.N;
+  const int n = static_cast<int>(min(static_cast<int64_t>(1024), max(static_cast<int64_t>(32), M / 32))) & ~31;
+  const int nwarps = (gridDim.x * blockDim.x) >> 5;
+  for (int q = f + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5); q < j.p; q += nwarps) {
+    const int i = j.perm[q];
+    float best = height_none().best, second = best;
+    for (int a = lane; a < n; a += 32) {
+      const int64_t k = M >= n ? static_cast<int64_t>(a) * (M / n) : a;   // distinct samples (0-based)
+      if (k >= M) break;
+      const uint4 v = philox4x32_10(make_uint4(static_cast<uint32_t>(k >> 2), r, static_cast<uint32_t>(i), kTagJoint),
+                                    j.key0, j.key1);
+      const uint32_t u = uint4_word(v, static_cast<uint32_t>(k & 3));
+      height_top2(wl[j.rec[rec_index(i, k, M)]] + height_draw(u), best, second);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const float b2 = __shfl_xor_sync(0xFFFFFFFFu, best, o), s2 = __shfl_xor_sync(0xFFFFFFFFu, second, o);
+      height_top2(b2, best, second);
+      second = fmaxf(second, s2);
+    }
+    if (lane == 0) heights(j)[i].second = second;
+  }
+}
+
+// Heights of the chains from the first pending one on, for a recorded round
+// (mc_height.cuh): items and queue as in summary_kernel, the levels' weights
+// in shared memory.
+template <class Factory>
+__global__ void __launch_bounds__(128) height_kernel(const DevJob j, const int cpw, const uint64_t t0, const int64_t S,
+                                                     const uint32_t r) {
+  if (j.stats[kStatPending] == 0) return;
+  const int f = static_cast<int>(j.stats[kStatFirstPending]);
+  const int nchains = j.p - f;
+  const long long items = static_cast<long long>(nchains) * j.ck_K;
+  const SmemPlan sp = smem_plan(j.L, Factory::kPlacement, cpw, blockDim.x >> 5, false, true);   // "histogram": weights
+  BlockCtx b = block_setup<false>(j, sp, cpw, 0, false);
+  float* wl = reinterpret_cast<float*>(b.hist);
+  const float* g = reinterpret_cast<const float*>(j.lvcnt);
+  for (int m = threadIdx.x; m < j.np1; m += blockDim.x) wl[m] = g[m];
+  __syncthreads();
+  const float slack = height_slack(j);
+  unsigned long long* queue = reinterpret_cast<unsigned long long*>(&j.stats[kStatQueueSearch]);
+  long long searched = 0;
+  for (;;) {
+    long long base = 0;
+    if (b.lane == 0) base = static_cast<long long>(atomicAdd(queue, static_cast<unsigned long long>(cpw)));
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    if (base >= items) break;
+    const long long item = base + b.lane;
+    if (b.lane < cpw && item < items) {
+      const int seg = static_cast<int>(item / nchains);
+      const int i = j.perm[f + static_cast<int>(item % nchains)];
+      HeightHook hk;
+      hk.wl = wl;
+      hk.entry = heights(j) + i;
+      hk.slack = slack;
+      hk.k = static_cast<int64_t>(seg) * j.seg_len;
+      hk.chain = static_cast<uint32_t>(i);
+      hk.r = r;
+      hk.k0 = j.key0;
+      hk.k1 = j.key1;
+      hk.done = false;
+      hk.begin();
+      const int64_t k_begin = hk.k;
+      record_segment(j, i, seg, S, hk);
+      if (hk.h.m != kNoLevel) height_store_max(heights(j) + i, hk.h);
       searched += hk.k - k_begin;
     }
     __syncwarp();
@@ -883,17 +964,34 @@ inline cudaError_t launch_join_t(const DevJob& j, const LaunchShape& s, uint64_t
     // new k's, and the ordinary passes catch what the scan left
     if ((e = pass(j.passes_scan, true)) != cudaSuccess) return e;
     if ((e = join_mark(j, st, false)) != cudaSuccess) return e;
-    if ((e = join_summary_init(j, st)) != cudaSuccess) return e;
-    if ((e = join_reset_queue(j, st)) != cudaSuccess) return e;
-    auto ks = summary_kernel<F, TS>;
-    if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes))) !=
-        cudaSuccess)
-      return e;
-    const unsigned grid_sum = static_cast<unsigned>(
-        std::min<long long>(blocks_for(items, per_block), resident_blocks(ks, 32 * s.wpb, bytes)));
-    ks<<<grid_sum, 32 * s.wpb, bytes, st>>>(j, s.cpw, t0, S, r);
-    launches_add(1);
-    if ((e = join_scan(j, st)) != cudaSuccess) return e;
+    if constexpr (IsRec<F>::value) {
+      if ((e = join_height_init(j, st)) != cudaSuccess) return e;
+      height_seed_kernel<F><<<std::min(2432u, blocks_for(j.p, 4)), 128, 0, st>>>(j, S, r);
+      launches_add(1);
+      if ((e = join_reset_queue(j, st)) != cudaSuccess) return e;
+      auto kh = height_kernel<F>;
+      const size_t hbytes = plan_bytes(j.L, s, false, true);
+      if ((e = cudaFuncSetAttribute(kh, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(hbytes))) !=
+          cudaSuccess)
+        return e;
+      const unsigned grid_h = static_cast<unsigned>(
+          std::min<long long>(blocks_for(items, per_block), resident_blocks(kh, 32 * s.wpb, hbytes)));
+      kh<<<grid_h, 32 * s.wpb, hbytes, st>>>(j, s.cpw, t0, S, r);
+      launches_add(1);
+      if ((e = join_height_scan(j, st)) != cudaSuccess) return e;
+    } else {
+      if ((e = join_summary_init(j, st)) != cudaSuccess) return e;
+      if ((e = join_reset_queue(j, st)) != cudaSuccess) return e;
+      auto ks = summary_kernel<F, TS>;
+      if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes))) !=
+          cudaSuccess)
+        return e;
+      const unsigned grid_sum = static_cast<unsigned>(
+          std::min<long long>(blocks_for(items, per_block), resident_blocks(ks, 32 * s.wpb, bytes)));
+      ks<<<grid_sum, 32 * s.wpb, bytes, st>>>(j, s.cpw, t0, S, r);
+      launches_add(1);
+      if ((e = join_scan(j, st)) != cudaSuccess) return e;
+    }
     if ((e = join_tj_list(j, st)) != cudaSuccess) return e;
     if ((e = search(1, 0)) != cudaSuccess) return e;
     if ((e = join_select(j, true, st)) != cudaSuccess) return e;

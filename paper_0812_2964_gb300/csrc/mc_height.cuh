@@ -1,0 +1,163 @@
+// The joint's exact path for recorded rounds: acceptance heights.
+//
+// Chain i keeps samples for input level x iff some sample k passes the joint
+// test u_k <= thr(W[m_k] - W[x]) (Sec. 2 step 4), that is iff
+// u_k < 2^32 exp(W[m_k] - W[x]), that is iff
+//     W[x] < max_k v_k,   v_k = W[m_k] - ln(u_k / 2^32).
+// So one number per chain -- its height, the largest v_k -- answers every
+// input, and the serial rule over chains becomes "the next chain that keeps
+// samples after chain q is the first one whose height exceeds W[m_q]": all
+// those successors are found independently, and the chains that keep
+// samples are the ones reached from the round's input by following them
+// (pointer doubling).  Nothing is carried chain by chain.
+//
+// Heights are kept in floating point, so decisions close to the line are
+// made on the sample itself: the chain's entry holds the best sample's level
+// and uniform (tested exactly, by the threshold function of the joint) and the
+// second-best v, whose upper estimate says whether any other sample could
+// pass where the best does not.  What neither settles (the two samples and
+// W[x] within rounding of one another) is undecided, and the ordinary
+// resolution passes finish from that chain on.
+//
+// What bounds the pass over the samples: a Philox word (10 operations), one
+// load of the level's weight from shared memory, and a filter of six
+// operations (one of them an exponential) that lets a sample through to the
+// exact bookkeeping only if it may be among the chain's two best.
+#pragma once
+#include "mc_chain.cuh"
+#include "mc_internal.h"
+
+namespace mcgpu {
+
+// best and second in log2 units relative to the joint's reference weight:
+// (W[m] - Wref) / ln 2 + 32 - log2 u
+struct alignas(16) Height {
+  uint32_t m, u;        // best sample: its level (kNoLevel: none yet) and joint uniform
+  float best, second;   // the two largest v
+};
+constexpr uint32_t kNoLevel = 0xFFFFFFFFu;
+// |height_value - exact v| stays below half of this: log2 of a float (relative
+// error 2^-22 of at most 32, plus the rounding of u) and the rounding of W
+constexpr double kHeightEps = 1e-4;
+
+#ifdef __CUDACC__
+
+__device__ __forceinline__ Height* heights(const DevJob& j) { return reinterpret_cast<Height*>(j.summ); }
+
+__device__ __forceinline__ Height height_none() {
+  Height h;
+  h.m = kNoLevel;
+  h.u = 0u;
+  h.best = h.second = __int_as_float(static_cast<int>(0xFF800000));
+  return h;
+}
+
+// -log2(u / 2^32); a uniform of 0 passes every test
+__device__ __forceinline__ float height_draw(uint32_t u) {
+  return u ? 32.0f - __log2f(static_cast<float>(u)) : __int_as_float(0x7F800000);
+}
+
+// v of the entry's best sample, from its level and uniform
+__device__ __forceinline__ double height_value(const DevJob& j, const Height& h) {
+  if (h.m == kNoLevel) return __longlong_as_double(static_cast<long long>(0xFFF0000000000000ull));
+  if (h.u == 0u) return __longlong_as_double(0x7FF0000000000000ll);
+  return j.W[h.m] + static_cast<double>(height_draw(h.u)) * 0.6931471805599453;
+}
+
+// Error of the float weights (log2 units): twice the rounding of the largest.
+__device__ __forceinline__ float height_slack(const DevJob& j) {
+  return 0.01f + __int_as_float(static_cast<int>(j.stats[kStatWeightMax])) * 0x1p-22f;
+}
+
+// No other sample of the chain has a larger v.
+__device__ __forceinline__ double height_second(const Height& h, double wref, float slack) {
+  return wref + (static_cast<double>(h.second) + slack) * 0.6931471805599453;
+}
+
+__device__ __forceinline__ Height height_load(const Height* p) {
+  const uint4 v = __ldcg(reinterpret_cast<const uint4*>(p));
+  Height h;
+  h.m = v.x;
+  h.u = v.y;
+  h.best = __uint_as_float(v.z);
+  h.second = __uint_as_float(v.w);
+  return h;
+}
+
+// The entry of two disjoint sets of samples.
+__device__ __forceinline__ Height height_merge(const Height& a, const Height& b) {
+  Height r = a.best >= b.best ? a : b;
+  r.second = fmaxf(fminf(a.best, b.best), fmaxf(a.second, b.second));
+  return r;
+}
+
+__device__ __forceinline__ void height_store_max(Height* p, const Height& mine) {
+  Height cur = height_load(p);
+  for (;;) {   // (a failed exchange means another lane's succeeded: at most one retry per lane that merges)
+    const Height nw = height_merge(cur, mine);
+    if (nw.m == cur.m && nw.u == cur.u && nw.second == cur.second) return;
+    const Height old = atomicCAS(p, cur, nw);
+    if (old.m == cur.m && old.u == cur.u && __float_as_uint(old.best) == __float_as_uint(cur.best) &&
+        __float_as_uint(old.second) == __float_as_uint(cur.second))
+      return;
+    cur = old;
+  }
+}
+
+// Hook of the pass over a segment's samples.  wl[m] = (W[m] - Wref) / ln 2 as
+// a float; a sample can be among the best two only if u / 2^32 <
+// 2^(wl[m] - bl), bl below the second-best v found so far by more than the
+// float weights' and the exponential's errors.
+struct HeightHook {
+  const float* wl;      // shared memory
+  const Height* entry;  // the chain's entry (polled for the other segments' second best)
+  float slack, bl;
+  int64_t k;
+  uint32_t chain, r, k0, k1;
+  uint32_t uj[32];
+  Height h;
+  bool done;            // never set: the whole segment is read
+  __device__ __forceinline__ void begin() {
+    h = height_none();
+    bl = height_load(entry).second - slack;
+  }
+  __device__ __forceinline__ void poll() { bl = fmaxf(bl, height_load(entry).second - slack); }
+  __device__ __forceinline__ void word(int nb) {
+    joint_fill(uj, nb, k, r, chain, k0, k1);
+    k += nb;
+  }
+  __device__ __forceinline__ void sample(int m4, int b) {
+    const float w = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(wl) + m4);
+    float e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(w - bl));
+    // 1 + u / 2^32 rounded down to 23 bits, against 1 + e and the rounding
+    const float u1 = __uint_as_float(__funnelshift_r(uj[b], 0x7Fu, 9));
+    if (!(u1 >= e + 1.0000005f)) {
+      const float v = uj[b] ? w + height_draw(uj[b]) : __int_as_float(0x7F800000);
+      if (v > h.second) {
+        const bool top = v > h.best;
+        h.second = top ? h.best : v;
+        if (top) {
+          h.best = v;
+          h.m = static_cast<uint32_t>(m4) >> 2;
+          h.u = uj[b];
+        }
+        bl = fmaxf(bl, h.second - slack);
+      }
+    }
+  }
+};
+
+// Whether the chain whose entry is h keeps samples for an input level of
+// weight wx: 1 yes, 0 no, 2 undecided.
+__device__ __forceinline__ int height_accepts(const DevJob& j, const Height& h, double wx, double wref, float slack) {
+  const double v = height_value(j, h);
+  const double eps = kHeightEps + 1e-13 * fabs(wx);
+  if (v > wx + eps) return 1;
+  if (!(v < wx - eps) && h.m != kNoLevel && h.u <= threshold_det(__dsub_rn(j.W[h.m], wx))) return 1;
+  return height_second(h, wref, slack) < wx - eps ? 0 : 2;
+}
+
+#endif  // __CUDACC__
+
+}  // namespace mcgpu

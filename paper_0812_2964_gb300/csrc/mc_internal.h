@@ -47,7 +47,8 @@ struct DevJob {
   unsigned long long* kmin;  // [p] earliest accepted sample found so far for the chain's input (kNoHit: none)
   int2* plist;         // [p*kcap] (chain, segment) work list of the prefix pass
   int32_t* summ;       // [5][p] summary pass: lowest and highest level visited, flag; then
-                       // [p][8] bytes: the exact scan's answers for candidate inputs
+                       // [p][8] bytes: the exact scan's answers for candidate inputs.  A recorded
+                       // round instead keeps every chain's height there (16 bytes, mc_height.cuh)
   uint8_t* visited;    // [np1] 1 once a weight update has seen h > 0 at the level
   int32_t* perm;       // [p] chain at each position of the joint (identity unless ordered)
   int32_t* lvcnt;      // [np1] scratch of the energy ordering
@@ -128,7 +129,8 @@ enum StatIndex : int {
   kStatFirstPending = 13,// lowest chain queued by the last mark pass (p if none)
   kStatScanned = 14,     // chains whose input the exact scan settled (last joint)
   kStatNoHit = 15,       // chains listed in work2
-  kStatCount = 16
+  kStatWeightMax = 16,   // largest |W - Wref| / ln 2 of the level weights, as float bits (recorded rounds' exact path)
+  kStatCount = 17
 };
 
 // ---- kernels (mc_kernels.cu) ----
@@ -175,6 +177,9 @@ cudaError_t join_reset_queue(const DevJob& j, cudaStream_t st);
 cudaError_t join_finalize(const DevJob& j, int64_t S, cudaStream_t st);
 cudaError_t join_summary_init(const DevJob& j, cudaStream_t st);
 cudaError_t join_scan(const DevJob& j, cudaStream_t st);
+// the same for recorded rounds, by acceptance heights (mc_height.cuh)
+cudaError_t join_height_init(const DevJob& j, cudaStream_t st);
+cudaError_t join_height_scan(const DevJob& j, cudaStream_t st);
 
 // per-unit launchers of the templated chain kernels (mc_inst_*.cu)
 #define MC_CHAIN_UNIT(name)                                                                              \

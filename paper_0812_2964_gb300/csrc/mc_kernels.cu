@@ -330,6 +330,7 @@ __global__ void clear_stats_kernel(const DevJob j) {
     j.stats[kStatWholeFill] = 0;
     j.stats[kStatScanned] = 0;
     j.stats[kStatFirstPending] = j.p;
+    j.stats[kStatWeightMax] = 0;
   }
   // earliest accepted sample of each chain: none found yet
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < j.p; i += gridDim.x * blockDim.x) j.kmin[i] = kNoHit;
@@ -626,6 +627,212 @@ __global__ void __launch_bounds__(1024) scan_kernel(const DevJob j) {
       if (j.k[j.perm[q]] < 0) j.work[s_count++] = j.perm[q];
     j.stats[kStatPending] = s_count;
     j.stats[kStatScanned] = static_cast<long long>(s_scanned);
+  }
+}
+
+// ------------------------------------------------------------------ heights (mc_height.cuh)
+// Set-up: empty entries for the chains from the first pending one on, and
+// the levels' weights as floats relative to the weight of a level met there.
+__global__ void height_init_kernel(const DevJob j) {
+  if (j.stats[kStatPending] == 0) return;
+  const int f = static_cast<int>(j.stats[kStatFirstPending]);
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+  const double wref = j.W[j.m[j.perm[f]]];
+  float* wl = reinterpret_cast<float*>(j.lvcnt);
+  float big = 0.0f;
+  for (int m = t; m < j.np1; m += nt) {
+    const float v = static_cast<float>((j.W[m] - wref) * 1.4426950408889634);
+    wl[m] = v;
+    if (fabsf(v) < CUDART_INF_F) big = fmaxf(big, fabsf(v));
+  }
+  if (big > 0.0f) atomicMax(&j.stats[kStatWeightMax], static_cast<long long>(__float_as_int(big)));
+  for (int q = f + t; q < j.p; q += nt) heights(j)[j.perm[q]] = height_none();
+}
+
+// Scratch of the scan in tj (its rows are rebuilt for the chains searched
+// next): values of the heights by position (the larger of the two samples'), their maxima over 32 and 1024
+// positions, successors (one more: the round's input), two jump arrays and
+// the marks -- at most 21 p + 40 of the 4 (N + 1) p >= 68 p bytes.
+struct HeightScratch {
+  double *val, *max32, *max1024;
+  int32_t *next, *jump;
+  uint8_t* mark;
+};
+__device__ __forceinline__ HeightScratch height_scratch(const DevJob& j) {
+  HeightScratch s;
+  const int p = j.p;
+  s.val = reinterpret_cast<double*>(j.tj);
+  s.max32 = s.val + p;
+  s.max1024 = s.max32 + (p + 31) / 32;
+  s.next = reinterpret_cast<int32_t*>(s.max1024 + (p + 1023) / 1024);
+  s.jump = s.next + p + 1;
+  s.mark = reinterpret_cast<uint8_t*>(s.jump + p + 1);
+  return s;
+}
+
+__global__ void __launch_bounds__(1024) height_value_kernel(const DevJob j) {
+  if (j.stats[kStatPending] == 0) return;
+  __shared__ double s_max[32];
+  const HeightScratch hs = height_scratch(j);
+  const int f = static_cast<int>(j.stats[kStatFirstPending]);
+  const int t = threadIdx.x;
+  const double wref = j.W[j.m[j.perm[f]]];
+  const float slack = height_slack(j);
+  for (int base = blockIdx.x * 1024; base < j.p; base += gridDim.x * 1024) {
+    const int q = base + t;
+    double v = -CUDART_INF;
+    if (q >= f && q < j.p) {
+      const Height h = heights(j)[j.perm[q]];
+      v = fmax(height_value(j, h), height_second(h, wref, slack));
+    }
+    if (q < j.p) hs.val[q] = v;
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    if ((t & 31) == 0) {
+      s_max[t >> 5] = v;
+      if (q < j.p) hs.max32[q >> 5] = v;
+    }
+    __syncthreads();
+    if (t < 32) {
+      v = s_max[t];
+      for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+      if (t == 0) hs.max1024[base >> 10] = v;
+    }
+    __syncthreads();
+  }
+}
+
+// First position from q on whose chain keeps samples for an input level of
+// weight wx; p if none; p + 1 + q' if that is undecided at q'.
+__device__ __forceinline__ int height_next(const DevJob& j, const HeightScratch& hs, int q, double wx, double wref,
+                                           float slack) {
+  const double low = wx - (kHeightEps + 1e-13 * fabs(wx));
+  while (q < j.p) {
+    if ((q & 1023) == 0 && hs.max1024[q >> 10] < low) {
+      q += 1024;
+      continue;
+    }
+    if ((q & 31) == 0 && hs.max32[q >> 5] < low) {
+      q += 32;
+      continue;
+    }
+    if (!(hs.val[q] < low)) {
+      const int a = height_accepts(j, heights(j)[j.perm[q]], wx, wref, slack);
+      if (a) return a == 1 ? q : j.p + 1 + q;
+    }
+    ++q;
+  }
+  return j.p;
+}
+
+__global__ void height_next_kernel(const DevJob j) {
+  if (j.stats[kStatPending] == 0) return;
+  const HeightScratch hs = height_scratch(j);
+  const int f = static_cast<int>(j.stats[kStatFirstPending]);
+  const double wref = j.W[j.m[j.perm[f]]];
+  const float slack = height_slack(j);
+  for (int q = f + blockIdx.x * blockDim.x + threadIdx.x; q <= j.p; q += gridDim.x * blockDim.x) {
+    int nx;
+    if (q < j.p) {
+      nx = height_next(j, hs, q + 1, j.W[j.m[j.perm[q]]], wref, slack);
+    } else {   // the round's input at position f: the last level passed on, or nothing yet (kept whole)
+      const int last = j.lastacc[f];
+      const int x = last >= 0 ? j.m[j.perm[last]]
+                              : (j.stats[kStatCarryValid] ? static_cast<int>(j.stats[kStatCarry]) : -1);
+      nx = x < 0 ? f : height_next(j, hs, f, j.W[x], wref, slack);
+    }
+    hs.next[q] = nx;
+  }
+}
+
+// One block: mark the positions reached from the round's input (after k
+// doublings the marks hold the first 2^k of them), then give every position
+// its input and outcome, as scan_kernel does.
+__global__ void __launch_bounds__(1024) height_path_kernel(const DevJob j) {
+  if (j.stats[kStatPending] == 0) return;
+  __shared__ int s_tmp[1024];
+  __shared__ int s_end, s_count, s_scanned;
+  const HeightScratch hs = height_scratch(j);
+  const int t = threadIdx.x, nt = blockDim.x, p = j.p;
+  const int f = static_cast<int>(j.stats[kStatFirstPending]);
+  const int last0 = j.lastacc[f];
+  const int x0 = last0 >= 0 ? j.m[j.perm[last0]]
+                            : (j.stats[kStatCarryValid] ? static_cast<int>(j.stats[kStatCarry]) : -1);
+  if (t == 0) {
+    s_end = p;
+    s_count = 0;
+    s_scanned = 0;
+  }
+  for (int q = f + t; q < p; q += nt) hs.mark[q] = q == hs.next[p] ? 1 : 0;
+  __syncthreads();
+  int32_t *src = hs.next, *dst = hs.jump;
+  for (long long len = 1; len < p - f; len <<= 1) {
+    for (int q = f + t; q < p; q += nt) {
+      const int a = src[q];
+      if (a < p) {
+        if (hs.mark[q]) hs.mark[a] = 1;
+        dst[q] = src[a];
+      } else {
+        dst[q] = a;
+      }
+    }
+    __syncthreads();
+    int32_t* o = src;
+    src = dst;
+    dst = o;
+  }
+  // every jump now leads past the path's end: p, or p + 1 + the position whose answer is undecided
+  if (t == 0) {
+    const int start = hs.next[p];
+    const int end = start < p ? src[start] : start;
+    if (end > p) s_end = end - (p + 1);
+  }
+  __syncthreads();
+  const int stop_at = s_end;
+  // inputs: the last marked position before each, each thread a range of positions
+  const int per = (p - f + nt - 1) / nt;
+  const int lo = min(p, f + t * per), hi = min(p, lo + per);
+  int last = -1;
+  for (int q = lo; q < hi; ++q)
+    if (hs.mark[q]) last = q;
+  s_tmp[t] = last;
+  __syncthreads();
+  for (int off = 1; off < nt; off <<= 1) {
+    const int v = (t >= off) ? s_tmp[t - off] : -1;
+    __syncthreads();
+    s_tmp[t] = max(s_tmp[t], v);
+    __syncthreads();
+  }
+  int run = t > 0 ? s_tmp[t - 1] : -1;
+  int scanned = 0;
+  for (int q = lo; q < hi; ++q) {
+    const int ch = j.perm[q];
+    const int64_t kc = j.k[ch];
+    const bool keeps = hs.mark[q] != 0;
+    if (q < stop_at) {
+      const int x = run >= 0 ? j.m[j.perm[run]] : x0;
+      if (kc < 0 || j.xused[ch] != x) {   // not known for this input
+        j.xused[ch] = x;
+        if (!keeps) {
+          j.k[ch] = 0;
+        } else if (x < 0) {               // no input yet: the chain is kept whole
+          j.k[ch] = 1;
+        } else {
+          j.k[ch] = -1;                   // to be searched under the exact input
+          j.kmin[ch] = kNoHit;
+          j.work[atomicAdd(&s_count, 1)] = ch;
+        }
+        ++scanned;
+      }
+    } else if (kc < 0) {
+      j.work[atomicAdd(&s_count, 1)] = ch;   // stopped early: chains still waiting for a search keep their inputs
+    }
+    if (keeps) run = q;
+  }
+  if (scanned) atomicAdd(&s_scanned, scanned);
+  __syncthreads();
+  if (t == 0) {
+    j.stats[kStatPending] = s_count;
+    j.stats[kStatScanned] = s_scanned;
   }
 }
 
@@ -1028,6 +1235,20 @@ cudaError_t join_scan(const DevJob& j, cudaStream_t st) {
   cand_kernel<<<std::min(1024u, blocks_for(static_cast<long long>(j.p) * kScanCand * 32, 256)), 256, 0, st>>>(j);
   scan_kernel<<<1, 1024, 0, st>>>(j);
   launches_add(2);
+  return cudaGetLastError();
+}
+
+cudaError_t join_height_init(const DevJob& j, cudaStream_t st) {
+  height_init_kernel<<<std::min(256u, blocks_for(std::max(j.p, j.np1), 256)), 256, 0, st>>>(j);
+  launches_add(1);
+  return cudaGetLastError();
+}
+
+cudaError_t join_height_scan(const DevJob& j, cudaStream_t st) {
+  height_value_kernel<<<std::min(152u, blocks_for(j.p, 1024)), 1024, 0, st>>>(j);
+  height_next_kernel<<<std::min(1024u, blocks_for(j.p + 1, 128)), 128, 0, st>>>(j);
+  height_path_kernel<<<1, 1024, 0, st>>>(j);
+  launches_add(3);
   return cudaGetLastError();
 }
 
