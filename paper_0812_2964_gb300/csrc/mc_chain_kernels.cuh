@@ -7,12 +7,13 @@
 #include <type_traits>
 
 #include "mc_chain.cuh"
-#include "mc_height.cuh"
 #include "mc_internal.h"
 
 namespace mcgpu {
 
 inline unsigned blocks_for(long long n, int t) { return static_cast<unsigned>((n + t - 1) / t); }
+
+static_assert(kRecGroupStride == 4 * kRecTile, "record layout: generation and joint agree");
 
 // ------------------------------------------------------------------ runners
 // A chain's lattice during a sweep, in registers (L <= 32, one word per row;
@@ -236,18 +237,6 @@ struct RunnerFactorySmem {
   }
 };
 
-// The joint's kernels for a recorded round: levels come from the round
-// record, so there is no lattice to replay and no threshold table (the
-// launch shape's placement only sizes shared memory: none for lattices).
-struct RecF {
-  static constexpr int kPlacement = kPlaceReg;
-};
-template <class F>
-struct IsRec : std::false_type {};
-template <>
-struct IsRec<RecF> : std::true_type {};
-static_assert(kRecGroupStride == 4 * kRecTile, "record layout: generation and joint agree");
-
 // Step 2: every chain performs S sweeps (M = S N attempts) under the current
 // weight; per-level dwell counts accumulate in shared memory, then in the
 // round histogram hgen.  trace[s][c] = energy after sweep s.
@@ -381,47 +370,6 @@ __device__ __forceinline__ void replay_segment(const DevJob& j, const BlockCtx& 
   }
 }
 
-// The same samples as replay_segment, read from the round's record of
-// levels (generation stored them, layout rec_index): a hook sees word(nb)
-// before every 32 samples and sample(4 m, b) for each, in order; no
-// Metropolis replay.  The joint uniforms of a hook depend only on the
-// sample's index, so words need not follow lattice rows.  The next 32
-// samples' groups are loaded while the current ones are tested, so a lane
-// waits on memory once a segment rather than once a word.  (Segments start
-// on multiples of 16 samples and hold multiples of 16.)
-template <class Hook>
-__device__ __forceinline__ void record_segment(const DevJob& j, int i, int seg, int64_t S, Hook& hk) {
-  const int64_t M = S * j.N;
-  const int64_t k0 = static_cast<int64_t>(seg) * j.seg_len;
-  const int64_t k1 = min(M, k0 + j.seg_len);
-  // group g (samples 4g .. 4g+3) of chain i is grp[g * kRecTile]
-  const uint2* grp = reinterpret_cast<const uint2*>(j.rec + rec_index(i, 0, M));
-  uint2 v[8], nv[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q)
-    v[q] = (k0 + 4 * q < k1) ? __ldg(grp + static_cast<size_t>((k0 >> 2) + q) * kRecTile) : make_uint2(0u, 0u);
-  int words = 0;
-  for (int64_t kb = k0; kb < k1 && !hk.done; kb += 32) {
-    const int nb = static_cast<int>(min(static_cast<int64_t>(32), k1 - kb));
-    const int64_t kn = kb + 32;
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-      nv[q] = (kn + 4 * q < k1) ? __ldg(grp + static_cast<size_t>((kn >> 2) + q) * kRecTile) : make_uint2(0u, 0u);
-    hk.word(nb);
-#pragma unroll
-    for (int b = 0; b < 32; ++b) {
-      if (b < nb) {
-        const uint32_t pair = (b & 2) ? v[b >> 2].y : v[b >> 2].x;
-        const uint32_t lv = (b & 1) ? (pair >> 16) : (pair & 0xFFFFu);
-        hk.sample(4 * static_cast<int>(lv), b);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = nv[q];
-    if ((++words & 31) == 0) hk.poll();
-  }
-}
-
 // Joint search (step 4) over segments [seg_lo, seg_hi): work item (chain,
 // segment) finds the first sample inside the segment that passes the
 // Metropolis test against the chain's input level and lowers the chain's
@@ -440,8 +388,7 @@ __device__ __forceinline__ void record_segment(const DevJob& j, int i, int seg, 
 template <class Factory, bool TSMEM>
 __global__ void __launch_bounds__(128) search_kernel(const DevJob j, const int cpw, const uint64_t t0,
                                                      const int64_t S, const uint32_t r, const int list_mode,
-                                                     const int seg_lo, const int seg_hi_in, const int exact_first) {
-  if (exact_first && rough_last_joint(j.stats[kStatRejected], j.p)) return;   // (the first search only)
+                                                     const int seg_lo, const int seg_hi_in) {
   const int nchains = list_mode == 0 ? j.p : static_cast<int>(j.stats[list_mode == 1 ? kStatPending : kStatNoHit]);
   const int seg_hi = min(seg_hi_in, j.ck_K);
   const long long items = static_cast<long long>(nchains) * max(0, seg_hi - seg_lo);
@@ -486,8 +433,7 @@ __global__ void __launch_bounds__(128) search_kernel(const DevJob j, const int c
           hk.kmin = &j.kmin[i];
           hk.stop = seg_start;
           const int64_t k_begin = hk.k;
-          if constexpr (IsRec<Factory>::value) record_segment(j, i, seg, S, hk);
-          else replay_segment<Factory>(j, b, i, seg, t0, S, hk);
+          replay_segment<Factory>(j, b, i, seg, t0, S, hk);
           found = hk.found;
           searched += hk.k - k_begin;
         }
@@ -552,94 +498,6 @@ __global__ void __launch_bounds__(128) summary_kernel(const DevJob j, const int 
     atomicAdd(reinterpret_cast<unsigned long long*>(&j.stats[kStatSearched]), static_cast<unsigned long long>(searched));
 }
 
-// A lower bound of every chain's second-best v before the pass over its
-// samples, so that the pass's filter is tight from the start (without it each
-// segment's first samples pass: 15 of 2048 a lane, a quarter of the warps'
-// iterations): the second best of up to 1024 samples spread over the chain,
-// one warp a chain.
-__device__ __forceinline__ void height_top2(float v, float& best, float& second) {
-  second = fmaxf(second, fminf(best, v));
-  best = fmaxf(best, v);
-}
-template <class Factory>
-__global__ void __launch_bounds__(128) height_seed_kernel(const DevJob j, const int64_t S, const uint32_t r) {
-  if (j.stats[kStatPending] == 0) return;
-  const int f = static_cast<int>(j.stats[kStatFirstPending]);
-  const float* wl = reinterpret_cast<const float*>(j.lvcnt);
-  const int lane = threadIdx.x & 31;
-  const int64_t M = S * j.N;
-  const int n = static_cast<int>(min(static_cast<int64_t>(1024), max(static_cast<int64_t>(32), M / 32))) & ~31;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (int q = f + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5); q < j.p; q += nwarps) {
-    const int i = j.perm[q];
-    float best = height_none().best, second = best;
-    for (int a = lane; a < n; a += 32) {
-      const int64_t k = M >= n ? static_cast<int64_t>(a) * (M / n) : a;   // distinct samples (0-based)
-      if (k >= M) break;
-      const uint4 v = philox4x32_10(make_uint4(static_cast<uint32_t>(k >> 2), r, static_cast<uint32_t>(i), kTagJoint),
-                                    j.key0, j.key1);
-      const uint32_t u = uint4_word(v, static_cast<uint32_t>(k & 3));
-      height_top2(wl[j.rec[rec_index(i, k, M)]] + height_draw(u), best, second);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const float b2 = __shfl_xor_sync(0xFFFFFFFFu, best, o), s2 = __shfl_xor_sync(0xFFFFFFFFu, second, o);
-      height_top2(b2, best, second);
-      second = fmaxf(second, s2);
-    }
-    if (lane == 0) heights(j)[i].second = second;
-  }
-}
-
-// Heights of the chains from the first pending one on, for a recorded round
-// (mc_height.cuh): items and queue as in summary_kernel, the levels' weights
-// in shared memory.
-template <class Factory>
-__global__ void __launch_bounds__(128) height_kernel(const DevJob j, const int cpw, const uint64_t t0, const int64_t S,
-                                                     const uint32_t r) {
-  if (j.stats[kStatPending] == 0) return;
-  const int f = static_cast<int>(j.stats[kStatFirstPending]);
-  const int nchains = j.p - f;
-  const long long items = static_cast<long long>(nchains) * j.ck_K;
-  const SmemPlan sp = smem_plan(j.L, Factory::kPlacement, cpw, blockDim.x >> 5, false, true);   // "histogram": weights
-  BlockCtx b = block_setup<false>(j, sp, cpw, 0, false);
-  float* wl = reinterpret_cast<float*>(b.hist);
-  const float* g = reinterpret_cast<const float*>(j.lvcnt);
-  for (int m = threadIdx.x; m < j.np1; m += blockDim.x) wl[m] = g[m];
-  __syncthreads();
-  const float slack = height_slack(j);
-  unsigned long long* queue = reinterpret_cast<unsigned long long*>(&j.stats[kStatQueueSearch]);
-  long long searched = 0;
-  for (;;) {
-    long long base = 0;
-    if (b.lane == 0) base = static_cast<long long>(atomicAdd(queue, static_cast<unsigned long long>(cpw)));
-    base = __shfl_sync(0xFFFFFFFFu, base, 0);
-    if (base >= items) break;
-    const long long item = base + b.lane;
-    if (b.lane < cpw && item < items) {
-      const int seg = static_cast<int>(item / nchains);
-      const int i = j.perm[f + static_cast<int>(item % nchains)];
-      HeightHook hk;
-      hk.wl = wl;
-      hk.entry = heights(j) + i;
-      hk.slack = slack;
-      hk.k = static_cast<int64_t>(seg) * j.seg_len;
-      hk.chain = static_cast<uint32_t>(i);
-      hk.r = r;
-      hk.k0 = j.key0;
-      hk.k1 = j.key1;
-      hk.done = false;
-      hk.begin();
-      const int64_t k_begin = hk.k;
-      record_segment(j, i, seg, S, hk);
-      if (hk.h.m != kNoLevel) height_store_max(heights(j) + i, hk.h);
-      searched += hk.k - k_begin;
-    }
-    __syncwarp();
-  }
-  if (searched)
-    atomicAdd(reinterpret_cast<unsigned long long*>(&j.stats[kStatSearched]), static_cast<unsigned long long>(searched));
-}
-
 // (k counts the samples of the words seen so far, as in SearchHook; done
 // once a word reaches the cut)
 struct PrefixHook {
@@ -659,14 +517,11 @@ struct PrefixHook {
 };
 
 // Discarded prefixes (samples before k_i; the whole chain if nothing is
-// kept) counted into dpre.  Replays take the work list plist of (chain,
-// segment) items; a recorded round takes every (segment, chain) pair,
-// segment-major, and skips those that start at or after the chain's cut.
+// kept) counted into dpre, from the work list plist of (chain, segment) items.
 template <class Factory, bool TSMEM>
 __global__ void __launch_bounds__(128) prefix_kernel(const DevJob j, const int cpw, const uint64_t t0,
                                                      const int64_t S) {
-  const long long items =
-      IsRec<Factory>::value ? static_cast<long long>(j.p) * j.ck_K : static_cast<long long>(j.stats[kStatQueuePrefix]);
+  const long long items = static_cast<long long>(j.stats[kStatQueuePrefix]);
   if (items == 0) return;
   const SmemPlan sp = smem_plan(j.L, Factory::kPlacement, cpw, blockDim.x >> 5, TSMEM, true);
   BlockCtx b = block_setup<TSMEM>(j, sp, cpw, 0, true);
@@ -684,16 +539,14 @@ __global__ void __launch_bounds__(128) prefix_kernel(const DevJob j, const int c
     if (base >= items) break;
     const long long item = base + b.slot;
     if (b.lane < cpw && item < items) {
-      const int2 w = IsRec<Factory>::value ? make_int2(static_cast<int>(item % j.p), static_cast<int>(item / j.p))
-                                           : j.plist[item];
+      const int2 w = j.plist[item];
       const int i = w.x, seg = w.y;
       const int64_t k = j.k[i];
       const int64_t cut = (k > 0) ? k : M + 1;
       const int64_t seg_first = static_cast<int64_t>(seg) * j.seg_len + 1;
       if (seg_first < cut) {
         PrefixHook hk{b.hist, seg_first - 1, cut, false};
-        if constexpr (IsRec<Factory>::value) record_segment(j, i, seg, S, hk);
-        else replay_segment<Factory>(j, b, i, seg, t0, S, hk);
+        replay_segment<Factory>(j, b, i, seg, t0, S, hk);
         atomicAdd(&s_samples, static_cast<unsigned long long>(hk.k - (seg_first - 1)));
       }
     }
@@ -817,11 +670,7 @@ __global__ void __launch_bounds__(128) resolve_kernel(const DevJob j, const int 
         hk.k0 = j.key0;
         hk.k1 = j.key1;
         hk.done = false;
-        if constexpr (IsRec<Factory>::value) {
-          for (int sg = 0; sg < j.ck_K && !hk.done; ++sg) record_segment(j, i, sg, S, hk);
-        } else {
-          replay_chain<Factory>(j, b, i, t0, S, hk);
-        }
+        replay_chain<Factory>(j, b, i, t0, S, hk);
         j.k[i] = hk.found;
         searched += hk.k;
       }
@@ -930,29 +779,27 @@ inline cudaError_t launch_join_t(const DevJob& j, const LaunchShape& s, uint64_t
   // a search over the chains of list_mode: their first segments, then the
   // later segments of those without a hit there
   const bool exact_scan = static_cast<long long>(j.p) * S * j.N <= j.scan_max_samples;
-  // a recorded round may skip the speculative first search (rough_last_joint)
-  const int exact_first = (IsRec<F>::value && exact_scan) ? 1 : 0;
-  auto search = [&](int list_mode, int first) -> cudaError_t {
+  auto search = [&](int list_mode) -> cudaError_t {
     cudaError_t e2 = join_reset_queue(j, st);
     if (e2 != cudaSuccess) return e2;
-    kq<<<grid_all, 32 * s.wpb, bytes, st>>>(j, s.cpw, t0, S, r, list_mode, 0, 1, first);
+    kq<<<grid_all, 32 * s.wpb, bytes, st>>>(j, s.cpw, t0, S, r, list_mode, 0, 1);
     launches_add(1);
     if (j.ck_K > 1) {
       if ((e2 = join_nohit(j, list_mode, st)) != cudaSuccess) return e2;
       if ((e2 = join_reset_queue(j, st)) != cudaSuccess) return e2;
-      kq<<<grid_all, 32 * s.wpb, bytes, st>>>(j, s.cpw, t0, S, r, 2, 1, j.ck_K, first);
+      kq<<<grid_all, 32 * s.wpb, bytes, st>>>(j, s.cpw, t0, S, r, 2, 1, j.ck_K);
       launches_add(1);
     }
     return cudaGetLastError();
   };
   // speculated inputs: every chain
-  if ((e = search(0, exact_first)) != cudaSuccess) return e;
-  if ((e = join_select(j, false, st, exact_first != 0)) != cudaSuccess) return e;
+  if ((e = search(0)) != cudaSuccess) return e;
+  if ((e = join_select(j, false, st)) != cudaSuccess) return e;
   // grid-wide speculative resolution passes
   auto pass = [&](int n, bool defer) -> cudaError_t {
     for (int q = 0; q < n; ++q) {
       cudaError_t e2 = join_mark(j, st, true, defer);
-      if (e2 == cudaSuccess) e2 = search(1, 0);
+      if (e2 == cudaSuccess) e2 = search(1);
       if (e2 == cudaSuccess) e2 = join_select(j, true, st);
       if (e2 != cudaSuccess) return e2;
     }
@@ -964,36 +811,19 @@ inline cudaError_t launch_join_t(const DevJob& j, const LaunchShape& s, uint64_t
     // new k's, and the ordinary passes catch what the scan left
     if ((e = pass(j.passes_scan, true)) != cudaSuccess) return e;
     if ((e = join_mark(j, st, false)) != cudaSuccess) return e;
-    if constexpr (IsRec<F>::value) {
-      if ((e = join_height_init(j, st)) != cudaSuccess) return e;
-      height_seed_kernel<F><<<std::min(2432u, blocks_for(j.p, 4)), 128, 0, st>>>(j, S, r);
-      launches_add(1);
-      if ((e = join_reset_queue(j, st)) != cudaSuccess) return e;
-      auto kh = height_kernel<F>;
-      const size_t hbytes = plan_bytes(j.L, s, false, true);
-      if ((e = cudaFuncSetAttribute(kh, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(hbytes))) !=
-          cudaSuccess)
-        return e;
-      const unsigned grid_h = static_cast<unsigned>(
-          std::min<long long>(blocks_for(items, per_block), resident_blocks(kh, 32 * s.wpb, hbytes)));
-      kh<<<grid_h, 32 * s.wpb, hbytes, st>>>(j, s.cpw, t0, S, r);
-      launches_add(1);
-      if ((e = join_height_scan(j, st)) != cudaSuccess) return e;
-    } else {
-      if ((e = join_summary_init(j, st)) != cudaSuccess) return e;
-      if ((e = join_reset_queue(j, st)) != cudaSuccess) return e;
-      auto ks = summary_kernel<F, TS>;
-      if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes))) !=
-          cudaSuccess)
-        return e;
-      const unsigned grid_sum = static_cast<unsigned>(
-          std::min<long long>(blocks_for(items, per_block), resident_blocks(ks, 32 * s.wpb, bytes)));
-      ks<<<grid_sum, 32 * s.wpb, bytes, st>>>(j, s.cpw, t0, S, r);
-      launches_add(1);
-      if ((e = join_scan(j, st)) != cudaSuccess) return e;
-    }
+    if ((e = join_summary_init(j, st)) != cudaSuccess) return e;
+    if ((e = join_reset_queue(j, st)) != cudaSuccess) return e;
+    auto ks = summary_kernel<F, TS>;
+    if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes))) !=
+        cudaSuccess)
+      return e;
+    const unsigned grid_sum = static_cast<unsigned>(
+        std::min<long long>(blocks_for(items, per_block), resident_blocks(ks, 32 * s.wpb, bytes)));
+    ks<<<grid_sum, 32 * s.wpb, bytes, st>>>(j, s.cpw, t0, S, r);
+    launches_add(1);
+    if ((e = join_scan(j, st)) != cudaSuccess) return e;
     if ((e = join_tj_list(j, st)) != cudaSuccess) return e;
-    if ((e = search(1, 0)) != cudaSuccess) return e;
+    if ((e = search(1)) != cudaSuccess) return e;
     if ((e = join_select(j, true, st)) != cudaSuccess) return e;
     if ((e = pass(j.passes_scan, false)) != cudaSuccess) return e;
   } else {
@@ -1008,8 +838,7 @@ inline cudaError_t launch_join_t(const DevJob& j, const LaunchShape& s, uint64_t
   if ((e = cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pbytes))) !=
       cudaSuccess)
     return e;
-  if constexpr (!IsRec<F>::value)
-    if ((e = join_prefix_list(j, st)) != cudaSuccess) return e;
+  if ((e = join_prefix_list(j, st)) != cudaSuccess) return e;
   if ((e = join_reset_queue(j, st)) != cudaSuccess) return e;
   const unsigned grid_pre = static_cast<unsigned>(
       std::min<long long>(blocks_for(items, sp.cpw * sp.wpb), resident_blocks(kp, 32 * sp.wpb, pbytes)));

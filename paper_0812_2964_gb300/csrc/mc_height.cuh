@@ -44,6 +44,12 @@ constexpr double kHeightEps = 1e-4;
 
 __device__ __forceinline__ Height* heights(const DevJob& j) { return reinterpret_cast<Height*>(j.summ); }
 
+// The levels' weights (W[m] - Wref) / ln 2, built at the start of the joint
+// in the scratch of the energy ordering; Wref is the weight of a level that
+// the round met.
+__device__ __forceinline__ float* level_weights(const DevJob& j) { return reinterpret_cast<float*>(j.lvcnt); }
+__device__ __forceinline__ double reference_weight(const DevJob& j) { return j.W[j.m[0]]; }
+
 __device__ __forceinline__ Height height_none() {
   Height h;
   h.m = kNoLevel;

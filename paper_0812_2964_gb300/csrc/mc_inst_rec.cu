@@ -1,24 +1,21 @@
-// The joint's kernels for a recorded round (search, summary, resolution,
-// prefix correction reading the round record instead of replaying
-// lattices): one instantiation serves every L, since nothing in them
-// depends on the lattice size at compile time.
-#include "mc_chain_kernels.cuh"
+// The joint of a recorded round: one instantiation serves every L, since
+// nothing in it depends on the lattice size at compile time.
+#include "mc_joint_kept.cuh"
 
 namespace mcgpu {
 
-// Samples per segment of a recorded round's joint.  A segment is one lane's
-// work item; with nothing to restore at its start it can be much shorter
-// than a replay segment, so that even the first pass (segment 0 of every
-// chain) and a few thousand chains keep the whole GPU busy.
-constexpr int64_t kRecordSegment = 2048;
-
-cudaError_t chain_kernels_record(const DevJob& j, uint64_t t0, int64_t S, uint32_t r, cudaStream_t st) {
+// Samples per segment: a lane's work item.  With nothing to restore at its
+// start it is as short as spreads the round over the GPU's lanes, down to 256
+// samples (a search's first pass reads one segment a chain), up to 2048 (an
+// item's set-up then costs a few percent).
+cudaError_t chain_kernels_record(const DevJob& j, int64_t S, uint32_t r, cudaStream_t st) {
   DevJob jr = j;
-  jr.seg_len = std::min<int64_t>(j.seg_len, kRecordSegment);
-  jr.ck_K = static_cast<int>((S * j.N + jr.seg_len - 1) / jr.seg_len);
-  // full warps, four a block; shared memory holds only the prefix pass's histogram
-  const LaunchShape s{kPlaceReg, 32, 4};
-  return launch_join_t<RecF, false>(jr, s, t0, S, r, st);
+  const int64_t M = S * j.N;
+  const int64_t spread = static_cast<int64_t>(j.p) * M / (152 * 512);
+  jr.seg_len = std::min<int64_t>(2048, std::max<int64_t>(256, spread & ~31ll));
+  jr.ck_K = static_cast<int>((M + jr.seg_len - 1) / jr.seg_len);
+  // full warps, four a block; shared memory holds only the level weights (or counts)
+  return launch_join_kept<SourceRec>(jr, LaunchShape{kPlaceReg, 32, 4}, S, r, st);
 }
 
 }  // namespace mcgpu

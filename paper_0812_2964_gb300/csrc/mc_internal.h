@@ -129,8 +129,11 @@ enum StatIndex : int {
   kStatFirstPending = 13,// lowest chain queued by the last mark pass (p if none)
   kStatScanned = 14,     // chains whose input the exact scan settled (last joint)
   kStatNoHit = 15,       // chains listed in work2
-  kStatWeightMax = 16,   // largest |W - Wref| / ln 2 of the level weights, as float bits (recorded rounds' exact path)
-  kStatCount = 17
+  kStatWeightMax = 16,   // largest |W - Wref| / ln 2 of the level weights, as float bits (0 between joints)
+  kStatQueueA = 17,      // next items of a kept round's searches: first segments,
+  kStatQueueB = 18,      // later segments
+  kStatCountKept = 19,   // 1: dpre counts the kept samples, 0: the discarded ones
+  kStatCount = 20
 };
 
 // ---- kernels (mc_kernels.cu) ----
@@ -167,19 +170,23 @@ cudaError_t join_mark(const DevJob& j, cudaStream_t st, bool thresholds = true, 
 cudaError_t join_tj_list(const DevJob& j, cudaStream_t st);
 // list (in work2) the chains of list_mode (0 all, 1 work) with no hit in segment 0
 cudaError_t join_nohit(const DevJob& j, int list_mode, cudaStream_t st);
-// exact_first: a recorded round whose exact path is enabled -- when the job's
-// previous joint rejected more than p/16 chains, the speculative first
-// search is skipped (select marks every chain unsearched) and the joint goes
-// straight to the summary and the exact scan
-cudaError_t join_select(const DevJob& j, bool listed, cudaStream_t st, bool exact_first = false);
+cudaError_t join_select(const DevJob& j, bool listed, cudaStream_t st);
 cudaError_t join_prefix_list(const DevJob& j, cudaStream_t st);
 cudaError_t join_reset_queue(const DevJob& j, cudaStream_t st);
 cudaError_t join_finalize(const DevJob& j, int64_t S, cudaStream_t st);
 cudaError_t join_summary_init(const DevJob& j, cudaStream_t st);
 cudaError_t join_scan(const DevJob& j, cudaStream_t st);
-// the same for recorded rounds, by acceptance heights (mc_height.cuh)
-cudaError_t join_height_init(const DevJob& j, cudaStream_t st);
-cudaError_t join_height_scan(const DevJob& j, cudaStream_t st);
+
+// pieces of the joint of a round whose samples were kept (mc_joint_kept.cuh)
+enum MarkFlags : int {
+  kMarkListed = 1,      // take the last search's results for work[] only (else for every chain)
+  kMarkDefer = 2,       // a speculative pass ahead of the exact path: leave many pending chains to it
+  kMarkExactFirst = 4,  // the first search was skipped if the previous joint was rough
+  kMarkFinal = 8,       // nothing follows but the fallback: fix the carry and what to count
+};
+cudaError_t kept_prelude(const DevJob& j, cudaStream_t st);
+cudaError_t kept_mark(const DevJob& j, int64_t S, int flags, cudaStream_t st);
+cudaError_t kept_scan(const DevJob& j, cudaStream_t st);
 
 // per-unit launchers of the templated chain kernels (mc_inst_*.cu)
 #define MC_CHAIN_UNIT(name)                                                                              \
@@ -203,7 +210,7 @@ MC_CHAIN_UNIT(chain_kernels_smem_L128);
 // generation with one chain per warp (any L; shape kPlaceSmem with one chain a warp)
 cudaError_t chain_kernels_warp(const DevJob& j, uint64_t t0, int64_t S, bool trace, cudaStream_t st);
 // the joint of a recorded round (any L): kernels without lattices or table
-cudaError_t chain_kernels_record(const DevJob& j, uint64_t t0, int64_t S, uint32_t r, cudaStream_t st);
+cudaError_t chain_kernels_record(const DevJob& j, int64_t S, uint32_t r, cudaStream_t st);
 
 // launch shape chosen by default for (L, p)
 LaunchShape default_shape(int L, int p, int num_sms);

@@ -7,6 +7,7 @@
 #include <math_constants.h>
 
 #include "mc_chain_kernels.cuh"
+#include "mc_height.cuh"
 #include "mc_scan_fsm.cuh"
 #include "mc_warp_chain.cuh"
 
@@ -257,51 +258,67 @@ __global__ void __launch_bounds__(1024) order_kernel(const DevJob j) {
   }
 }
 
+// Inclusive sum over the block (1024 threads); *total = the whole block's.
+__device__ __forceinline__ long long block_sum_scan(long long v, long long* s_warp, long long* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long u = __shfl_up_sync(0xFFFFFFFFu, v, o);
+    if (lane >= o) v += u;
+  }
+  if (lane == 31) s_warp[warp] = v;
+  __syncthreads();
+  long long w = s_warp[lane];
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long u = __shfl_up_sync(0xFFFFFFFFu, w, o);
+    if (lane >= o) w += u;
+  }
+  *total = __shfl_sync(0xFFFFFFFFu, w, 31);
+  if (warp > 0) v += __shfl_sync(0xFFFFFFFFu, w, warp - 1);
+  __syncthreads();
+  return v;
+}
+
 // Segmented scan and histogram: kept length of chain i is M - k_i + 1 (0 if
-// nothing is kept); offsets are the exclusive scan; h += hgen - dpre.
-__global__ void __launch_bounds__(1024) finalize_kernel(const DevJob j, const int64_t M) {
-  __shared__ long long s_tmp[1024];
-  const int t = threadIdx.x, nt = blockDim.x;
-  for (int m = t; m < j.np1; m += nt) {
-    j.h[m] += static_cast<long long>(j.hgen[m] - j.dpre[m]);
-    j.hgen[m] = 0ull;
-    j.dpre[m] = 0ull;
+// nothing is kept); offsets are the exclusive scan (block 0, 1024 positions
+// at a time); h += hgen - dpre, or += dpre where that holds the kept samples
+// (the other blocks).
+__global__ void __launch_bounds__(1024) finalize_kernel(const DevJob j, const int64_t M, const int may_count_kept) {
+  const int t = threadIdx.x;
+  if (blockIdx.x > 0) {
+    const bool kept = may_count_kept && j.stats[kStatCountKept];
+    for (int m = (blockIdx.x - 1) * 1024 + t; m < j.np1; m += (gridDim.x - 1) * 1024) {
+      const unsigned long long d = j.dpre[m];
+      j.h[m] += static_cast<long long>(kept ? d : j.hgen[m] - d);
+      j.hgen[m] = 0ull;
+      j.dpre[m] = 0ull;
+    }
+    return;
   }
-  const int per = (j.p + nt - 1) / nt;
-  const int lo = min(j.p, t * per), hi = min(j.p, lo + per);  // positions in the joint
-  long long sum = 0, rej = 0;
-  for (int q = lo; q < hi; ++q) {
-    const int64_t k = j.k[j.perm[q]];
-    sum += k > 0 ? (M - k + 1) : 0;
-    rej += k > 0 ? 0 : 1;
+  __shared__ long long s_warp[32];
+  long long run = 0, rej = 0;
+  for (int base = 0; base < j.p; base += 1024) {
+    const int q = base + t;
+    const int i = q < j.p ? j.perm[q] : 0;
+    const int64_t k = q < j.p ? j.k[i] : 0;
+    const long long len = k > 0 ? M - k + 1 : 0;
+    rej += q < j.p && k <= 0 ? 1 : 0;
+    long long total;
+    const long long incl = block_sum_scan(len, s_warp, &total);
+    if (q < j.p) j.offsets[i] = run + incl - len;
+    run += total;
   }
-  s_tmp[t] = sum;
-  __syncthreads();
-  for (int off = 1; off < nt; off <<= 1) {
-    const long long v = (t >= off) ? s_tmp[t - off] : 0;
-    __syncthreads();
-    s_tmp[t] += v;
-    __syncthreads();
-  }
-  long long run = s_tmp[t] - sum;
-  for (int q = lo; q < hi; ++q) {
-    const int i = j.perm[q];
-    j.offsets[i] = run;
-    const int64_t k = j.k[i];
-    run += k > 0 ? (M - k + 1) : 0;
-  }
-  if (t == nt - 1) {
-    j.stats[kStatJoined] = s_tmp[t];
-    j.stats[kStatJoinedTotal] += s_tmp[t];
-  }
-  __syncthreads();
-  s_tmp[t] = rej;
-  __syncthreads();
+  long long rejected;
+  block_sum_scan(rej, s_warp, &rejected);
   if (t == 0) {
-    long long r = 0;
-    for (int q = 0; q < nt; ++q) r += s_tmp[q];
-    j.stats[kStatRejected] = r;
+    j.stats[kStatJoined] = run;
+    j.stats[kStatJoinedTotal] += run;
+    j.stats[kStatRejected] = rejected;
+    j.stats[kStatWeightMax] = 0;
   }
+}
+
+static void launch_finalize(const DevJob& j, int64_t M, bool may_count_kept, cudaStream_t st) {
+  finalize_kernel<<<1 + blocks_for(j.np1, 1024), 1024, 0, st>>>(j, M, may_count_kept ? 1 : 0);
 }
 
 // Control experiment (no detailed balance at the joints): keep everything.
@@ -330,7 +347,6 @@ __global__ void clear_stats_kernel(const DevJob j) {
     j.stats[kStatWholeFill] = 0;
     j.stats[kStatScanned] = 0;
     j.stats[kStatFirstPending] = j.p;
-    j.stats[kStatWeightMax] = 0;
   }
   // earliest accepted sample of each chain: none found yet
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < j.p; i += gridDim.x * blockDim.x) j.kmin[i] = kNoHit;
@@ -630,23 +646,157 @@ __global__ void __launch_bounds__(1024) scan_kernel(const DevJob j) {
   }
 }
 
-// ------------------------------------------------------------------ heights (mc_height.cuh)
-// Set-up: empty entries for the chains from the first pending one on, and
-// the levels' weights as floats relative to the weight of a level met there.
-__global__ void height_init_kernel(const DevJob j) {
-  if (j.stats[kStatPending] == 0) return;
-  const int f = static_cast<int>(j.stats[kStatFirstPending]);
+// ------------------------------------------------------------------ kept rounds (mc_joint_kept.cuh)
+// For every position of the joint, the last position before it whose chain
+// `keeps` (-1: none): each(q, last) for all q in [f, p); returns the last
+// one of all to every thread.  One block of 1024 threads; positions are read
+// 1024 at a time, coalesced, as bits of 32 positions a word.
+template <class Keeps, class Each>
+__device__ __forceinline__ int block_last_kept(const int f, const int p, const Keeps& keeps, const Each& each) {
+  __shared__ uint32_t s_bits[1024];
+  __shared__ int s_before[1024], s_warp[32];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  int carry = -1;
+  for (int base = f; base < p; base += 32768) {
+    const int its = min(32, (p - base + 1023) / 1024);
+    for (int it = 0; it < its; ++it) {
+      const int q = base + it * 1024 + t;
+      const uint32_t b = __ballot_sync(0xFFFFFFFFu, q < p && keeps(q));
+      if (lane == 0) s_bits[it * 32 + warp] = b;
+    }
+    __syncthreads();
+    const uint32_t w = t < 32 * its ? s_bits[t] : 0u;
+    int v = w ? base + 32 * t + 31 - __clz(w) : -1;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xFFFFFFFFu, v, o);
+      if (lane >= o) v = max(v, u);
+    }
+    if (lane == 31) s_warp[warp] = v;
+    __syncthreads();
+    int x = s_warp[lane];
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xFFFFFFFFu, x, o);
+      if (lane >= o) x = max(x, u);
+    }
+    const int all = __shfl_sync(0xFFFFFFFFu, x, 31);
+    int before = __shfl_up_sync(0xFFFFFFFFu, v, 1);
+    if (lane == 0) before = -1;
+    const int warps_before = warp > 0 ? __shfl_sync(0xFFFFFFFFu, x, warp - 1) : -1;
+    s_before[t] = max(carry, max(before, warps_before));
+    __syncthreads();
+    for (int it = 0; it < its; ++it) {
+      const int q = base + it * 1024 + t;
+      if (q < p) {
+        const uint32_t m = s_bits[it * 32 + warp] & ((1u << lane) - 1u);
+        each(q, m ? q - lane + 31 - __clz(m) : s_before[it * 32 + warp]);
+      }
+    }
+    carry = max(carry, all);
+    __syncthreads();
+  }
+  return carry;
+}
+
+// Start of a kept round's joint: the joint order where it is the chains' own,
+// the speculated inputs (spec_inputs_kernel), nothing found yet, the level
+// weights and the cleared counters.
+__global__ void kept_prelude_kernel(const DevJob j) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-  const double wref = j.W[j.m[j.perm[f]]];
-  float* wl = reinterpret_cast<float*>(j.lvcnt);
+  if (t == 0) {
+    for (const int s : {kStatSearched, kStatMismatch, kStatPasses, kStatPending, kStatScanned, kStatNoHit,
+                        kStatQueueSearch, kStatQueueA, kStatQueueB})
+      j.stats[s] = 0;
+    j.stats[kStatFirstPending] = j.p;
+  }
+  const int carry_in = j.stats[kStatCarryValid] ? static_cast<int>(j.stats[kStatCarry]) : -1;
+  for (int q = t; q < j.p; q += nt) {
+    const int i = j.ordered ? j.perm[q] : q;
+    const int prev = q > 0 ? (j.ordered ? j.perm[q - 1] : q - 1) : -1;
+    if (!j.ordered) j.perm[q] = q;
+    j.xused[i] = prev >= 0 ? j.m[prev] : carry_in;
+    j.kmin[i] = kNoHit;
+  }
+  const double wref = reference_weight(j);
+  float* wl = level_weights(j);
   float big = 0.0f;
   for (int m = t; m < j.np1; m += nt) {
     const float v = static_cast<float>((j.W[m] - wref) * 1.4426950408889634);
     wl[m] = v;
     if (fabsf(v) < CUDART_INF_F) big = fmaxf(big, fabsf(v));
   }
+  // (0 before: finalize_kernel clears it)
   if (big > 0.0f) atomicMax(&j.stats[kStatWeightMax], static_cast<long long>(__float_as_int(big)));
-  for (int q = f + t; q < j.p; q += nt) heights(j)[j.perm[q]] = height_none();
+}
+
+// Results of the last search, then one resolution pass, part 1 (as
+// mark_kernel, which see for `defer`): the chains whose actual input is not
+// the one their k was found for go to work[], with the new input in xused.
+// With kMarkFinal and nothing pending: the carry, and whether fewer samples
+// are kept than discarded.
+__global__ void __launch_bounds__(1024) kept_mark_kernel(const DevJob j, const int64_t M, const int flags) {
+  __shared__ int s_count, s_first, s_new;
+  __shared__ unsigned long long s_kept;
+  const int t = threadIdx.x, nt = blockDim.x;
+  if (t == 0) {
+    s_count = 0;
+    s_first = j.p;
+    s_new = 0;
+    s_kept = 0ull;
+  }
+  const bool unsearched = (flags & kMarkExactFirst) && rough_last_joint(j.stats[kStatRejected], j.p);
+  const int n = (flags & kMarkListed) ? static_cast<int>(j.stats[kStatPending]) : j.p;
+  for (int q = t; q < n; q += nt) {
+    const int i = (flags & kMarkListed) ? j.work[q] : q;
+    const unsigned long long k = j.kmin[i];
+    j.k[i] = unsearched ? -1 : (k == kNoHit ? 0 : static_cast<int64_t>(k));
+  }
+  const int carry_in = j.stats[kStatCarryValid] ? static_cast<int>(j.stats[kStatCarry]) : -1;
+  __syncthreads();
+  unsigned long long kept = 0;
+  const int last_all = block_last_kept(
+      0, j.p, [&](int q) { return j.k[j.perm[q]] > 0; },
+      [&](int q, int last) {
+        const int x = last >= 0 ? j.m[j.perm[last]] : carry_in;
+        const int i = j.perm[q];
+        const int64_t k = j.k[i];
+        j.lastacc[q] = last;
+        if (k > 0) kept += static_cast<unsigned long long>(M - k + 1);
+        const bool moved = x != j.xused[i];
+        if (moved || k < 0) {
+          j.work[atomicAdd(&s_count, 1)] = i;
+          atomicMin(&s_first, q);
+        }
+        if (moved) {
+          j.xused[i] = x;
+          j.k[i] = -1;
+          j.kmin[i] = kNoHit;
+          atomicAdd(&s_new, 1);
+        }
+      });
+  // (a warp's sum first: 64-bit shared atomics are compare-and-swap loops, 30 us when 1024 threads meet in one)
+  for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(0xFFFFFFFFu, kept, o);
+  if (kept && (t & 31) == 0) atomicAdd(&s_kept, kept);
+  __syncthreads();
+  if (t == 0) {
+    const bool deferred = (flags & kMarkDefer) && s_count > j.p / 16;
+    j.stats[kStatPending] = deferred ? 0 : s_count;
+    j.stats[kStatFirstPending] = s_first;
+    if (s_new) {
+      j.stats[kStatPasses] += 1;
+      j.stats[kStatMismatch] += s_new;
+    }
+    j.stats[kStatNoHit] = 0;
+    j.stats[kStatQueueSearch] = 0;
+    j.stats[kStatQueueA] = 0;
+    j.stats[kStatQueueB] = 0;
+    if ((flags & kMarkFinal) && s_count == 0) {
+      if (last_all >= 0) {
+        j.stats[kStatCarry] = j.m[j.perm[last_all]];
+        j.stats[kStatCarryValid] = 1;
+      }
+      j.stats[kStatCountKept] = 2ull * s_kept < static_cast<unsigned long long>(j.p) * static_cast<unsigned long long>(M);
+    }
+  }
 }
 
 // Scratch of the scan in tj (its rows are rebuilt for the chains searched
@@ -670,15 +820,15 @@ __device__ __forceinline__ HeightScratch height_scratch(const DevJob& j) {
   return s;
 }
 
-__global__ void __launch_bounds__(1024) height_value_kernel(const DevJob j) {
-  if (j.stats[kStatPending] == 0) return;
+// Values and maxima of the positions [1024 block, 1024 block + 1024), in steps of `blocks` blocks.
+__device__ __forceinline__ void height_values(const DevJob& j, int block, int blocks) {
   __shared__ double s_max[32];
   const HeightScratch hs = height_scratch(j);
   const int f = static_cast<int>(j.stats[kStatFirstPending]);
   const int t = threadIdx.x;
-  const double wref = j.W[j.m[j.perm[f]]];
+  const double wref = reference_weight(j);
   const float slack = height_slack(j);
-  for (int base = blockIdx.x * 1024; base < j.p; base += gridDim.x * 1024) {
+  for (int base = block * 1024; base < j.p; base += blocks * 1024) {
     const int q = base + t;
     double v = -CUDART_INF;
     if (q >= f && q < j.p) {
@@ -724,20 +874,25 @@ __device__ __forceinline__ int height_next(const DevJob& j, const HeightScratch&
   return j.p;
 }
 
-__global__ void height_next_kernel(const DevJob j) {
-  if (j.stats[kStatPending] == 0) return;
+// The input at position f: the last level passed on (-1: none yet).
+__device__ __forceinline__ int height_input(const DevJob& j, int f) {
+  const int last = j.lastacc[f];
+  return last >= 0 ? j.m[j.perm[last]] : (j.stats[kStatCarryValid] ? static_cast<int>(j.stats[kStatCarry]) : -1);
+}
+
+// Successors: next[q] = the next chain that keeps samples if the chain at q
+// does; next[p] = the first one for the input at f (none yet: f, kept whole).
+__device__ __forceinline__ void height_successors(const DevJob& j, int t, int nt) {
   const HeightScratch hs = height_scratch(j);
   const int f = static_cast<int>(j.stats[kStatFirstPending]);
-  const double wref = j.W[j.m[j.perm[f]]];
+  const double wref = reference_weight(j);
   const float slack = height_slack(j);
-  for (int q = f + blockIdx.x * blockDim.x + threadIdx.x; q <= j.p; q += gridDim.x * blockDim.x) {
+  for (int q = f + t; q <= j.p; q += nt) {
     int nx;
     if (q < j.p) {
       nx = height_next(j, hs, q + 1, j.W[j.m[j.perm[q]]], wref, slack);
-    } else {   // the round's input at position f: the last level passed on, or nothing yet (kept whole)
-      const int last = j.lastacc[f];
-      const int x = last >= 0 ? j.m[j.perm[last]]
-                              : (j.stats[kStatCarryValid] ? static_cast<int>(j.stats[kStatCarry]) : -1);
+    } else {
+      const int x = height_input(j, f);
       nx = x < 0 ? f : height_next(j, hs, f, j.W[x], wref, slack);
     }
     hs.next[q] = nx;
@@ -747,16 +902,12 @@ __global__ void height_next_kernel(const DevJob j) {
 // One block: mark the positions reached from the round's input (after k
 // doublings the marks hold the first 2^k of them), then give every position
 // its input and outcome, as scan_kernel does.
-__global__ void __launch_bounds__(1024) height_path_kernel(const DevJob j) {
-  if (j.stats[kStatPending] == 0) return;
-  __shared__ int s_tmp[1024];
+__device__ __forceinline__ void height_path(const DevJob& j) {
   __shared__ int s_end, s_count, s_scanned;
   const HeightScratch hs = height_scratch(j);
   const int t = threadIdx.x, nt = blockDim.x, p = j.p;
   const int f = static_cast<int>(j.stats[kStatFirstPending]);
-  const int last0 = j.lastacc[f];
-  const int x0 = last0 >= 0 ? j.m[j.perm[last0]]
-                            : (j.stats[kStatCarryValid] ? static_cast<int>(j.stats[kStatCarry]) : -1);
+  const int x0 = height_input(j, f);
   if (t == 0) {
     s_end = p;
     s_count = 0;
@@ -788,52 +939,59 @@ __global__ void __launch_bounds__(1024) height_path_kernel(const DevJob j) {
   }
   __syncthreads();
   const int stop_at = s_end;
-  // inputs: the last marked position before each, each thread a range of positions
-  const int per = (p - f + nt - 1) / nt;
-  const int lo = min(p, f + t * per), hi = min(p, lo + per);
-  int last = -1;
-  for (int q = lo; q < hi; ++q)
-    if (hs.mark[q]) last = q;
-  s_tmp[t] = last;
-  __syncthreads();
-  for (int off = 1; off < nt; off <<= 1) {
-    const int v = (t >= off) ? s_tmp[t - off] : -1;
-    __syncthreads();
-    s_tmp[t] = max(s_tmp[t], v);
-    __syncthreads();
-  }
-  int run = t > 0 ? s_tmp[t - 1] : -1;
   int scanned = 0;
-  for (int q = lo; q < hi; ++q) {
-    const int ch = j.perm[q];
-    const int64_t kc = j.k[ch];
-    const bool keeps = hs.mark[q] != 0;
-    if (q < stop_at) {
-      const int x = run >= 0 ? j.m[j.perm[run]] : x0;
-      if (kc < 0 || j.xused[ch] != x) {   // not known for this input
-        j.xused[ch] = x;
-        if (!keeps) {
-          j.k[ch] = 0;
-        } else if (x < 0) {               // no input yet: the chain is kept whole
-          j.k[ch] = 1;
-        } else {
-          j.k[ch] = -1;                   // to be searched under the exact input
-          j.kmin[ch] = kNoHit;
-          j.work[atomicAdd(&s_count, 1)] = ch;
+  block_last_kept(
+      f, p, [&](int q) { return hs.mark[q] != 0; },
+      [&](int q, int last) {
+        const int ch = j.perm[q];
+        const int64_t kc = j.k[ch];
+        if (q < stop_at) {
+          const int x = last >= 0 ? j.m[j.perm[last]] : x0;
+          if (kc < 0 || j.xused[ch] != x) {   // not known for this input
+            j.xused[ch] = x;
+            if (!hs.mark[q]) {
+              j.k[ch] = 0;
+            } else if (x < 0) {               // no input yet: the chain is kept whole
+              j.k[ch] = 1;
+            } else {
+              j.k[ch] = -1;                   // to be searched under the exact input
+              j.kmin[ch] = kNoHit;
+              j.work[atomicAdd(&s_count, 1)] = ch;
+            }
+            ++scanned;
+          }
+        } else if (kc < 0) {
+          j.work[atomicAdd(&s_count, 1)] = ch;   // stopped early: chains still waiting for a search keep their inputs
         }
-        ++scanned;
-      }
-    } else if (kc < 0) {
-      j.work[atomicAdd(&s_count, 1)] = ch;   // stopped early: chains still waiting for a search keep their inputs
-    }
-    if (keeps) run = q;
-  }
+      });
   if (scanned) atomicAdd(&s_scanned, scanned);
   __syncthreads();
   if (t == 0) {
     j.stats[kStatPending] = s_count;
     j.stats[kStatScanned] = s_scanned;
+    j.stats[kStatNoHit] = 0;
+    j.stats[kStatQueueA] = 0;
+    j.stats[kStatQueueB] = 0;
   }
+}
+
+__global__ void __launch_bounds__(1024) height_value_kernel(const DevJob j) {
+  if (j.stats[kStatPending]) height_values(j, blockIdx.x, gridDim.x);
+}
+__global__ void height_next_kernel(const DevJob j) {
+  if (j.stats[kStatPending]) height_successors(j, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+__global__ void __launch_bounds__(1024) height_path_kernel(const DevJob j) {
+  if (j.stats[kStatPending]) height_path(j);
+}
+// the three in one launch
+__global__ void __launch_bounds__(1024) height_scan_kernel(const DevJob j) {
+  if (j.stats[kStatPending] == 0) return;
+  height_values(j, 0, 1);
+  __syncthreads();
+  height_successors(j, threadIdx.x, blockDim.x);
+  __syncthreads();
+  height_path(j);
 }
 
 __global__ void tj_list_kernel(const DevJob j) {
@@ -1053,7 +1211,7 @@ cudaError_t k_join_attempts(const DevJob& j, uint64_t t0, int64_t M, uint32_t r,
   } else {
     serial_joint_kernel<<<1, 32, 0, st>>>(j, t0, M, r);
   }
-  finalize_kernel<<<1, 1024, 0, st>>>(j, M);
+  launch_finalize(j, M, false, st);
   launches_add(3);
   return cudaGetLastError();
 }
@@ -1169,15 +1327,11 @@ cudaError_t join_prelude(const DevJob& j, cudaStream_t st) {
 }
 
 // k_i = the earliest accepted sample the search found (0: none).
-__global__ void select_kernel(const DevJob j, const int listed, const int exact_first) {
+__global__ void select_kernel(const DevJob j, const int listed) {
   const int n = listed ? static_cast<int>(j.stats[kStatPending]) : j.p;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= n) return;
   const int i = listed ? j.work[q] : q;
-  if (exact_first && rough_last_joint(j.stats[kStatRejected], j.p)) {
-    j.k[i] = -1;   // not searched: every chain waits for the exact path
-    return;
-  }
   const unsigned long long k = j.kmin[i];
   j.k[i] = k == kNoHit ? 0 : static_cast<int64_t>(k);
 }
@@ -1238,13 +1392,26 @@ cudaError_t join_scan(const DevJob& j, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t join_height_init(const DevJob& j, cudaStream_t st) {
-  height_init_kernel<<<std::min(256u, blocks_for(std::max(j.p, j.np1), 256)), 256, 0, st>>>(j);
+cudaError_t kept_prelude(const DevJob& j, cudaStream_t st) {
+  if (j.ordered) order_kernel<<<1, 1024, 0, st>>>(j);
+  kept_prelude_kernel<<<std::min(304u, blocks_for(std::max(j.p, j.np1), 256)), 256, 0, st>>>(j);
+  launches_add(j.ordered ? 2 : 1);
+  return cudaGetLastError();
+}
+
+cudaError_t kept_mark(const DevJob& j, int64_t S, int flags, cudaStream_t st) {
+  kept_mark_kernel<<<1, 1024, 0, st>>>(j, S * j.N, flags);
   launches_add(1);
   return cudaGetLastError();
 }
 
-cudaError_t join_height_scan(const DevJob& j, cudaStream_t st) {
+// (one block does the whole scan where its three parts are short: two launches saved)
+cudaError_t kept_scan(const DevJob& j, cudaStream_t st) {
+  if (j.p <= 4096) {
+    height_scan_kernel<<<1, 1024, 0, st>>>(j);
+    launches_add(1);
+    return cudaGetLastError();
+  }
   height_value_kernel<<<std::min(152u, blocks_for(j.p, 1024)), 1024, 0, st>>>(j);
   height_next_kernel<<<std::min(1024u, blocks_for(j.p + 1, 128)), 128, 0, st>>>(j);
   height_path_kernel<<<1, 1024, 0, st>>>(j);
@@ -1266,8 +1433,8 @@ cudaError_t join_prefix_list(const DevJob& j, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t join_select(const DevJob& j, bool listed, cudaStream_t st, bool exact_first) {
-  select_kernel<<<blocks_for(j.p, 256), 256, 0, st>>>(j, listed ? 1 : 0, !listed && exact_first ? 1 : 0);
+cudaError_t join_select(const DevJob& j, bool listed, cudaStream_t st) {
+  select_kernel<<<blocks_for(j.p, 256), 256, 0, st>>>(j, listed ? 1 : 0);
   launches_add(1);
   return cudaGetLastError();
 }
@@ -1291,7 +1458,7 @@ cudaError_t join_tj_list(const DevJob& j, cudaStream_t st) {
 }
 
 cudaError_t join_finalize(const DevJob& j, int64_t S, cudaStream_t st) {
-  finalize_kernel<<<1, 1024, 0, st>>>(j, S * j.N);
+  launch_finalize(j, S * j.N, j.rec != nullptr, st);
   launches_add(1);
   return cudaGetLastError();
 }
@@ -1338,11 +1505,11 @@ cudaError_t k_join(const DevJob& j, const LaunchShape& s, uint64_t t0, int64_t S
   if (naive) {
     order_kernel<<<1, 1024, 0, st>>>(j);
     naive_kernel<<<blocks_for(j.p, 256), 256, 0, st>>>(j);
-    finalize_kernel<<<1, 1024, 0, st>>>(j, S * j.N);
+    launch_finalize(j, S * j.N, false, st);
     launches_add(3);
     return cudaGetLastError();
   }
-  if (j.rec) return chain_kernels_record(j, t0, S, r, st);   // levels recorded: no replays
+  if (j.rec) return chain_kernels_record(j, S, r, st);   // levels recorded: no replays
   return dispatch(j, join_shape(j.L, s), false, t0, S, false, r, st);
 }
 
