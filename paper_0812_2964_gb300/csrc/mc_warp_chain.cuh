@@ -1,5 +1,6 @@
-// Generation with one chain per warp (Sec. 2 step 2): the 32 sites of a
-// lattice word are resolved together, one site a lane.
+// Generation with one chain per warp (Sec. 2 step 2): the sites of a window
+// of the row are resolved together: a lattice word, one site a lane (Words),
+// or 64 sites, two neighbouring ones a lane (TwoWords; warp_pairs).
 //
 // A chain's attempts are serial -- the level after each decides the next
 // one's threshold, and its flip the right neighbour's aligned count -- but
@@ -25,9 +26,11 @@
 // visited range ends in a cliff).
 //
 // What bounds it: few chains (fewer than about four warps a scheduler) --
-// the latency of the solve and of each evaluation (two dependent population
-// counts, a table load, a compare, a vote); more chains -- instruction
-// issue, about 100 instructions a word.  One chain per lane (mc_chain.cuh)
+// the latency of the solve and of each evaluation (population counts, a table
+// load, a compare, a vote), 600 cycles a word, 900 a window of 64; more
+// chains -- instruction issue and the integer pipe, 135 instructions a word,
+// 270 a window of 64 (at L = 64 and 4096 chains 77 % of the issue slots, the
+// integer pipe 77 % busy).  One chain per lane (mc_chain.cuh)
 // issues about 35 a site for 32 chains and takes 59 (table in shared memory)
 // to 108 (table through L1) cycles a site however few chains there are, so
 // this form is the better one up to the chain counts of warp_chain_better().
@@ -40,8 +43,13 @@
 namespace mcgpu {
 
 constexpr int kRingWords = 256;      // uniforms in flight a warp (two batches of 128 attempts)
-constexpr int kTablePad = 64;        // a mask on the way to the fixed point may put a site up to
-                                     // 62 levels outside [0, N]: words a table read may stray
+constexpr int kTablePad = 160;       // a mask on the way to the fixed point may put a site up to
+                                     // 126 levels outside [0, N]: words a table read may stray
+static_assert(kRingWords > 128, "the ring before the table takes the strays below it");
+
+// Words a row of the block's own lattice copy (two sites a lane: an even and
+// an odd word per window of 64 sites -- as many for the sizes that use it).
+__host__ __device__ inline int warp_row_words(int L) { return (L + 31) / 32; }
 
 // Shared memory of a block: [rings][table (opt.)][pad][histogram][lattices], in words.
 struct WarpPlan {
@@ -49,13 +57,13 @@ struct WarpPlan {
 };
 
 __host__ __device__ inline WarpPlan warp_plan(int L, int warps, bool tsmem) {
-  const int np1 = L * L + 1, wd = (L + 31) / 32;
+  const int np1 = L * L + 1;
   WarpPlan w;
   w.ring = 0;
   w.table = kRingWords * warps;
   w.hist = w.table + (tsmem ? ((5 * np1 + 3) & ~3) + kTablePad : 0);
   w.lat = w.hist + ((np1 + 3) & ~3);
-  w.total = w.lat + warps * L * wd;
+  w.total = w.lat + warps * L * warp_row_words(L);
   return w;
 }
 
@@ -65,6 +73,19 @@ constexpr int kWarpChainBlock = 32;   // most warps (chains) a block: 64 registe
 inline int64_t warp_flush_sweeps(int warps, int N, int64_t S) {
   const int64_t f = 0xFFFFFFFFll / (static_cast<int64_t>(warps) * N);
   return S > f ? f : 0;
+}
+
+// Two sites a lane (windows of 64) or one (a window a word).  A window of 64
+// takes 1.5 times a word's latency, so it wins where it halves the windows of
+// a row and latency is the bound: rows of two words at any number of chains
+// (9 against 10 ns a site at 1024 chains and L = 64, the same 19 at 4096),
+// rows of four with at most two warps a scheduler (L = 100, 32 chains: 9.0
+// against 11.8; L = 128, 1024 chains: 9.7 against 11.7; 4096 chains: 31
+// against 26).  Rows of three words would still be two windows: one a lane
+// (L = 96, 1280 chains: 12.0 against 15.7).
+__host__ __device__ inline bool warp_pairs(int L, int p, int num_sms) {
+  const int wd = (L + 31) / 32;
+  return wd == 2 || (wd == 4 && p <= 8 * num_sms);
 }
 
 // Warps a block and the table's place.  The time of a round is set by the
@@ -106,11 +127,11 @@ inline void warp_chain_shape(int L, int p, int num_sms, int* warps, bool* tsmem)
 //   L = 20    16 / 33 at 1200, 25 / 33 at 3000
 //   L = 32    8.9 / 28 at 512 or fewer, 13 / 28 at 2048, 21 / 28 at 4096, 41 / 29 at 5500
 //   L = 36    19 / 96 at 2048 (no lane kernel with L fixed at compile time)
-//   L = 64    9.4 / 26 at 1024, 20 / 29 at 4096, 33 / 42 at 5500, 37 / 42 at 8192
+//   L = 64    8.7 / 26 at 1024, 19 / 29 at 4096, 33 / 42 at 5500, 43 / 42 at 8192
 //   L = 76    39 / 80 at 6000, 50 / 80 at 9000
 //   L = 96    13 / 44 at 1280, 19 / 45 at 4096, 40 / 52 at 8192
-//   L = 100   12 / 53 at 32, 23 / 76 at 4096, 46 / 169 at 8000
-//   L = 128   12 / 53 at 1024, 25 / 64 at 4096, 59 / 69 at 6000, 88 / 75 at 8192
+//   L = 100   9.0 / 53 at 32, 23 / 76 at 4096, 46 / 169 at 8000
+//   L = 128   9.6 / 53 at 1024, 20 / 64 at 4096, 59 / 69 at 6000, 88 / 75 at 8192
 inline bool warp_chain_better(int L, int p, int num_sms) {
   int most = 8;                                               // one wave
   if (L < 12) most = 0;
@@ -138,11 +159,30 @@ __device__ __forceinline__ uint32_t warp_threshold(const uint32_t* __restrict__ 
   }
 }
 
-// Evaluate the flip mask F until it reproduces itself (at most one
-// evaluation a site: the sites before the first wrong one stay right).
-// Returns this lane's level change before its site (lane 0: of the whole
-// word).  Written as one PTX block so that the loop's branch is uniform.
-#define MC_EVAL(WRAP_, LOAD_)                                        \
+// Flips along a row of sites of which lane l's flips iff its left neighbour
+// (lane l - 1) did and H1 says so, or did not and H0 says so; H0 and H1 agree
+// at lane 0.  The nearest lane at or before l where they agree fixes the
+// flip there; each lane between where only the unflipped neighbour lets the
+// site flip inverts it.
+__device__ __forceinline__ uint32_t warp_solve(uint32_t H0, uint32_t H1, uint32_t le) {
+  const uint32_t dif = H0 ^ H1;
+  const int anchor = 31 - __clz(~dif & le);
+  const uint32_t inv = dif & H0 & le & (0xFFFFFFFEu << anchor);
+  return __ballot_sync(0xFFFFFFFFu, ((H0 >> anchor) ^ __popc(inv)) & 1u);
+}
+
+// The fixed-point loops, written as PTX blocks so that their branch is
+// uniform (as C++ loops the compiler re-converged the warp at every vote: 10 %
+// slower).  Both end after at most one evaluation a site: the sites before
+// the first wrong one stay right.
+#define MC_LOAD_SHARED(at, to) "ld.shared.u32 " to ", [" at "];\n\t"
+#define MC_LOAD_GLOBAL(at, to, T, last)            \
+  "min.u32 " at ", " at ", " last ";\n\t"          \
+  "{ .reg .b64 g; cvt.u64.u32 g, " at "; add.s64 g, g, " T "; ld.global.nc.u32 " to ", [g]; }\n\t"
+
+// One site a lane.  Returns this lane's level change before its site (lane 0,
+// whose `before` is the whole word: of the word).
+#define MC_EVAL1(WRAP_, LOAD_)                                       \
   "{\n\t"                                                            \
   ".reg .pred p, q, v;\n\t"                                          \
   ".reg .b32 fs, x, a, b, c, at, t, fn;\n\t"                         \
@@ -168,14 +208,10 @@ __device__ __forceinline__ uint32_t warp_threshold(const uint32_t* __restrict__ 
   "mov.b32 %0, fn;\n\t"                                              \
   "@q bra.uni EVAL;\n\t"                                             \
   "}"
-#define MC_EVAL_WRAP                       \
-  "and.b32 t, %0, 1;\n\t"                  \
-  "setp.eq.u32 q, t, 0;\n\t"               \
-  "@q add.s32 at, at, %10;\n\t"
-#define MC_EVAL_SHARED "ld.shared.u32 t, [at];\n\t"
-#define MC_EVAL_GLOBAL                     \
-  "min.u32 at, at, %14;\n\t"               \
-  "{ .reg .b64 g; cvt.u64.u32 g, at; add.s64 g, g, %13; ld.global.nc.u32 t, [g]; }\n\t"
+#define MC_EVAL_WRAP(at, F, delta)         \
+  "and.b32 x, " F ", 1;\n\t"               \
+  "setp.eq.u32 q, x, 0;\n\t"               \
+  "@q add.s32 " at ", " at ", " delta ";\n\t"
 template <bool WRAP, bool TSMEM>
 __device__ __forceinline__ int warp_fixed_point(uint32_t& F, uint32_t s0, uint32_t ns1, uint32_t el, uint32_t before,
                                                 uint32_t bit, int row, int row1, int dwrap, int scale, uint32_t u,
@@ -186,167 +222,439 @@ __device__ __forceinline__ int warp_fixed_point(uint32_t& F, uint32_t s0, uint32
   : "r"(s0), "r"(ns1), "r"(el), "r"(before), "r"(bit), "r"(row), "r"(row1), "r"(scale), "r"(dwrap), "r"(u),     \
     "r"(static_cast<uint32_t>(valid)), "l"(T), "r"(last)
   if constexpr (WRAP) {
-    if constexpr (TSMEM) asm volatile(MC_EVAL(MC_EVAL_WRAP, MC_EVAL_SHARED) MC_EVAL_ARGS);
-    else asm volatile(MC_EVAL(MC_EVAL_WRAP, MC_EVAL_GLOBAL) MC_EVAL_ARGS);
+    if constexpr (TSMEM) asm volatile(MC_EVAL1(MC_EVAL_WRAP("at", "%0", "%10"), MC_LOAD_SHARED("at", "t")) MC_EVAL_ARGS);
+    else asm volatile(MC_EVAL1(MC_EVAL_WRAP("at", "%0", "%10"), MC_LOAD_GLOBAL("at", "t", "%13", "%14")) MC_EVAL_ARGS);
   } else {
-    if constexpr (TSMEM) asm volatile(MC_EVAL("", MC_EVAL_SHARED) MC_EVAL_ARGS);
-    else asm volatile(MC_EVAL("", MC_EVAL_GLOBAL) MC_EVAL_ARGS);
+    if constexpr (TSMEM) asm volatile(MC_EVAL1("", MC_LOAD_SHARED("at", "t")) MC_EVAL_ARGS);
+    else asm volatile(MC_EVAL1("", MC_LOAD_GLOBAL("at", "t", "%13", "%14")) MC_EVAL_ARGS);
   }
 #undef MC_EVAL_ARGS
   return d;
 }
-#undef MC_EVAL
-#undef MC_EVAL_WRAP
-#undef MC_EVAL_SHARED
-#undef MC_EVAL_GLOBAL
+#undef MC_EVAL1
 
-// 2-byte store of the round record, opaque to the compiler's memory ordering (nothing here reads it)
+// Two sites a lane: masks of the even and of the odd sites; the even site's
+// left neighbour is the odd site of the lane before, the odd site's is the
+// lane's own even site.  Returns the level change before the even site (lane
+// 0: of the window) and, in `mid`, 4 times the change before the odd one.
+#define MC_EVAL2(WRAP_, LOAD_E_, LOAD_O_)                            \
+  "{\n\t"                                                            \
+  ".reg .pred p, q, r, v;\n\t"                                       \
+  ".reg .b32 fs, x, a, b, c, e, f, g, t, ae, ao, mv;\n\t"            \
+  "setp.ne.u32 v, %22, 0;\n\t"                                       \
+  "EVAL:\n\t"                                                        \
+  "shl.b32 fs, %1, 1;\n\t"                                           \
+  "and.b32 x, %0, %10;\n\t"                                          \
+  "and.b32 t, %1, %10;\n\t"                                          \
+  "and.b32 a, x, %4;\n\t"                                            \
+  "lop3.b32 b, fs, %6, x, 0x28;\n\t"                                 \
+  "and.b32 c, x, %5;\n\t"                                            \
+  "and.b32 e, t, %7;\n\t"                                            \
+  "lop3.b32 f, %0, %9, t, 0x28;\n\t"                                 \
+  "and.b32 g, t, %8;\n\t"                                            \
+  "popc.b32 a, a;\n\t"                                               \
+  "popc.b32 b, b;\n\t"                                               \
+  "popc.b32 c, c;\n\t"                                               \
+  "popc.b32 e, e;\n\t"                                               \
+  "popc.b32 f, f;\n\t"                                               \
+  "popc.b32 g, g;\n\t"                                               \
+  "and.b32 x, fs, %11;\n\t"                                          \
+  "setp.ne.u32 q, x, 0;\n\t"                                         \
+  "and.b32 x, %0, %11;\n\t"                                          \
+  "setp.ne.u32 r, x, 0;\n\t"                                         \
+  "selp.b32 ae, %13, %12, q;\n\t"                                    \
+  "selp.b32 ao, %15, %14, r;\n\t"                                    \
+  "selp.b32 mv, %17, %16, q;\n\t"                                    \
+  "selp.b32 mv, mv, 0, r;\n\t" WRAP_                                 \
+  "add.s32 a, a, b;\n\t"                                             \
+  "add.s32 e, e, f;\n\t"                                             \
+  "add.s32 c, c, g;\n\t"                                             \
+  "add.s32 a, a, e;\n\t"                                             \
+  "mad.lo.s32 %2, c, -2, a;\n\t"                                     \
+  "mad.lo.s32 ae, %2, %18, ae;\n\t"                                  \
+  "mad.lo.s32 %3, %2, %18, mv;\n\t"                                  \
+  "add.s32 ao, ao, %3;\n\t" LOAD_E_ LOAD_O_                          \
+  "setp.le.and.u32 p, %19, a, v;\n\t"                                \
+  "setp.le.and.u32 q, %20, b, v;\n\t"                                \
+  "vote.sync.ballot.b32 a, p, 0xffffffff;\n\t"                       \
+  "vote.sync.ballot.b32 b, q, 0xffffffff;\n\t"                       \
+  "xor.b32 c, a, %0;\n\t"                                            \
+  "lop3.b32 c, b, %1, c, 0xBE;\n\t"                                  \
+  "setp.ne.u32 q, c, 0;\n\t"                                         \
+  "mov.b32 %0, a;\n\t"                                               \
+  "mov.b32 %1, b;\n\t"                                               \
+  "@q bra.uni EVAL;\n\t"                                             \
+  "}"
+template <bool WRAP, bool TSMEM>
+__device__ __forceinline__ int warp_fixed_point2(uint32_t& FE, uint32_t& FO, int& mid, uint32_t s0E, uint32_t nsE,
+                                                 uint32_t elE, uint32_t s0O, uint32_t nsO, uint32_t elO,
+                                                 uint32_t before, uint32_t bit, int rowE, int rowE1, int rowO,
+                                                 int rowO1, int moveE, int moveE1, int scale, uint32_t uE, uint32_t uO,
+                                                 int dwrap, bool valid, const uint32_t* __restrict__ T, uint32_t last) {
+  int d;
+#define MC_EVAL_ARGS                                                                                              \
+  : "+r"(FE), "+r"(FO), "=&r"(d), "=&r"(mid)                                                                      \
+  : "r"(s0E), "r"(nsE), "r"(elE), "r"(s0O), "r"(nsO), "r"(elO), "r"(before), "r"(bit), "r"(rowE), "r"(rowE1),     \
+    "r"(rowO), "r"(rowO1), "r"(moveE), "r"(moveE1), "r"(scale), "r"(uE), "r"(uO), "r"(dwrap),                     \
+    "r"(static_cast<uint32_t>(valid)), "l"(T), "r"(last)
+  if constexpr (TSMEM) {
+    if constexpr (WRAP)
+      asm volatile(MC_EVAL2(MC_EVAL_WRAP("ao", "%0", "%21"), MC_LOAD_SHARED("ae", "a"), MC_LOAD_SHARED("ao", "b")) MC_EVAL_ARGS);
+    else
+      asm volatile(MC_EVAL2("", MC_LOAD_SHARED("ae", "a"), MC_LOAD_SHARED("ao", "b")) MC_EVAL_ARGS);
+  } else {
+    if constexpr (WRAP)
+      asm volatile(MC_EVAL2(MC_EVAL_WRAP("ao", "%0", "%21"), MC_LOAD_GLOBAL("ae", "a", "%23", "%24"), MC_LOAD_GLOBAL("ao", "b", "%23", "%24")) MC_EVAL_ARGS);
+    else
+      asm volatile(MC_EVAL2("", MC_LOAD_GLOBAL("ae", "a", "%23", "%24"), MC_LOAD_GLOBAL("ao", "b", "%23", "%24")) MC_EVAL_ARGS);
+  }
+#undef MC_EVAL_ARGS
+  return d;
+}
+#undef MC_EVAL2
+#undef MC_EVAL_WRAP
+#undef MC_LOAD_SHARED
+#undef MC_LOAD_GLOBAL
+
+// What every window needs of the block and the lane.
+struct WarpLane {
+  int L, lane;
+  uint32_t bit, lt, le, before;   // this lane, those before it, and it; `before` is everything for lane 0
+  int scale;                      // 4; 0 for lane 0, whose sum is the window's
+  int r1, r1z, row2;              // a table row in bytes; 0 for lane 0; row 2 at level 0
+  const uint32_t* T;
+  uint32_t t_last;                // last byte offset of the table (global memory)
+  uint32_t hist_a;                // shared address of the level counters
+  uint16_t* rec;                  // this lane's place in the round record
+};
+
+// Uniforms: a ring in shared memory, filled 128 at a time, a Philox block a lane.
+struct WarpRing {
+  char* ring;
+  int avail = 0;
+  uint32_t fill_at = 0, use_at;
+  uint64_t blk;
+  uint32_t chain, k0, k1;
+  __device__ __forceinline__ void need(int nb, int lane) {
+    if (avail < nb) {
+      const uint4 v =
+          philox4x32_10(make_uint4(static_cast<uint32_t>(blk), static_cast<uint32_t>(blk >> 32), chain, kTagFlip), k0, k1);
+      blk += 32;
+      *reinterpret_cast<uint4*>(ring + fill_at + 16 * lane) = v;
+      fill_at ^= 512u;
+      avail += 128;
+      __syncwarp();
+    }
+    avail -= nb;
+  }
+  __device__ __forceinline__ void step(int nb) { use_at = (use_at + 4u * nb) & (4u * kRingWords - 1u); }
+};
+
+// stores of the round record, opaque to the compiler's memory ordering (nothing here reads it)
 __device__ __forceinline__ void st_record1(uint16_t* p, int lvl) {
   asm volatile("st.global.u16 [%0], %1;" ::"l"(p), "h"(static_cast<uint16_t>(lvl)));
 }
+__device__ __forceinline__ void st_record2(uint16_t* p, uint32_t pair) {
+  asm volatile("st.global.u32 [%0], %1;" ::"l"(p), "r"(pair));
+}
+__device__ __forceinline__ void warp_count(uint32_t addr) {
+  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(1u));
+}
 
-// One block of the round: `warps` chains, chain blockIdx-wise first + warp.
-template <int WD, bool TSMEM, bool REC>
+// Rows of WD words, a window a word: lane l holds site l of the word.
+template <int WD>
+struct Words {
+  static constexpr int kRowWords = WD, kSitesPerLane = 1;
+  uint32_t up[WD], cur[WD];
+  __device__ __forceinline__ void begin(const uint32_t* lat, int L) {
+#pragma unroll
+    for (int w = 0; w < WD; ++w) {
+      up[w] = lat[(L - 1) * WD + w];
+      cur[w] = lat[w];
+    }
+  }
+  __device__ __forceinline__ static void load(uint32_t* lat, const uint32_t* g, int L, int lane) {
+    for (int i = lane; i < L * WD; i += 32) lat[i] = g[i];
+  }
+  __device__ __forceinline__ static void store(uint32_t* g, size_t stride, const uint32_t* lat, int L, int lane) {
+    for (int i = lane; i < L * WD; i += 32) g[i * stride] = lat[i];
+  }
+  template <bool TSMEM, bool REC>
+  __device__ __forceinline__ void row(uint32_t* lat, int y, int& m, WarpLane& w, WarpRing& ring) {
+    const int L = w.L, lw = L - 32 * (WD - 1);   // sites of the last word
+    const int yp = y + 1 == L ? 0 : y + 1;
+    uint32_t dn[WD];
+#pragma unroll
+    for (int v = 0; v < WD; ++v) dn[v] = lat[yp * WD + v];
+#pragma unroll
+    for (int v = 0; v < WD; ++v) {
+      const bool lastv = v == WD - 1;
+      const int nb = lastv ? lw : 32;
+      const bool valid = lastv ? w.lane < lw : true, wrap = WD == 1 && w.lane == lw - 1;
+      ring.need(nb, w.lane);
+      const uint32_t u = *reinterpret_cast<const uint32_t*>(ring.ring + ring.use_at);
+      ring.step(nb);
+      // agreements with the neighbours: up and left as swept, down and right as they are (the last site of
+      // the row sees site 0 as swept: in a one-word row that is taken as flipped, as most attempts are
+      // accepted, and corrected where F says otherwise)
+      const uint32_t c = cur[v];
+      const uint32_t right =
+          (c >> 1) | (lastv ? (((WD == 1 ? ~c : cur[0]) & 1u) << (lw - 1)) : (cur[(v + 1) % WD] << 31));
+      const uint32_t left =
+          (c << 1) | (v > 0 ? (cur[(v + WD - 1) % WD] >> 31) : ((cur[WD - 1] >> (lw - 1)) & 1u));
+      const uint32_t eu = ~(c ^ up[v]), ed = ~(c ^ dn[v]), er = ~(c ^ right), el = ~(c ^ left);
+      const uint32_t s0 = eu ^ ed ^ er;
+      const uint32_t ns1 = ~((eu & ed) | (er & (eu ^ ed)));
+      // table entries at the word's first level for an unflipped and a flipped left neighbour (the first
+      // site's left neighbour is outside the word: the same)
+      int off = w.row2, off1 = w.r1z;
+      if (s0 & w.bit) off += w.r1;
+      if (ns1 & w.bit) off -= 2 * w.r1;
+      if (el & w.bit) {
+        off += w.r1;
+        off1 = -w.r1z;
+      }
+      const int dwrap = wrap ? ((er & w.bit) ? -w.r1 : w.r1) : 0;
+      const int row = 4 * m + off, row1 = row + off1;
+      const uint32_t ta = warp_threshold<TSMEM>(w.T, row, w.t_last);
+      const uint32_t tb = warp_threshold<TSMEM>(w.T, row1, w.t_last);
+      const uint32_t G0 = __ballot_sync(0xFFFFFFFFu, valid && u <= ta);
+      const uint32_t G1 = __ballot_sync(0xFFFFFFFFu, valid && u <= tb);
+      uint32_t F = warp_solve(G0, G1, w.le);
+      const int d = warp_fixed_point<WD == 1, TSMEM>(F, s0, ns1, el, w.before, w.bit, row, row1, dwrap, w.scale, u,
+                                                     valid, w.T, w.t_last);
+      // the samples' levels: what the next site finds before its attempt, lane 0's sum after the last
+      int lvl = m + __shfl_sync(0xFFFFFFFFu, d, (w.lane + 1) & 31);
+      int m1 = m + __shfl_sync(0xFFFFFFFFu, d, 0);
+      if constexpr (WD == 1) {
+        if (!(F & 1u) && ((F >> (lw - 1)) & 1u)) {   // the last site's move, with site 0 as it is
+          const int fix = ((er >> (lw - 1)) & 1u) ? -1 : 1;
+          m1 += fix;
+          if (wrap) lvl += fix;
+        }
+      }
+      m = m1;
+      if (valid) warp_count(w.hist_a + 4u * lvl);
+      if constexpr (REC) {
+        if (valid) st_record1(w.rec, lvl);
+        w.rec += (nb >> 2) * kRecGroupStride;
+      }
+      cur[v] = c ^ F;
+    }
+    // (every lane stores the same words)
+#pragma unroll
+    for (int v = 0; v < WD; ++v) {
+      lat[y * WD + v] = up[v] = cur[v];
+      cur[v] = dn[v];
+    }
+  }
+};
+
+// Even bits of x in the low half, and back.
+__device__ __forceinline__ uint32_t bits_even(uint32_t x) {
+  x &= 0x55555555u;
+  x = (x | (x >> 1)) & 0x33333333u;
+  x = (x | (x >> 2)) & 0x0F0F0F0Fu;
+  x = (x | (x >> 4)) & 0x00FF00FFu;
+  return (x | (x >> 8)) & 0xFFFFu;
+}
+__device__ __forceinline__ uint32_t bits_spread(uint32_t x) {
+  x &= 0xFFFFu;
+  x = (x | (x << 8)) & 0x00FF00FFu;
+  x = (x | (x << 4)) & 0x0F0F0F0Fu;
+  x = (x | (x << 2)) & 0x33333333u;
+  return (x | (x << 1)) & 0x55555555u;
+}
+
+// Rows of more than 32 sites, in windows of 64: lane l holds sites 2l and
+// 2l + 1 of the window, the lattice copy the window's even and odd sites as
+// two words (so that neighbours in the row are the other word, or its
+// neighbour bit).  Against 32 sites a window, one a lane: half the solves and
+// a third fewer evaluations a site (2.1 for 64 sites, 1.6 for 32).
+template <int NW>
+struct TwoWords {
+  static constexpr int kRowWords = 2 * NW, kSitesPerLane = 2;
+  uint32_t upE[NW], upO[NW], E[NW], O[NW];
+  __device__ __forceinline__ void begin(const uint32_t* lat, int L) {
+#pragma unroll
+    for (int v = 0; v < NW; ++v) {
+      upE[v] = lat[(L - 1) * 2 * NW + 2 * v];
+      upO[v] = lat[(L - 1) * 2 * NW + 2 * v + 1];
+      E[v] = lat[2 * v];
+      O[v] = lat[2 * v + 1];
+    }
+  }
+  __device__ __forceinline__ static void load(uint32_t* lat, const uint32_t* g, int L, int lane) {
+    const int wd = (L + 31) / 32;
+    for (int i = lane; i < L * NW; i += 32) {
+      const int y = i / NW, v = i % NW;
+      const uint32_t a = g[y * wd + 2 * v], b = 2 * v + 1 < wd ? g[y * wd + 2 * v + 1] : 0u;
+      lat[2 * i] = bits_even(a) | (bits_even(b) << 16);
+      lat[2 * i + 1] = bits_even(a >> 1) | (bits_even(b >> 1) << 16);
+    }
+  }
+  __device__ __forceinline__ static void store(uint32_t* g, size_t stride, const uint32_t* lat, int L, int lane) {
+    const int wd = (L + 31) / 32;
+    for (int i = lane; i < L * wd; i += 32) {
+      const int y = i / wd, x = i % wd, at = 2 * (y * NW + x / 2), sh = 16 * (x & 1);
+      g[i * stride] = bits_spread(lat[at] >> sh) | (bits_spread(lat[at + 1] >> sh) << 1);
+    }
+  }
+  template <bool TSMEM, bool REC>
+  __device__ __forceinline__ void row(uint32_t* lat, int y, int& m, WarpLane& w, WarpRing& ring) {
+    const int L = w.L;
+    const int yp = y + 1 == L ? 0 : y + 1;
+    const int nl = L - 64 * (NW - 1), hl = nl >> 1;   // sites and lanes of the last window
+    uint32_t dnE[NW], dnO[NW];
+#pragma unroll
+    for (int v = 0; v < NW; ++v) {
+      dnE[v] = lat[yp * 2 * NW + 2 * v];
+      dnO[v] = lat[yp * 2 * NW + 2 * v + 1];
+    }
+#pragma unroll
+    for (int v = 0; v < NW; ++v) {
+      const bool lastv = v == NW - 1;
+      const int nb = lastv ? nl : 64;
+      const bool valid = lastv ? w.lane < hl : true;
+      ring.need(nb, w.lane);
+      const uint2 u = *reinterpret_cast<const uint2*>(ring.ring + ring.use_at);
+      ring.step(nb);
+      // agreements with the neighbours, as in Words: `pair` between the lane's two sites
+      const uint32_t e = E[v], o = O[v];
+      const uint32_t left = (o << 1) | (v > 0 ? (O[(v + NW - 1) % NW] >> 31) : ((O[NW - 1] >> (hl - 1)) & 1u));
+      const uint32_t right =
+          (e >> 1) | (lastv ? (((NW == 1 ? ~e : E[0]) & 1u) << (hl - 1)) : (E[(v + 1) % NW] << 31));
+      const uint32_t pair = ~(e ^ o), elE = ~(e ^ left), erO = ~(o ^ right);
+      const uint32_t euE = ~(e ^ upE[v]), edE = ~(e ^ dnE[v]), euO = ~(o ^ upO[v]), edO = ~(o ^ dnO[v]);
+      const uint32_t s0E = euE ^ edE ^ pair, s0O = euO ^ edO ^ erO;
+      const uint32_t nsE = ~((euE & edE) | (pair & (euE ^ edE))), nsO = ~((euO & edO) | (erO & (euO ^ edO)));
+      // the moves in levels (aligned neighbours - 2) with an unflipped left neighbour, and their change
+      // with a flipped one (none for the window's first site)
+      int mE = 0, mO = 0, cE = w.lane ? 1 : 0, cO = 1;
+      if (s0E & w.bit) mE += 1;
+      if (nsE & w.bit) mE -= 2;
+      if (elE & w.bit) mE += 1, cE = -cE;
+      if (s0O & w.bit) mO += 1;
+      if (nsO & w.bit) mO -= 2;
+      if (pair & w.bit) mO += 1, cO = -1;
+      int dwrap = 0;
+      if constexpr (NW == 1)
+        if (w.lane == hl - 1) dwrap = (erO & w.bit) ? -w.r1 : w.r1;
+      const int base = 4 * m + w.row2;
+      const int rowE = base + mE * w.r1, rowE1 = rowE + cE * w.r1;
+      const int rowO = base + mO * w.r1, rowO1 = rowO + cO * w.r1;
+      const uint32_t tE0 = warp_threshold<TSMEM>(w.T, rowE, w.t_last);
+      const uint32_t tE1 = warp_threshold<TSMEM>(w.T, rowE1, w.t_last);
+      const uint32_t tO0 = warp_threshold<TSMEM>(w.T, rowO, w.t_last);
+      const uint32_t tO1 = warp_threshold<TSMEM>(w.T, rowO1, w.t_last);
+      const uint32_t GE0 = __ballot_sync(0xFFFFFFFFu, valid && u.x <= tE0);
+      const uint32_t GE1 = __ballot_sync(0xFFFFFFFFu, valid && u.x <= tE1);
+      const uint32_t GO0 = __ballot_sync(0xFFFFFFFFu, valid && u.y <= tO0);
+      const uint32_t GO1 = __ballot_sync(0xFFFFFFFFu, valid && u.y <= tO1);
+      // solve the odd sites, each pair of sites one step; the even ones follow
+      uint32_t FO = warp_solve((GE0 & GO1) | (~GE0 & GO0), (GE1 & GO1) | (~GE1 & GO0), w.le);
+      uint32_t FE = ((FO << 1) & GE1) | (~(FO << 1) & GE0);
+      int mid;
+      const int d = warp_fixed_point2<NW == 1, TSMEM>(FE, FO, mid, s0E, nsE, elE, s0O, nsO, pair, w.before, w.bit, rowE,
+                                                      rowE1, rowO, rowO1, 4 * mE, 4 * (mE + cE), w.scale, u.x, u.y,
+                                                      dwrap, valid, w.T, w.t_last);
+      // the samples' levels: after the even site, what the odd one finds; after the odd site, what the
+      // next lane finds (lane 0's sum after the last)
+      const int m4 = 4 * m;
+      int lo = m + __shfl_sync(0xFFFFFFFFu, d, (w.lane + 1) & 31);
+      int m1 = m + __shfl_sync(0xFFFFFFFFu, d, 0);
+      if constexpr (NW == 1) {
+        if (!(FE & 1u) && ((FO >> (hl - 1)) & 1u)) {   // the last site's move, with site 0 as it is
+          const int fix = ((erO >> (hl - 1)) & 1u) ? -1 : 1;
+          m1 += fix;
+          if (w.lane == hl - 1) lo += fix;
+        }
+      }
+      m = m1;
+      if (valid) {
+        warp_count(w.hist_a + static_cast<uint32_t>(m4 + mid));
+        warp_count(w.hist_a + 4u * lo);
+      }
+      if constexpr (REC) {
+        if (valid) st_record2(w.rec, (static_cast<uint32_t>(m4 + mid) >> 2) | (static_cast<uint32_t>(lo) << 16));
+        w.rec += (nb >> 2) * kRecGroupStride;
+      }
+      E[v] = e ^ FE;
+      O[v] = o ^ FO;
+    }
+    // (every lane stores the same words)
+#pragma unroll
+    for (int v = 0; v < NW; ++v) {
+      lat[y * 2 * NW + 2 * v] = upE[v] = E[v];
+      lat[y * 2 * NW + 2 * v + 1] = upO[v] = O[v];
+      E[v] = dnE[v];
+      O[v] = dnO[v];
+    }
+  }
+};
+
+// One block of the round: its warps' chains, first + warp.
+template <class Rows, bool TSMEM, bool REC>
 __device__ __forceinline__ void warp_gen_body(const DevJob& j, const uint64_t t0, const int64_t S,
                                               const int64_t flushF, const int do_trace, const int block) {
   extern __shared__ __align__(16) uint32_t smem[];
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
   const int L = j.L, np1 = j.np1;
   const WarpPlan pl = warp_plan(L, nthr >> 5, TSMEM);
-  uint32_t* ring = smem + pl.ring + warp * kRingWords;
   uint32_t* hist = smem + pl.hist;
-  uint32_t* lat = smem + pl.lat + warp * L * WD;
+  uint32_t* lat = smem + pl.lat + warp * L * Rows::kRowWords;
   if constexpr (TSMEM)
     for (int i = tid; i < 5 * np1; i += nthr) smem[pl.table + i] = j.T[i];
   for (int i = tid; i < np1; i += nthr) hist[i] = 0u;
-  const uint32_t* __restrict__ T = j.T;
-  const uint32_t t_last = static_cast<uint32_t>(4 * (5 * np1 - 1));
-  const int t_base = TSMEM ? static_cast<int>(__cvta_generic_to_shared(smem + pl.table)) : 0;
   const int chain = block * (nthr >> 5) + warp;
   const bool active = chain < j.p;   // (uniform in a warp)
+  uint32_t* spins = j.spins + static_cast<size_t>(active ? chain : 0) * L * j.wd;
   int m = 0;
   if (active) {
-    const uint32_t* g = j.spins + static_cast<size_t>(chain) * L * WD;
-    for (int i = lane; i < L * WD; i += 32) lat[i] = g[i];
+    Rows::load(lat, spins, L, lane);
     m = j.m[chain];
   }
   __syncthreads();
-  const int lw = L - 32 * (WD - 1);
-  const uint32_t bit = 1u << lane, lt = bit - 1u, le = (bit << 1) - 1u;
-  // lane 0 sums the whole word's level changes instead of the (none) before its site
-  const uint32_t before = lane ? lt : 0xFFFFFFFFu;
-  const int scale = lane ? 4 : 0;
-  const int r1 = 4 * np1, r1z = lane ? r1 : 0;   // a row of the table in bytes; none for site 0's left neighbour
-  const int row2 = 2 * r1 + t_base;
-  const bool in_last = lane < lw;                // this lane has a site in the row's last word
-  const bool wrap = WD == 1 && lane == lw - 1;   // ... the site that sees site 0 of the same word
-  int avail = 0;                                 // uniforms in the ring not used yet
-  uint32_t fill_at = 0, use_at = 4u * lane;      // ring positions, bytes
-  const uint32_t hist_a = static_cast<uint32_t>(__cvta_generic_to_shared(hist));
-  uint64_t blk = (t0 >> 2) + static_cast<uint64_t>(lane);   // this lane's next Philox block
-  uint16_t* rec = nullptr;
-  if constexpr (REC)
-    rec = j.rec + rec_index(active ? chain : 0, 0, S * j.N) + (lane >> 2) * kRecGroupStride + (lane & 3);
+  WarpLane w;
+  w.L = L;
+  w.lane = lane;
+  w.bit = 1u << lane;
+  w.lt = w.bit - 1u;
+  w.le = (w.bit << 1) - 1u;
+  w.before = lane ? w.lt : 0xFFFFFFFFu;
+  w.scale = lane ? 4 : 0;
+  w.r1 = 4 * np1;
+  w.r1z = lane ? w.r1 : 0;
+  w.row2 = 2 * w.r1 + (TSMEM ? static_cast<int>(__cvta_generic_to_shared(smem + pl.table)) : 0);
+  w.T = j.T;
+  w.t_last = static_cast<uint32_t>(4 * (5 * np1 - 1));
+  w.hist_a = static_cast<uint32_t>(__cvta_generic_to_shared(hist));
+  w.rec = nullptr;
+  if constexpr (REC) {
+    const int k = Rows::kSitesPerLane * lane;   // this lane's first sample in a window
+    w.rec = j.rec + rec_index(active ? chain : 0, 0, S * j.N) + (k >> 2) * kRecGroupStride + (k & 3);
+  }
+  WarpRing ring;
+  ring.ring = reinterpret_cast<char*>(smem + pl.ring + warp * kRingWords);
+  ring.use_at = 4u * Rows::kSitesPerLane * lane;
+  ring.blk = (t0 >> 2) + static_cast<uint64_t>(lane);
+  ring.chain = static_cast<uint32_t>(chain);
+  ring.k0 = j.key0;
+  ring.k1 = j.key1;
   int ck_left = 0, seg = 0;
   int64_t fl_left = flushF;
   for (int64_t s = 0; s < S; ++s) {
     if (active) {
       if (j.ckpt && ck_left == 0) {
         // lattice and level at the start of segment s / C, for the joint's replays
-        uint32_t* ck = j.ckpt + static_cast<size_t>(seg) * L * WD * j.p + chain;
-        for (int i = lane; i < L * WD; i += 32) ck[static_cast<size_t>(i) * j.p] = lat[i];
+        Rows::store(j.ckpt + static_cast<size_t>(seg) * L * j.wd * j.p + chain, static_cast<size_t>(j.p), lat, L, lane);
         if (lane == 0) j.ckm[static_cast<size_t>(seg) * j.p + chain] = m;
       }
-      uint32_t up[WD], cur[WD];
-#pragma unroll
-      for (int w = 0; w < WD; ++w) {
-        up[w] = lat[(L - 1) * WD + w];
-        cur[w] = lat[w];
-      }
+      Rows rows;
+      rows.begin(lat, L);
 #pragma unroll 1
       for (int y = 0; y < L; ++y) {
-        uint32_t dn[WD];
-        const int yp = (y + 1 == L) ? 0 : y + 1;
-#pragma unroll
-        for (int w = 0; w < WD; ++w) dn[w] = lat[yp * WD + w];
-#pragma unroll
-        for (int w = 0; w < WD; ++w) {
-          const bool lastw = w == WD - 1;
-          const int nb = lastw ? lw : 32;
-          const bool valid = lastw ? in_last : true;
-          if (avail < nb) {   // the next 128 uniforms, a Philox block a lane
-            const uint4 v = philox4x32_10(
-                make_uint4(static_cast<uint32_t>(blk), static_cast<uint32_t>(blk >> 32), static_cast<uint32_t>(chain),
-                           kTagFlip),
-                j.key0, j.key1);
-            blk += 32;
-            *reinterpret_cast<uint4*>(ring + (fill_at >> 2) + 4 * lane) = v;
-            fill_at ^= 512u;
-            avail += 128;
-            __syncwarp();
-          }
-          const uint32_t u = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(ring) + use_at);
-          use_at = (use_at + 4u * nb) & (4u * kRingWords - 1u);
-          avail -= nb;
-          // agreements with the neighbours: up and left as swept, down and right as they are
-          // (the last site of a row sees site 0 as swept: in a one-word row it is taken as flipped,
-          // as most attempts are accepted, and corrected where F says otherwise)
-          const uint32_t c = cur[w];
-          const uint32_t right =
-              (c >> 1) | (lastw ? (((WD == 1 ? ~c : cur[0]) & 1u) << (lw - 1)) : (cur[(w + 1) % WD] << 31));
-          const uint32_t left =
-              (c << 1) | (w > 0 ? (cur[(w + WD - 1) % WD] >> 31) : ((cur[WD - 1] >> (lw - 1)) & 1u));
-          const uint32_t eu = ~(c ^ up[w]), ed = ~(c ^ dn[w]), er = ~(c ^ right), el = ~(c ^ left);
-          const uint32_t s0 = eu ^ ed ^ er;
-          const uint32_t ns1 = ~((eu & ed) | (er & (eu ^ ed)));
-          // entry of the table at the word's first level for an unflipped and a flipped left neighbour
-          // (site 0's left neighbour is outside the word: the same)
-          int row = 4 * m + row2, row1 = r1z;
-          if (s0 & bit) row += r1;
-          if (ns1 & bit) row -= 2 * r1;
-          if (el & bit) {
-            row += r1;
-            row1 = -r1z;
-          }
-          row1 += row;
-          const int dwrap = wrap ? ((er & bit) ? -r1 : r1) : 0;
-          // solve with every site at the word's first level
-          const uint32_t ta = warp_threshold<TSMEM>(T, row, t_last);
-          const uint32_t tb = warp_threshold<TSMEM>(T, row1, t_last);
-          const uint32_t G0 = __ballot_sync(0xFFFFFFFFu, valid && u <= ta);
-          const uint32_t G1 = __ballot_sync(0xFFFFFFFFu, valid && u <= tb);
-          const uint32_t dif = G0 ^ G1;
-          const int anchor = 31 - __clz(~dif & le);   // (bit 0 always agrees)
-          const uint32_t inv = dif & G0 & le & (0xFFFFFFFEu << anchor);
-          uint32_t F = __ballot_sync(0xFFFFFFFFu, ((G0 >> anchor) ^ __popc(inv)) & 1u);
-          // evaluate until the mask reproduces itself (at most one evaluation a site)
-          const int d = warp_fixed_point<WD == 1, TSMEM>(F, s0, ns1, el, before, bit, row, row1, dwrap, scale, u,
-                                                         lastw ? in_last : true, T, t_last);
-          // the samples' levels: what the next site finds before its attempt, lane 0's sum after the last
-          int lvl = m + __shfl_sync(0xFFFFFFFFu, d, (lane + 1) & 31);
-          int m1 = m + __shfl_sync(0xFFFFFFFFu, d, 0);
-          if constexpr (WD == 1) {
-            if (!(F & 1u) && ((F >> (lw - 1)) & 1u)) {   // the last site's move, with site 0 as it is
-              const int fix = ((er >> (lw - 1)) & 1u) ? -1 : 1;
-              m1 += fix;
-              if (wrap) lvl += fix;
-            }
-          }
-          m = m1;
-          if (valid) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(hist_a + 4u * lvl), "r"(1u));
-          if constexpr (REC) {
-            if (valid) st_record1(rec, lvl);
-            rec += (nb >> 2) * kRecGroupStride;
-          }
-          cur[w] = c ^ F;
-        }
-        // (every lane stores the same words)
-#pragma unroll
-        for (int w = 0; w < WD; ++w) {
-          lat[y * WD + w] = cur[w];
-          up[w] = cur[w];
-          cur[w] = dn[w];
-        }
+        rows.template row<TSMEM, REC>(lat, y, m, w, ring);
         __syncwarp();
       }
       if (do_trace && lane == 0) j.trace[s * j.p + chain] = 4 * m - 2 * j.N;
@@ -371,8 +679,7 @@ __device__ __forceinline__ void warp_gen_body(const DevJob& j, const uint64_t t0
     }
   }
   if (active) {
-    uint32_t* g = j.spins + static_cast<size_t>(chain) * L * WD;
-    for (int i = lane; i < L * WD; i += 32) g[i] = lat[i];
+    Rows::store(spins, 1, lat, L, lane);
     if (lane == 0) j.m[chain] = m;
   }
   asm volatile("" ::: "memory");
