@@ -214,7 +214,7 @@ cudaError_t chain_kernels_record(const DevJob& j, int64_t S, uint32_t r, cudaStr
 
 // launch shape chosen by default for (L, p)
 LaunchShape default_shape(int L, int p, int num_sms);
-// fullest warps with the same table placement (what concurrent jobs want)
+// the shape of a job that runs beside others
 LaunchShape dense_shape(int L, int p, int num_sms);
 bool shape_supported(int L, const LaunchShape& s);
 size_t gen_smem_bytes(int L, const LaunchShape& s, bool* table_in_smem);

@@ -1260,13 +1260,17 @@ LaunchShape default_shape(int L, int p, int num_sms) {
   return lane_shape(L, p, num_sms);
 }
 
-// Densest shape for L and p: as many chains per warp as there are (up to 32),
-// keeping the threshold table in shared memory if the default shape has it
-// there.  The time of a round is set by the latency of one chain, which a
-// fuller warp does not change (measured: within 5 % for L <= 64 and 128), so
-// a job shaped this way takes the same time on far fewer warps -- the rest
-// of the GPU stays free for other jobs (the server uses it).
+// Shape of a job that shares the GPU with others (the server's).  One chain a
+// warp where that is the faster form alone: its rounds are so much shorter
+// that it also serves more (the 20-jobs-a-second stream of 400 jobs through 16
+// slots: 3.06e10 kept samples/s against 2.70e10 with full warps of one chain
+// a lane, latency p50 3.2 against 4.2 s).  Else as many chains a warp as there
+// are (up to 32), keeping the threshold table in shared memory if the default
+// shape has it there: the time of a round is set by the latency of one chain,
+// which a fuller warp does not change (measured: within 5 % for L <= 64 and
+// 128), so the job takes the same time on far fewer warps.
 LaunchShape dense_shape(int L, int p, int num_sms) {
+  if (warp_chain_better(L, p, num_sms)) return default_shape(L, p, num_sms);
   LaunchShape def = lane_shape(L, p, num_sms);
   // full warps at L = 100, 128 keep their lattices in global memory: a block
   // of 128 chains then needs only the histogram's shared memory, so blocks

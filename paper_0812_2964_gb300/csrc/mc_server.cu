@@ -98,7 +98,7 @@ int admit_job(mc_server* srv, Rec* r) {
   int rc = mc_init(s.L, s.n_chains, s.seed, s.start, &j);
   if (rc == MC_OK) rc = mc_set_stream(j, srv->slots[r->slot].st);
   if (rc == MC_OK) {
-    // fullest warps: the job's rounds take as long as alone, on fewer warps
+    // (a shape for jobs that share the GPU)
     const mcgpu::LaunchShape d = mcgpu::dense_shape(s.L, s.n_chains, srv->num_sms);
     rc = mc_set_launch_shape(j, d.placement, d.cpw, d.wpb);
   }
