@@ -118,7 +118,10 @@ int mc_run_attempts(mc_job *job, int64_t n_attempts);
  * from checkpoints (performance and memory only: both give the serial
  * rule's result).  The default is 2^33 (16 GiB of record); max_samples < 0
  * restores it, 0 turns the record off.  The record holds p rounded up to a
- * multiple of 32 chains.
+ * multiple of 32 chains.  At the default, larger rounds of up to 2^36 samples
+ * keep their accepted flips instead, one bit a sample (at most 8 GiB; where
+ * that cannot be allocated the round is replayed), from which the joint
+ * rebuilds the levels; any other limit turns that off too.
  * Rounds of mc_batch_run are not recorded.  MC_ESTATE while a round is
  * pending. */
 int mc_set_round_record(mc_job *job, int64_t max_samples);
@@ -178,7 +181,8 @@ int mc_set_weights(mc_job *job, const double *w, int n);
 
 /* How the joint resolves wrong speculations (performance only: every
  * policy gives the serial rule's result).  Rounds of at most
- * scan_max_samples samples (all chains; < 0: the default 2e10) run
+ * scan_max_samples samples (all chains; < 0: the default 2e10, no limit for
+ * rounds that keep their levels or flips) run
  * passes_before_scan speculative passes, then the summary replay and the
  * exact scan if chains are still pending, then passes_before_scan passes
  * more; larger rounds run passes_without_scan passes; whatever is left goes
@@ -193,7 +197,7 @@ int mc_set_join_policy(mc_job *job, int64_t scan_max_samples, int passes_before_
  * levels, the count of its discarded prefix) runs one segment per GPU lane,
  * so the segment length bounds the joint's critical path.  The library
  * aims at segments of about `samples` attempts (whole sweeps; 0 restores
- * the default of 2^16), keeps at least min(32, S) segments and at most
+ * the default of 2^16, of 2^14 where the round keeps its flips), keeps at least min(32, S) segments and at most
  * 2^24 samples per segment, and takes fewer, longer segments where their
  * checkpoints would exceed 4 GiB.  mc_get_info reports the choice of the
  * last round.  MC_EINVAL for samples < 0, MC_ESTATE while a round is

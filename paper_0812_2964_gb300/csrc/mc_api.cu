@@ -68,6 +68,8 @@ struct mc_job {
   uint16_t* rec_buf = nullptr;  // record of whole-sweep rounds (d.rec points here when used)
   size_t rec_cap = 0;           // uint16 entries of rec_buf
   long long rec_max = 0;                         // largest p * M recorded (set by mc_init)
+  uint32_t* flip_buf = nullptr; // flips of larger rounds (d.flips points here when used)
+  size_t flip_cap = 0;          // words of flip_buf
   bool pending = false;
   bool trace_on = false;
   bool trace_valid = false;
@@ -134,7 +136,10 @@ void free_all(mc_job* j) {
     raw_free(j, j->d.trace);
     raw_free(j, j->d.plv);
     raw_free(j, j->rec_buf);
+    raw_free(j, j->flip_buf);
   }
+  j->flip_buf = nullptr;
+  j->d.flips = nullptr;
   j->d.plv = nullptr;
   j->rec_buf = nullptr;
   j->d.rec = nullptr;
@@ -319,6 +324,10 @@ namespace {
 // samples each (the prefix pass relies on that bound), and no more segments
 // than kCheckpointBytes of checkpoints allow.
 constexpr int64_t kSegmentSamples = int64_t(1) << 16;   // default target
+// ... of rounds that keep their flips: rebuilding a segment's levels is so much
+// shorter than running it again that the first segments of a few hundred
+// chains, one a lane, would be most of a search (0.9 ms at 2^16)
+constexpr int64_t kFlipSegmentSamples = int64_t(1) << 14;
 constexpr int64_t kCheckpointBytes = int64_t(4) << 30;   // per job
 
 // Bytes of the checkpoint buffers per segment: lattices, levels, prefix work list.
@@ -338,6 +347,15 @@ void round_segments(int L, int p, int64_t n_sweeps, int64_t target, int* K, int*
   c = std::min<int64_t>(c, std::max<int64_t>(1, (int64_t(1) << 24) / N));
   *C = static_cast<int>(c);
   *K = static_cast<int>((n_sweeps + c - 1) / c);
+}
+
+// Words of the flip record of a round, 0 if it keeps none: rounds too large
+// for the record of levels (where that is not limited by mc_set_round_record)
+// up to kFlipMax samples.
+size_t flip_record_words(int L, int p, int64_t n_sweeps, long long rec_max) {
+  const long long samples = static_cast<long long>(p) * n_sweeps * L * L;
+  if (rec_max != mcgpu::default_record_max(L) || samples <= rec_max || samples > mcgpu::kFlipMax) return 0;
+  return static_cast<size_t>(p) * static_cast<size_t>(mcgpu::flip_words(L, n_sweeps));
 }
 
 // Bytes of the checkpoint buffers for K segments.
@@ -421,6 +439,31 @@ int ensure_record(mc_job* job, int64_t M, bool allow) {
   return MC_OK;
 }
 
+// Buffer for the round's flips; without memory for it the round is replayed.
+void ensure_flips(mc_job* job, int64_t n_sweeps, bool allow) {
+  DevJob& d = job->d;
+  d.flips = nullptr;
+  const size_t words = allow && !d.rec ? flip_record_words(job->L, job->p, n_sweeps, job->rec_max) : 0;
+  if (words == 0) return;
+  if (words > job->flip_cap) {
+    if (job->flip_buf) {
+      raw_free(job, job->flip_buf);
+      job->bytes -= job->flip_cap * sizeof(uint32_t);
+      job->flip_buf = nullptr;
+      job->flip_cap = 0;
+    }
+    void* v = nullptr;
+    if (raw_alloc(job, &v, words * sizeof(uint32_t)) != cudaSuccess) {
+      cudaGetLastError();   // (not an error of the call)
+      return;
+    }
+    job->flip_buf = static_cast<uint32_t*>(v);
+    job->flip_cap = words;
+    job->bytes += words * sizeof(uint32_t);
+  }
+  d.flips = job->flip_buf;
+}
+
 // Start a round: checks, round-start copies (for the joint's replays) and the
 // host bookkeeping; *t0 = attempts each chain made before this round.  With
 // allow_record the round's levels are recorded when it is small enough (the
@@ -434,9 +477,11 @@ int round_prepare(mc_job* job, int64_t n_sweeps, uint64_t* t0, bool allow_record
   if (job->trace_on)
     if (int rc = ensure_trace(job, n_sweeps)) return rc;
   int K = 0, C = 0;
-  round_segments(job->L, job->p, n_sweeps, job->seg_samples, &K, &C);
+  const bool flips = allow_record && flip_record_words(job->L, job->p, n_sweeps, job->rec_max) > 0;
+  round_segments(job->L, job->p, n_sweeps, job->seg_samples > 0 || !flips ? job->seg_samples : kFlipSegmentSamples, &K, &C);
   if (int rc = ensure_segments(job, K)) return rc;
   if (int rc = ensure_record(job, M, allow_record)) return rc;
+  ensure_flips(job, n_sweeps, allow_record);
   DevJob& d = job->d;
   d.ck_K = K;
   d.ck_C = C;
@@ -465,6 +510,7 @@ int attempts_prepare(mc_job* job, int64_t n, uint64_t* t0) {
   if (n < 1 || n >= (int64_t(1) << 34)) return fail(MC_EINVAL, "n_attempts=%lld", static_cast<long long>(n));
   DevJob& d = job->d;
   d.rec = nullptr;   // (their levels go to plv)
+  d.flips = nullptr;
   const long long entries = static_cast<long long>(job->p) * n;
   job->attempts_recorded = entries <= job->plv_max;
   if (job->attempts_recorded && static_cast<size_t>(entries) > job->plv_cap) {
@@ -1150,6 +1196,7 @@ static int mc_autotune_impl(mc_job* job, int64_t probe_sweeps, int use_cache, in
     d.trace = nullptr;
     d.ckpt = nullptr;  // probes write no checkpoints
     d.rec = nullptr;   // nor records
+    d.flips = nullptr;
     for (const auto& s : cands) {
       float ms = 0.f;
       for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {  // first run warms up
@@ -1275,6 +1322,7 @@ static int mc_batch_autotune_impl(mc_job** jobs, int n_jobs, int64_t probe_sweep
     d[i].trace = nullptr;
     d[i].ckpt = nullptr;   // probes write no checkpoints
     d[i].rec = nullptr;
+    d[i].flips = nullptr;
   }
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
@@ -1374,13 +1422,14 @@ uint64_t mc_job_device_bytes(int L, int n_chains, int64_t sweeps) {
   uint64_t b = lat * 4 * 2 + p * 4 * 2 + np1 * 8 + 5 * np1 * 4 + np1 * 8 * 3 + p * 8 + p * 4 + p * np1 * 4 +
                p * 8 + p * 4 + p * 4 + p * 4 + p * 20 + np1 + p * 4 + np1 * 4 + p * 8 + mcgpu::kStatCount * 8;
   int K = 0, C = 0;
-  round_segments(L, n_chains, sweeps, 0, &K, &C);
+  const size_t flip_words = flip_record_words(L, n_chains, sweeps, mcgpu::default_record_max(L));
+  round_segments(L, n_chains, sweeps, flip_words ? kFlipSegmentSamples : 0, &K, &C);
   (void)lw;
   const uint64_t samples = p * static_cast<uint64_t>(sweeps) * N;   // record of the round, if small
   const uint64_t rec = samples <= static_cast<uint64_t>(mcgpu::default_record_max(L))
                            ? static_cast<uint64_t>(mcgpu::rec_entries(n_chains, sweeps * static_cast<int64_t>(N))) * 2
                            : 0;
-  return b + static_cast<uint64_t>(K) * bytes_per_segment(L, n_chains) + rec;
+  return b + static_cast<uint64_t>(K) * bytes_per_segment(L, n_chains) + rec + 4ull * flip_words;
 }
 
 int mc_sync(mc_job* job) {

@@ -20,8 +20,19 @@ static_assert(kRecGroupStride == 4 * kRecTile, "record layout: generation and jo
 // rows rotate through the register array so that every index is static) or
 // in shared memory (any L; per-thread column with a stride of the number of
 // lanes that hold chains, so that a warp's accesses hit distinct banks).
+// FLIPS sweeps append each word's flips to the chain's flip record (flip; on
+// the lanes with keep set).
+struct FlipStream {
+  uint32_t* flip = nullptr;
+  bool keep = false;
+  __device__ __forceinline__ void put(uint32_t before, uint32_t after) {
+    if (keep) __stcs(flip, before ^ after);
+    ++flip;
+  }
+};
+
 template <int L>
-struct RegRunner {
+struct RegRunner : FlipStream {
   static constexpr int WD = 1;
   uint32_t R[L];
   __device__ __forceinline__ void load(const uint32_t* __restrict__ g) {
@@ -41,7 +52,7 @@ struct RegRunner {
 #pragma unroll
     for (int y = 0; y < L; ++y) R[y] = g[y * stride];
   }
-  template <bool EARLY, int GL = 1, class Hook>
+  template <bool EARLY, int GL = 1, bool FLIPS = false, class Hook>
   __device__ __forceinline__ void sweep(int& m, Prefetch& pf, const uint32_t* __restrict__ T, int np1,
                                         uint32_t chain, uint32_t k0, uint32_t k1, Hook& hk) {
 #pragma unroll 1
@@ -50,6 +61,7 @@ struct RegRunner {
       const uint32_t up[1] = {R[L - 1]};
       const uint32_t dn[1] = {R[1]};
       sweep_row<1, GL>(cur, up, dn, L, m, T, np1, pf, chain, k0, k1, hk);
+      if constexpr (FLIPS) put(R[0], cur[0]);
 #pragma unroll
       for (int i = 0; i < L - 1; ++i) R[i] = R[i + 1];
       R[L - 1] = cur[0];
@@ -62,7 +74,7 @@ struct RegRunner {
 
 // SL > 0 fixes L at compile time (no per-site guards); SL == 0 reads L at run time.
 template <int WD_, int SL = 0>
-struct SmemRunner {
+struct SmemRunner : FlipStream {
   static constexpr int WD = WD_;
   uint32_t* lat;  // this chain's column
   int stride, Lrt;
@@ -83,7 +95,7 @@ struct SmemRunner {
     const int L = len();
     for (int i = 0; i < L * WD; ++i) lat[i * stride] = g[i * gstride];
   }
-  template <bool EARLY, int GL = 1, class Hook>
+  template <bool EARLY, int GL = 1, bool FLIPS = false, class Hook>
   __device__ __forceinline__ void sweep(int& m, Prefetch& pf, const uint32_t* __restrict__ T, int np1,
                                         uint32_t chain, uint32_t k0, uint32_t k1, Hook& hk) {
     const int L = len();
@@ -97,7 +109,16 @@ struct SmemRunner {
         up[w] = lat[(ym * WD + w) * stride];
         dn[w] = lat[(yp * WD + w) * stride];
       }
+      uint32_t old[FLIPS ? WD : 1];
+      if constexpr (FLIPS) {
+#pragma unroll
+        for (int w = 0; w < WD; ++w) old[w] = cur[w];
+      }
       sweep_row<WD, GL>(cur, up, dn, L, m, T, np1, pf, chain, k0, k1, hk);
+      if constexpr (FLIPS) {
+#pragma unroll
+        for (int w = 0; w < WD; ++w) put(old[w], cur[w]);
+      }
 #pragma unroll
       for (int w = 0; w < WD; ++w) lat[(y * WD + w) * stride] = cur[w];
       if constexpr (EARLY) {
@@ -117,7 +138,7 @@ struct SmemRunner {
 // share an SM.  The lanes of a lane group store the same words.  Generation
 // only (the joint's replays restore checkpoints into shared memory).
 template <int WD_, int SL>
-struct GlobRunner {
+struct GlobRunner : FlipStream {
   static_assert(SL >= 4, "compile-time L");
   static constexpr int WD = WD_;
   uint32_t* lat;  // this chain's L rows of WD words
@@ -129,7 +150,7 @@ struct GlobRunner {
   __device__ __forceinline__ void save_strided(uint32_t* __restrict__ g, size_t gstride) const {
     for (int i = 0; i < SL * WD; ++i) g[i * gstride] = lat[i];
   }
-  template <bool EARLY, int GL = 1, class Hook>
+  template <bool EARLY, int GL = 1, bool FLIPS = false, class Hook>
   __device__ __forceinline__ void sweep(int& m, Prefetch& pf, const uint32_t* __restrict__ T, int np1,
                                         uint32_t chain, uint32_t k0, uint32_t k1, Hook& hk) {
     constexpr int L = SL;
@@ -144,7 +165,16 @@ struct GlobRunner {
     }
 #pragma unroll 1
     for (int y = 0; y < L; ++y) {
+      uint32_t old[FLIPS ? WD : 1];
+      if constexpr (FLIPS) {
+#pragma unroll
+        for (int w = 0; w < WD; ++w) old[w] = cur[w];
+      }
       sweep_row<WD, GL>(cur, up, dn, L, m, T, np1, pf, chain, k0, k1, hk);
+      if constexpr (FLIPS) {
+#pragma unroll
+        for (int w = 0; w < WD; ++w) put(old[w], cur[w]);
+      }
 #pragma unroll
       for (int w = 0; w < WD; ++w) {
         lat[y * WD + w] = cur[w];
@@ -247,7 +277,9 @@ struct RunnerFactorySmem {
 // lane group share one chain -- same lattice column, same uniforms (split
 // between them, see philox_fill) -- and only the group's first lane writes
 // counts, checkpoints, trace and the final state.
-template <class Factory, bool TSMEM, int GL = 1, bool REC = false>
+// KEEP: what the round keeps for the joint (kKeepNone: lattice checkpoints only).
+enum Keep : int { kKeepNone = 0, kKeepLevels = 1, kKeepFlips = 2 };
+template <class Factory, bool TSMEM, int GL = 1, int KEEP = kKeepNone>
 __device__ __forceinline__ void gen_body(const DevJob& j, const int cpw, const uint64_t t0, const int64_t S,
                                          const int64_t flushF, const int do_trace, const int block) {
   const SmemPlan sp = smem_plan(j.L, Factory::kPlacement, cpw, blockDim.x >> 5, TSMEM, true);
@@ -259,6 +291,7 @@ __device__ __forceinline__ void gen_body(const DevJob& j, const int cpw, const u
   Prefetch pf;
   // (one lane a chain: every lane counts; a compile-time 1 keeps the
   // reduction's operand an immediate)
+  constexpr bool REC = KEEP == kKeepLevels;
   GenHook<decltype(run)::WD == 1 ? 32 : 8, REC> hk;
   hk.init(b.hist, GL == 1 ? 1u : (b.owner ? 1u : 0u), j.np1);
   const bool writer = GL == 1 ? b.active : b.owner;
@@ -268,6 +301,10 @@ __device__ __forceinline__ void gen_body(const DevJob& j, const int cpw, const u
     // drop the writer test), only the writer stores
     hk.rec = j.rec + rec_index(b.active ? b.chain : 0, 0, S * j.N);
     hk.rec_on = writer;
+  }
+  if constexpr (KEEP == kKeepFlips) {
+    run.flip = j.flips + static_cast<size_t>(b.active ? b.chain : 0) * flip_words(j.L, S);
+    run.keep = writer;
   }
   if (b.active) {
     run.load(j.spins + static_cast<size_t>(b.chain) * j.L * j.wd);
@@ -291,7 +328,7 @@ __device__ __forceinline__ void gen_body(const DevJob& j, const int cpw, const u
         j.ckm[static_cast<size_t>(seg) * j.p + b.chain] = m;
       }
       if constexpr (GL > 1) __syncwarp(amask);
-      run.template sweep<false, GL>(m, pf, b.T, j.np1, static_cast<uint32_t>(b.chain), j.key0, j.key1, hk);
+      run.template sweep<false, GL, KEEP == kKeepFlips>(m, pf, b.T, j.np1, static_cast<uint32_t>(b.chain), j.key0, j.key1, hk);
       if (do_trace && writer) j.trace[s * j.p + b.chain] = 4 * m - 2 * j.N;
       if constexpr (GL > 1) __syncwarp(amask);
     }
@@ -328,10 +365,10 @@ __device__ __forceinline__ void gen_body(const DevJob& j, const int cpw, const u
   }
 }
 
-template <class Factory, bool TSMEM, int GL = 1, bool REC = false>
+template <class Factory, bool TSMEM, int GL = 1, int KEEP = kKeepNone>
 __global__ void __launch_bounds__(128) gen_kernel(const DevJob j, const int cpw, const uint64_t t0,
                                                   const int64_t S, const int64_t flushF, const int do_trace) {
-  gen_body<Factory, TSMEM, GL, REC>(j, cpw, t0, S, flushF, do_trace, blockIdx.x);
+  gen_body<Factory, TSMEM, GL, KEEP>(j, cpw, t0, S, flushF, do_trace, blockIdx.x);
 }
 
 // ------------------------------------------------------------------ joint: replays
@@ -740,10 +777,12 @@ inline cudaError_t launch_gen_t(const DevJob& j, const LaunchShape& s, uint64_t 
   const size_t bytes = plan_bytes(j.L, s, TS, true);
   // lattice in shared memory with at most 8 chains a warp: lane groups of 4
   // (groups of 8 for at most 4 chains measured slower at L = 48, 64 and 128)
-  const bool rec = j.rec != nullptr;
-  auto kern = rec ? gen_kernel<F, TS, 1, true> : gen_kernel<F, TS, 1, false>;
+  auto kern = j.rec ? gen_kernel<F, TS, 1, kKeepLevels>
+                    : (j.flips ? gen_kernel<F, TS, 1, kKeepFlips> : gen_kernel<F, TS, 1, kKeepNone>);
   if constexpr (F::kPlacement != kPlaceReg)
-    if (s.cpw <= 8) kern = rec ? gen_kernel<F, TS, 4, true> : gen_kernel<F, TS, 4, false>;
+    if (s.cpw <= 8)
+      kern = j.rec ? gen_kernel<F, TS, 4, kKeepLevels>
+                   : (j.flips ? gen_kernel<F, TS, 4, kKeepFlips> : gen_kernel<F, TS, 4, kKeepNone>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
   if (e != cudaSuccess) return e;
   const int per_block = s.cpw * s.wpb;

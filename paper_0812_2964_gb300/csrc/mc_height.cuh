@@ -110,6 +110,16 @@ __device__ __forceinline__ void height_store_max(Height* p, const Height& mine) 
   }
 }
 
+// Whether a sample may pass u / 2^32 < 2^x, x within the filter's slack of
+// exact: 1 + u / 2^32 rounded down to 23 bits, against 1 + 2^x and the
+// rounding (a NaN passes).
+__device__ __forceinline__ bool height_filter(float x, uint32_t u) {
+  float e;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x));
+  const float u1 = __uint_as_float(__funnelshift_r(u, 0x7Fu, 9));
+  return !(u1 >= e + 1.0000005f);
+}
+
 // Hook of the pass over a segment's samples.  wl[m] = (W[m] - Wref) / ln 2 as
 // a float; a sample can be among the best two only if u / 2^32 <
 // 2^(wl[m] - bl), bl below the second-best v found so far by more than the
@@ -122,6 +132,8 @@ struct HeightHook {
   uint32_t chain, r, k0, k1;
   uint32_t uj[32];
   Height h;
+  int mq[4];            // the current group of four samples: levels (times 4),
+  bool any;             // whether one of them passed the filter
   bool done;            // never set: the whole segment is read
   __device__ __forceinline__ void begin() {
     h = height_none();
@@ -132,27 +144,45 @@ struct HeightHook {
     joint_fill(uj, nb, k, r, chain, k0, k1);
     k += nb;
   }
+  // (one branch and one copy of the bookkeeping per four samples: unrolled a
+  // word at a time, a copy a sample overran the instruction cache)
   __device__ __forceinline__ void sample(int m4, int b) {
     const float w = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(wl) + m4);
-    float e;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(w - bl));
-    // 1 + u / 2^32 rounded down to 23 bits, against 1 + e and the rounding
-    const float u1 = __uint_as_float(__funnelshift_r(uj[b], 0x7Fu, 9));
-    if (!(u1 >= e + 1.0000005f)) {
-      const float v = uj[b] ? w + height_draw(uj[b]) : __int_as_float(0x7F800000);
-      if (v > h.second) {
-        const bool top = v > h.best;
-        h.second = top ? h.best : v;
-        if (top) {
-          h.best = v;
-          h.m = static_cast<uint32_t>(m4) >> 2;
-          h.u = uj[b];
+    const bool pass = height_filter(w - bl, uj[b]);
+    mq[b & 3] = m4;
+    any = (b & 3) == 0 ? pass : (any || pass);
+    if ((b & 3) == 3 && any) {
+#pragma unroll 1
+      for (int q = 0; q < 4; ++q) {
+        const int mm = q == 0 ? mq[0] : (q == 1 ? mq[1] : (q == 2 ? mq[2] : mq[3]));
+        const uint32_t u = q == 0 ? uj[b - 3] : (q == 1 ? uj[b - 2] : (q == 2 ? uj[b - 1] : uj[b]));
+        const float wq = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(wl) + mm);
+        const float v = u ? wq + height_draw(u) : __int_as_float(0x7F800000);
+        if (v > h.second) {
+          const bool top = v > h.best;
+          h.second = top ? h.best : v;
+          if (top) {
+            h.best = v;
+            h.m = static_cast<uint32_t>(mm) >> 2;
+            h.u = u;
+          }
         }
-        bl = fmaxf(bl, h.second - slack);
       }
+      bl = fmaxf(bl, h.second - slack);
     }
   }
 };
+
+// The chains whose samples kept_count_kernel counts, into work2 (one block;
+// work2 and its counter are free once nothing is searched any more).
+__device__ __forceinline__ void kept_list_counted(const DevJob& j) {
+  const bool kept = j.stats[kStatCountKept] != 0;
+  for (int i = threadIdx.x; i < j.p; i += blockDim.x) {
+    const int64_t k = j.k[i];
+    if (kept ? k > 0 : k != 1)
+      j.work2[atomicAdd(reinterpret_cast<unsigned long long*>(&j.stats[kStatNoHit]), 1ull)] = i;
+  }
+}
 
 // Whether the chain whose entry is h keeps samples for an input level of
 // weight wx: 1 yes, 0 no, 2 undecided.

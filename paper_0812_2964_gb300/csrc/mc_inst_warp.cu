@@ -1,21 +1,20 @@
 // Instantiation unit: generation with one chain per warp, rows of up to 32, 64 and 128 sites, L read at run time.
-#include "mc_chain_kernels.cuh"
 #include "mc_warp_chain.cuh"
 
 namespace mcgpu {
 
-template <class Rows, bool TSMEM, bool REC>
+template <class Rows, bool TSMEM, int KEEP>
 __global__ void __launch_bounds__(32 * kWarpChainBlock, 1)
     warp_gen_kernel(const DevJob j, const uint64_t t0, const int64_t S, const int64_t flushF, const int do_trace) {
-  warp_gen_body<Rows, TSMEM, REC>(j, t0, S, flushF, do_trace, blockIdx.x);
+  warp_gen_body<Rows, TSMEM, KEEP>(j, t0, S, flushF, do_trace, blockIdx.x);
 }
 
 template <class Rows>
 static cudaError_t launch_rows(const DevJob& j, int warps, bool ts, uint64_t t0, int64_t S, bool trace,
                                cudaStream_t st) {
-  const bool rec = j.rec != nullptr;
-  auto kern = ts ? (rec ? warp_gen_kernel<Rows, true, true> : warp_gen_kernel<Rows, true, false>)
-                 : (rec ? warp_gen_kernel<Rows, false, true> : warp_gen_kernel<Rows, false, false>);
+  auto kern = ts ? warp_gen_kernel<Rows, true, kKeepNone> : warp_gen_kernel<Rows, false, kKeepNone>;
+  if (j.rec) kern = ts ? warp_gen_kernel<Rows, true, kKeepLevels> : warp_gen_kernel<Rows, false, kKeepLevels>;
+  else if (j.flips) kern = ts ? warp_gen_kernel<Rows, true, kKeepFlips> : warp_gen_kernel<Rows, false, kKeepFlips>;
   const size_t bytes = 4ull * warp_plan(j.L, warps, ts).total;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
   if (e != cudaSuccess) return e;

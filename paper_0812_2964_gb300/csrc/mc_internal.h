@@ -67,7 +67,23 @@ struct DevJob {
   uint16_t* rec;       // level after each attempt of the current whole-sweep round, when the
                        // round is small enough to record (nullable; layout: rec_index): the
                        // joint reads it instead of replaying the chains
+  uint32_t* flips;     // accepted flips of the current whole-sweep round, a bit a sample, when it is too
+                       // large for `rec` but not for this (nullable; layout: flip_words): with the
+                       // segments' lattices the joint rebuilds every sample's level from them
 };
+
+// Flip record layout: chain c's lattice words in the order they are swept,
+// one 32-bit mask each (bit b: site b of the word flipped), from word
+// c * flip_words(L, S) on -- word (s L + y) wd + w for word w of row y in
+// sweep s -- padded to whole 128-byte lines.
+__host__ __device__ inline int64_t flip_words(int L, int64_t S) {
+  return (S * L * ((L + 31) / 32) + 31) / 32 * 32;
+}
+// whole-sweep rounds of more than kRecordMax samples, up to this many, keep
+// their flips (at most 8 GiB): iterations with chains that reject, measured
+// at 1.7e10 samples, L = 32 173 -> 52 ms and L = 64 253 -> 124 ms against
+// replaying from checkpoints
+constexpr long long kFlipMax = 1ll << 36;
 
 // Round record layout: chains in tiles of 32; inside a tile, each group of
 // four consecutive samples of the 32 chains lies side by side, so that a warp
@@ -211,6 +227,8 @@ MC_CHAIN_UNIT(chain_kernels_smem_L128);
 cudaError_t chain_kernels_warp(const DevJob& j, uint64_t t0, int64_t S, bool trace, cudaStream_t st);
 // the joint of a recorded round (any L): kernels without lattices or table
 cudaError_t chain_kernels_record(const DevJob& j, int64_t S, uint32_t r, cudaStream_t st);
+// the joint of a round that kept its flips
+cudaError_t chain_kernels_flips(const DevJob& j, int64_t S, uint32_t r, cudaStream_t st);
 
 // launch shape chosen by default for (L, p)
 LaunchShape default_shape(int L, int p, int num_sms);

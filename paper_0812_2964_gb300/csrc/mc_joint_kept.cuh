@@ -76,7 +76,7 @@ struct SourceRec {
 
 // ------------------------------------------------------------------ hooks
 // The exact test of one sample (off the main path: one call per candidate).
-__device__ __noinline__ bool joint_test(const double* __restrict__ W, int m, double wx, uint32_t u) {
+static __device__ __noinline__ bool joint_test(const double* __restrict__ W, int m, double wx, uint32_t u) {
   return u <= threshold_det(__dsub_rn(W[m], wx));
 }
 
@@ -91,21 +91,28 @@ struct TestHook {
   int64_t k, kw, found;
   uint32_t chain, r, k0, k1;
   uint32_t uj[32];
+  int mq[4];
+  bool any;
   bool done;
   __device__ __forceinline__ void word(int nb) {
     joint_fill(uj, nb, k, r, chain, k0, k1);
     kw = k;
     k += nb;
   }
-  __device__ __forceinline__ void sample(int m4, int b) {
+  __device__ __forceinline__ void sample(int m4, int b) {   // (by fours, as in HeightHook)
     const float w = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(wl) + m4);
-    float e;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(w - bl));
-    const float u1 = __uint_as_float(__funnelshift_r(uj[b], 0x7Fu, 9));   // 1 + u / 2^32, rounded down
-    if (!(u1 >= e + 1.0000005f)) {
-      if (!done && joint_test(W, m4 >> 2, wx, uj[b])) {
-        found = kw + b + 1;
-        done = true;
+    const bool pass = height_filter(w - bl, uj[b]);
+    mq[b & 3] = m4;
+    any = (b & 3) == 0 ? pass : (any || pass);
+    if ((b & 3) == 3 && any) {
+#pragma unroll 1
+      for (int q = 0; q < 4 && !done; ++q) {
+        const int mm = q == 0 ? mq[0] : (q == 1 ? mq[1] : (q == 2 ? mq[2] : mq[3]));
+        const uint32_t u = q == 0 ? uj[b - 3] : (q == 1 ? uj[b - 2] : (q == 2 ? uj[b - 1] : uj[b]));
+        if (joint_test(W, mm >> 2, wx, u)) {
+          found = kw + (b - 3 + q) + 1;
+          done = true;
+        }
       }
     }
   }
@@ -312,24 +319,27 @@ __global__ void __launch_bounds__(128) kept_height_kernel(const DevJob j, const 
 
 // The samples to count into dpre: the kept ones where they are fewer than
 // the discarded ones (kStatCountKept), else the discarded ones (the samples
-// before k_i, the whole chain if nothing is kept).  Every (segment, chain)
-// pair, dealt out in turn, segment-major; a block counts at most its share
-// of the round (below 2^32: the rounds kept hold at most 2^36 samples, and a
-// grid is smaller than the chip only when there are few items).
+// before k_i, the whole chain if nothing is kept), of the chains listed in
+// work2.  Every (segment, chain) pair, dealt out in turn, segment-major; a
+// block counts at most its share of the round (below 2^32: the rounds kept
+// hold at most 2^36 samples, and a grid is smaller than the chip only when
+// there are few items).
 template <class Src>
 __global__ void __launch_bounds__(128) kept_count_kernel(const DevJob j, const int cpw, const int64_t S) {
+  const int nchains = static_cast<int>(j.stats[kStatNoHit]);
+  const long long items = static_cast<long long>(nchains) * j.ck_K;
+  const int slots = (blockDim.x >> 5) * cpw;
+  if (static_cast<long long>(blockIdx.x) * slots >= items) return;
   const SmemPlan sp = smem_plan(j.L, Src::kPlacement, cpw, blockDim.x >> 5, false, true);
   BlockCtx b = block_setup<false>(j, sp, cpw, 0, true);
   __syncthreads();
-  const long long items = static_cast<long long>(j.p) * j.ck_K;
-  const int slots = (blockDim.x >> 5) * cpw;
   const int64_t M = S * j.N;
   const bool kept = j.stats[kStatCountKept] != 0;
   for (long long base = static_cast<long long>(blockIdx.x) * slots; base < items;
        base += static_cast<long long>(gridDim.x) * slots) {
     const long long item = base + b.slot;
     if (b.lane < cpw && item < items) {
-      const int i = static_cast<int>(item % j.p), seg = static_cast<int>(item / j.p);
+      const int i = j.work2[item % nchains], seg = static_cast<int>(item / nchains);
       const int64_t k = j.k[i];
       int64_t lo = kept ? (k > 0 ? k - 1 : M) : 0;                // 0-based, [lo, hi)
       int64_t hi = kept ? M : (k > 0 ? k - 1 : M);
@@ -429,7 +439,10 @@ __global__ void __launch_bounds__(128) kept_resolve_kernel(const DevJob j, const
     j.stats[kStatCountKept] = 2ull * s_sum < static_cast<unsigned long long>(j.p) * static_cast<unsigned long long>(M);
     j.stats[kStatMismatch] += mism_total;
     j.stats[kStatPasses] += passes;
+    j.stats[kStatNoHit] = 0;
   }
+  __syncthreads();
+  kept_list_counted(j);
   if (searched) atomicAdd(reinterpret_cast<unsigned long long*>(&j.stats[kStatSearched]),
                           static_cast<unsigned long long>(searched));
 }
@@ -459,7 +472,8 @@ inline cudaError_t launch_join_kept(const DevJob& j, const LaunchShape& s, int64
     return static_cast<unsigned>(std::max<long long>(1, std::min<long long>(blocks_for(n, per_block), resident)));
   };
   const long long res_q = resident_blocks(kq, threads, bytes);
-  const bool exact = static_cast<long long>(j.p) * S * j.N <= j.scan_max_samples;
+  // (the default limit is the replays': a kept round of any size takes the exact path)
+  const bool exact = static_cast<long long>(j.p) * S * j.N <= j.scan_max_samples || j.scan_max_samples == kScanMaxSamples;
   auto search = [&](int listed, int first) -> cudaError_t {
     kq<<<grid(j.p, res_q), threads, bytes, st>>>(j, s.cpw, S, r, listed, 0, first);
     launches_add(1);

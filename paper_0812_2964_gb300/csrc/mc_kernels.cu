@@ -799,6 +799,8 @@ __global__ void __launch_bounds__(1024) kept_mark_kernel(const DevJob j, const i
       j.stats[kStatCountKept] = 2ull * s_kept < static_cast<unsigned long long>(j.p) * static_cast<unsigned long long>(M);
     }
   }
+  __syncthreads();
+  if ((flags & kMarkFinal) && s_count == 0) kept_list_counted(j);
 }
 
 // Scratch of the scan in tj (its rows are rebuilt for the chains searched
@@ -1464,7 +1466,7 @@ cudaError_t join_tj_list(const DevJob& j, cudaStream_t st) {
 }
 
 cudaError_t join_finalize(const DevJob& j, int64_t S, cudaStream_t st) {
-  launch_finalize(j, S * j.N, j.rec != nullptr, st);
+  launch_finalize(j, S * j.N, j.rec || j.flips, st);
   launches_add(1);
   return cudaGetLastError();
 }
@@ -1516,6 +1518,7 @@ cudaError_t k_join(const DevJob& j, const LaunchShape& s, uint64_t t0, int64_t S
     return cudaGetLastError();
   }
   if (j.rec) return chain_kernels_record(j, S, r, st);   // levels recorded: no replays
+  if (j.flips) return chain_kernels_flips(j, S, r, st);   // nor where the flips are
   return dispatch(j, join_shape(j.L, s), false, t0, S, false, r, st);
 }
 

@@ -37,8 +37,7 @@
 #pragma once
 #include <algorithm>
 
-#include "mc_chain.cuh"
-#include "mc_internal.h"
+#include "mc_chain_kernels.cuh"
 
 namespace mcgpu {
 
@@ -326,6 +325,7 @@ struct WarpLane {
   uint32_t t_last;                // last byte offset of the table (global memory)
   uint32_t hist_a;                // shared address of the level counters
   uint16_t* rec;                  // this lane's place in the round record
+  uint32_t* flip;                 // the chain's place in the flip record
 };
 
 // Uniforms: a ring in shared memory, filled 128 at a time, a Philox block a lane.
@@ -379,7 +379,7 @@ struct Words {
   __device__ __forceinline__ static void store(uint32_t* g, size_t stride, const uint32_t* lat, int L, int lane) {
     for (int i = lane; i < L * WD; i += 32) g[i * stride] = lat[i];
   }
-  template <bool TSMEM, bool REC>
+  template <bool TSMEM, int KEEP>
   __device__ __forceinline__ void row(uint32_t* lat, int y, int& m, WarpLane& w, WarpRing& ring) {
     const int L = w.L, lw = L - 32 * (WD - 1);   // sites of the last word
     const int yp = y + 1 == L ? 0 : y + 1;
@@ -435,11 +435,15 @@ struct Words {
       }
       m = m1;
       if (valid) warp_count(w.hist_a + 4u * lvl);
-      if constexpr (REC) {
+      if constexpr (KEEP == kKeepLevels) {
         if (valid) st_record1(w.rec, lvl);
         w.rec += (nb >> 2) * kRecGroupStride;
       }
       cur[v] = c ^ F;
+      if constexpr (KEEP == kKeepFlips) {
+        if (w.lane == 0) __stcs(w.flip, F);
+        ++w.flip;
+      }
     }
     // (every lane stores the same words)
 #pragma unroll
@@ -500,7 +504,7 @@ struct TwoWords {
       g[i * stride] = bits_spread(lat[at] >> sh) | (bits_spread(lat[at + 1] >> sh) << 1);
     }
   }
-  template <bool TSMEM, bool REC>
+  template <bool TSMEM, int KEEP>
   __device__ __forceinline__ void row(uint32_t* lat, int y, int& m, WarpLane& w, WarpRing& ring) {
     const int L = w.L;
     const int yp = y + 1 == L ? 0 : y + 1;
@@ -575,12 +579,21 @@ struct TwoWords {
         warp_count(w.hist_a + static_cast<uint32_t>(m4 + mid));
         warp_count(w.hist_a + 4u * lo);
       }
-      if constexpr (REC) {
+      if constexpr (KEEP == kKeepLevels) {
         if (valid) st_record2(w.rec, (static_cast<uint32_t>(m4 + mid) >> 2) | (static_cast<uint32_t>(lo) << 16));
         w.rec += (nb >> 2) * kRecGroupStride;
       }
       E[v] = e ^ FE;
       O[v] = o ^ FO;
+      if constexpr (KEEP == kKeepFlips) {
+        // the window's two words in site order: lane l votes for sites l and 32 + l
+        const uint32_t half = (w.lane & 1) ? FO : FE;
+        const uint32_t w0 = __ballot_sync(0xFFFFFFFFu, (half >> (w.lane >> 1)) & 1u);
+        const uint32_t w1 = __ballot_sync(0xFFFFFFFFu, (half >> (16 + (w.lane >> 1))) & 1u);
+        const int nw = lastv ? (nl + 31) / 32 : 2;
+        if (w.lane < nw) __stcs(w.flip + w.lane, w.lane ? w1 : w0);
+        w.flip += nw;
+      }
     }
     // (every lane stores the same words)
 #pragma unroll
@@ -594,7 +607,7 @@ struct TwoWords {
 };
 
 // One block of the round: its warps' chains, first + warp.
-template <class Rows, bool TSMEM, bool REC>
+template <class Rows, bool TSMEM, int KEEP>
 __device__ __forceinline__ void warp_gen_body(const DevJob& j, const uint64_t t0, const int64_t S,
                                               const int64_t flushF, const int do_trace, const int block) {
   extern __shared__ __align__(16) uint32_t smem[];
@@ -630,7 +643,9 @@ __device__ __forceinline__ void warp_gen_body(const DevJob& j, const uint64_t t0
   w.t_last = static_cast<uint32_t>(4 * (5 * np1 - 1));
   w.hist_a = static_cast<uint32_t>(__cvta_generic_to_shared(hist));
   w.rec = nullptr;
-  if constexpr (REC) {
+  w.flip = nullptr;
+  if constexpr (KEEP == kKeepFlips) w.flip = j.flips + static_cast<size_t>(active ? chain : 0) * flip_words(L, S);
+  if constexpr (KEEP == kKeepLevels) {
     const int k = Rows::kSitesPerLane * lane;   // this lane's first sample in a window
     w.rec = j.rec + rec_index(active ? chain : 0, 0, S * j.N) + (k >> 2) * kRecGroupStride + (k & 3);
   }
@@ -654,7 +669,7 @@ __device__ __forceinline__ void warp_gen_body(const DevJob& j, const uint64_t t0
       rows.begin(lat, L);
 #pragma unroll 1
       for (int y = 0; y < L; ++y) {
-        rows.template row<TSMEM, REC>(lat, y, m, w, ring);
+        rows.template row<TSMEM, KEEP>(lat, y, m, w, ring);
         __syncwarp();
       }
       if (do_trace && lane == 0) j.trace[s * j.p + chain] = 4 * m - 2 * j.N;
