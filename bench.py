@@ -283,7 +283,7 @@ def batch_record(torch, mc, S, steps, warmup, tune, rank=0):
     """The uneven batch run three ways on the same chains; kept samples/s of each."""
     from paper_0812_2964_gb300.workloads import BATCH_GROUPS
 
-    modes = {0: "one launch per job", 1: "one fused launch", 2: "fused launch, CUDA graph"}
+    modes = {0: "one launch per job", 1: "one fused launch", 2: "one branch per job, CUDA graph"}
     out = {}
     t_wall = time.perf_counter()
     for mode in (0, 1, 2):
@@ -532,7 +532,7 @@ def run_gpu(args):
 def run_batch(args):
     """The uneven batch: L in {16, 24, 32, 48, 64} with 8192/4096/4096/2048/1024
     chains, every weight iteration run three ways -- one generation launch per
-    job, one fused launch, the fused loop as a CUDA graph -- on the same
+    job, one fused launch, every job a branch of one CUDA graph -- on the same
     chains (identical results); value = the graph form's kept samples/s."""
     import torch
 

@@ -122,8 +122,8 @@ int mc_run_attempts(mc_job *job, int64_t n_attempts);
  * keep their accepted flips instead, one bit a sample (at most 8 GiB; where
  * that cannot be allocated the round is replayed), from which the joint
  * rebuilds the levels; any other limit turns that off too.
- * Rounds of mc_batch_run are not recorded.  MC_ESTATE while a round is
- * pending. */
+ * Fused rounds of mc_batch_run are not recorded.  MC_ESTATE while a round
+ * is pending. */
 int mc_set_round_record(mc_job *job, int64_t max_samples);
 
 /* Largest record (p * n_attempts entries, int32 each) that a round of
@@ -297,15 +297,19 @@ int mc_set_launch_shape(mc_job *job, int placement, int chains_per_warp, int war
  * size has a fused form (L = 8, 16, 24, 32 in registers; 24, 32, 48, 64 in
  * shared memory; up to 8 jobs), each with the shape mc_batch_autotune chose
  * for it, or by rule (full warps; shared memory at L = 24, 32, 48, 64), the
- * others keep their own launch; mode 2: mode 1 with the whole loop captured
- * once as a CUDA graph and launched.  The
+ * others keep their own launch; mode 2: every job's whole loop a branch of
+ * one CUDA graph, captured once and launched (up to 8 jobs): the jobs run
+ * side by side, each with its own launches -- the shape it was given, else
+ * one chosen for the set of jobs -- and a job's joint beside the others'
+ * generation.  Rounds of modes 0 and 2 keep their samples for the joint as
+ * mc_run_sweeps's do, where there is memory for it.  The
  * chains, and so every result, are the same in all modes.  Synchronises.
  * No round may be pending on any job.  The paper has no counterpart: a
  * scheduling form of running independent weight estimations together. */
 int mc_batch_run(mc_job **jobs, int n_jobs, int iterations, int64_t n_sweeps, int mode);
 
-/* Launch shapes of the jobs in a fused batch launch (mc_batch_run modes 1
- * and 2), by measurement: each job's candidate shapes (lattice in registers
+/* Launch shapes of the jobs in a fused batch launch (mc_batch_run mode 1),
+ * by measurement: each job's candidate shapes (lattice in registers
  * or shared memory where the fused kernel has that form, 4..32 chains per
  * warp, lane groups of 4 for shared-memory lattices above L = 32 with at
  * most 8 chains a warp) are tried in turn, longest chains first, each trial

@@ -75,6 +75,7 @@ struct mc_job {
   bool trace_valid = false;
   size_t trace_cap = 0;  // int32 elements
   LaunchShape shape;
+  bool shape_chosen = false;     // by mc_set_launch_shape or mc_autotune (else the default rule's)
   LaunchShape bshape{};          // shape in a fused batch launch (mc_batch_autotune)
   bool bshape_valid = false;
   int64_t seg_samples = 0;  // target samples per checkpoint segment (0: default)
@@ -310,6 +311,7 @@ int mc_set_launch_shape(mc_job* job, int placement, int cpw, int wpb) {
   if (!mcgpu::shape_supported(job->L, s))
     return fail(MC_EINVAL, "launch shape (%d, %d, %d) not supported for L=%d", placement, cpw, wpb, job->L);
   job->shape = s;
+  job->shape_chosen = true;
   return MC_OK;
 }
 
@@ -464,6 +466,25 @@ void ensure_flips(mc_job* job, int64_t n_sweeps, bool allow) {
   d.flips = job->flip_buf;
 }
 
+// Segments of the job's round: finer ones by default where it keeps its flips.
+void choose_segments(const mc_job* job, int64_t n_sweeps, bool allow_record, int* K, int* C) {
+  const bool flips = allow_record && flip_record_words(job->L, job->p, n_sweeps, job->rec_max) > 0;
+  round_segments(job->L, job->p, n_sweeps, job->seg_samples > 0 || !flips ? job->seg_samples : kFlipSegmentSamples, K, C);
+}
+
+// The round's record (of levels or flips) for a batch, where there is memory
+// for it; false: the round is replayed.
+bool ensure_kept(mc_job* job, int64_t n_sweeps) {
+  if (n_sweeps < 1 || n_sweeps > (int64_t(1) << 34) / job->N) return false;   // (round_prepare refuses it)
+  if (ensure_record(job, n_sweeps * job->N, true) != MC_OK) {
+    cudaGetLastError();   // (not an error of the call)
+    g_err.clear();
+    return false;
+  }
+  ensure_flips(job, n_sweeps, true);
+  return job->d.rec || job->d.flips;
+}
+
 // Start a round: checks, round-start copies (for the joint's replays) and the
 // host bookkeeping; *t0 = attempts each chain made before this round.  With
 // allow_record the round's levels are recorded when it is small enough (the
@@ -477,8 +498,7 @@ int round_prepare(mc_job* job, int64_t n_sweeps, uint64_t* t0, bool allow_record
   if (job->trace_on)
     if (int rc = ensure_trace(job, n_sweeps)) return rc;
   int K = 0, C = 0;
-  const bool flips = allow_record && flip_record_words(job->L, job->p, n_sweeps, job->rec_max) > 0;
-  round_segments(job->L, job->p, n_sweeps, job->seg_samples > 0 || !flips ? job->seg_samples : kFlipSegmentSamples, &K, &C);
+  choose_segments(job, n_sweeps, allow_record, &K, &C);
   if (int rc = ensure_segments(job, K)) return rc;
   if (int rc = ensure_record(job, M, allow_record)) return rc;
   ensure_flips(job, n_sweeps, allow_record);
@@ -657,12 +677,16 @@ static LaunchShape batch_rule_shape(int L, int p) {
   return s;
 }
 
-// `iterations` weight iterations of several independent jobs, everything on
-// the first job's stream: per iteration every job runs one round of n_sweeps
+// `iterations` weight iterations of several independent jobs, ordered on the
+// first job's stream: per iteration every job runs one round of n_sweeps
 // sweeps, is joined and updates its weight.  mode 0: one generation launch
 // per job; 1: one fused generation launch for all jobs that fit it (others
-// keep their own launch); 2: as 1, with the whole loop captured once as a
-// CUDA graph and launched.  Results are identical in all modes.
+// keep their own launch); 2: every job's whole loop a branch of one CUDA
+// graph -- the jobs do not wait for one another's rounds, a job's joint runs
+// beside others' generation, and each keeps its own launch shape and its
+// rounds' samples for the joint, which the fused kernel does not (the uneven
+// batch at 200 sweeps, two iterations: 40 ms, 116 as a graph of fused launches).
+// Results are identical in all modes.
 static int mc_batch_run_impl(mc_job** jobs, int n_jobs, int iterations, int64_t n_sweeps, int mode) {
   if (!jobs || n_jobs < 1) return fail(MC_EINVAL, "no jobs");
   if (mode < 0 || mode > 2) return fail(MC_EINVAL, "mode=%d: 0 per-job, 1 fused, 2 fused + graph", mode);
@@ -678,6 +702,7 @@ static int mc_batch_run_impl(mc_job** jobs, int n_jobs, int iterations, int64_t 
       if (jobs[k] == jobs[i]) return fail(MC_EINVAL, "job %d listed twice", i);
   }
   cudaStream_t st = jobs[0]->stream;
+  const bool branches = mode == 2;
   std::vector<cudaStream_t> saved(n_jobs);
   for (int i = 0; i < n_jobs; ++i) {
     MC_CUDA(cudaStreamSynchronize(jobs[i]->stream), "batch start");
@@ -687,11 +712,17 @@ static int mc_batch_run_impl(mc_job** jobs, int n_jobs, int iterations, int64_t 
   // shapes for the fused launch: the autotuned ones (mc_batch_autotune), else
   // the rule of batch_rule_shape
   std::vector<LaunchShape> bshape(n_jobs);
-  std::vector<char> fused(n_jobs, 0);
-  for (int i = 0; i < n_jobs && mode > 0; ++i) {
+  std::vector<char> fused(n_jobs, 0), keeps(n_jobs, 0);
+  for (int i = 0; i < n_jobs && mode == 1; ++i) {
     const LaunchShape s = jobs[i]->bshape_valid ? jobs[i]->bshape : batch_rule_shape(jobs[i]->L, jobs[i]->p);
     bshape[i] = s;
     fused[i] = mcgpu::batch_supported(jobs[i]->L, s) ? 1 : 0;
+  }
+  std::vector<LaunchShape> branch_shape(n_jobs);
+  {
+    std::vector<int> Ls(n_jobs), ps(n_jobs);
+    for (int i = 0; i < n_jobs; ++i) Ls[i] = jobs[i]->L, ps[i] = jobs[i]->p;
+    mcgpu::batch_branch_shapes(n_jobs, Ls.data(), ps.data(), jobs[0]->num_sms, branch_shape.data());
   }
   // fused blocks in order of decreasing work per chain (N), so that the
   // longest chains start first
@@ -702,14 +733,27 @@ static int mc_batch_run_impl(mc_job** jobs, int n_jobs, int iterations, int64_t 
   for (int i = 0; i < n_jobs && rc == MC_OK; ++i) {  // no allocation inside a capture
     if (jobs[i]->trace_on) rc = ensure_trace(jobs[i], n_sweeps);
     int K = 0, C = 0;
-    round_segments(jobs[i]->L, jobs[i]->p, n_sweeps, jobs[i]->seg_samples, &K, &C);
+    choose_segments(jobs[i], n_sweeps, !fused[i], &K, &C);
     if (rc == MC_OK) rc = ensure_segments(jobs[i], K);
+    keeps[i] = !fused[i] && rc == MC_OK && ensure_kept(jobs[i], n_sweeps);
   }
+  std::vector<cudaEvent_t> done(n_jobs, nullptr);
+  cudaEvent_t fork = nullptr;
   bool capturing = false;
-  if (rc == MC_OK && mode == 2) {
-    const cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
+  if (rc == MC_OK && branches) {
+    cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+    for (int i = 0; i < n_jobs && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&done[i], cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) rc = cuda_fail(e, "graph capture");
     else capturing = true;
+    // every job continues on its own stream from here
+    if (rc == MC_OK) e = cudaEventRecord(fork, st);
+    for (int i = 0; i < n_jobs && rc == MC_OK && e == cudaSuccess; ++i)
+      if (jobs[i]->own_stream != st) {
+        e = cudaStreamWaitEvent(jobs[i]->own_stream, fork, 0);
+        jobs[i]->stream = jobs[i]->own_stream;
+      }
+    if (rc == MC_OK && e != cudaSuccess) rc = cuda_fail(e, "graph capture");
   }
   for (int it = 0; it < iterations && rc == MC_OK; ++it) {
     mcgpu::BatchParams P;
@@ -719,9 +763,9 @@ static int mc_batch_run_impl(mc_job** jobs, int n_jobs, int iterations, int64_t 
     for (int oi = 0; oi < n_jobs && rc == MC_OK; ++oi) {
       const int i = order[oi];
       uint64_t t0 = 0;
-      if ((rc = round_prepare(jobs[i], n_sweeps, &t0, false))) break;
+      if ((rc = round_prepare(jobs[i], n_sweeps, &t0, keeps[i] != 0))) break;
       cudaError_t e = cudaSuccess;
-      if (mode > 0 && fused[i]) {
+      if (fused[i]) {
         mcgpu::BatchItem& item = P.items[P.n++];
         size_t b = 0;
         int nb = 0;
@@ -730,7 +774,8 @@ static int mc_batch_run_impl(mc_job** jobs, int n_jobs, int iterations, int64_t 
         blocks += nb;
         smem = std::max(smem, b);
       } else {
-        e = mcgpu::k_generate(jobs[i]->d, jobs[i]->shape, t0, n_sweeps, jobs[i]->trace_on, st);
+        const LaunchShape s = branches && !jobs[i]->shape_chosen ? branch_shape[i] : jobs[i]->shape;
+        e = mcgpu::k_generate(jobs[i]->d, s, t0, n_sweeps, jobs[i]->trace_on, jobs[i]->stream);
       }
       if (e != cudaSuccess) rc = cuda_fail(e, "generation");
     }
@@ -741,8 +786,8 @@ static int mc_batch_run_impl(mc_job** jobs, int n_jobs, int iterations, int64_t 
     for (int i = 0; i < n_jobs && rc == MC_OK; ++i) {
       mc_job* j = jobs[i];
       const int64_t M = j->last_S * j->N;
-      cudaError_t e = mcgpu::k_join(j->d, j->shape, j->t - static_cast<uint64_t>(M), j->last_S, j->r, false, st);
-      if (e == cudaSuccess) e = mcgpu::k_update_weights(j->d, st);
+      cudaError_t e = mcgpu::k_join(j->d, j->shape, j->t - static_cast<uint64_t>(M), j->last_S, j->r, false, j->stream);
+      if (e == cudaSuccess) e = mcgpu::k_update_weights(j->d, j->stream);
       if (e != cudaSuccess) {
         rc = cuda_fail(e, "joint / weight update");
         break;
@@ -753,7 +798,15 @@ static int mc_batch_run_impl(mc_job** jobs, int n_jobs, int iterations, int64_t 
   }
   if (capturing) {
     cudaGraph_t g = nullptr;
-    const cudaError_t e = cudaStreamEndCapture(st, &g);
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < n_jobs; ++i)   // (also after a failure: a capture ends with its branches joined)
+      if (jobs[i]->stream != st) {
+        const cudaError_t e1 = cudaEventRecord(done[i], jobs[i]->stream);
+        const cudaError_t e2 = e1 == cudaSuccess ? cudaStreamWaitEvent(st, done[i], 0) : e1;
+        if (e == cudaSuccess) e = e2;
+      }
+    const cudaError_t e_end = cudaStreamEndCapture(st, &g);
+    if (e == cudaSuccess) e = e_end;
     if (rc == MC_OK && e != cudaSuccess) rc = cuda_fail(e, "graph capture");
     if (rc == MC_OK) {
       cudaGraphExec_t ge = nullptr;
@@ -765,6 +818,9 @@ static int mc_batch_run_impl(mc_job** jobs, int n_jobs, int iterations, int64_t 
     }
     if (g) cudaGraphDestroy(g);
   }
+  for (cudaEvent_t ev : done)
+    if (ev) cudaEventDestroy(ev);
+  if (fork) cudaEventDestroy(fork);
   for (int i = 0; i < n_jobs; ++i) jobs[i]->stream = saved[i];
   if (rc != MC_OK) {
     for (int i = 0; i < n_jobs; ++i) jobs[i]->pending = false;
@@ -1153,6 +1209,7 @@ static int mc_autotune_impl(mc_job* job, int64_t probe_sweeps, int use_cache, in
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
       job->shape = it->second;
+      job->shape_chosen = true;
       if (placement) *placement = job->shape.placement;
       if (cpw) *cpw = job->shape.cpw;
       if (wpb) *wpb = job->shape.wpb;
@@ -1223,6 +1280,7 @@ static int mc_autotune_impl(mc_job* job, int64_t probe_sweeps, int use_cache, in
   if (sh) cudaFree(sh);
   if (e != cudaSuccess) return cuda_fail(e, "autotune");
   job->shape = best;
+  job->shape_chosen = true;
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tune_cache[key] = best;

@@ -234,6 +234,8 @@ cudaError_t chain_kernels_flips(const DevJob& j, int64_t S, uint32_t r, cudaStre
 LaunchShape default_shape(int L, int p, int num_sms);
 // the shape of a job that runs beside others
 LaunchShape dense_shape(int L, int p, int num_sms);
+// shapes of n jobs that run side by side to the end of the longest
+void batch_branch_shapes(int n, const int* L, const int* p, int num_sms, LaunchShape* out);
 bool shape_supported(int L, const LaunchShape& s);
 size_t gen_smem_bytes(int L, const LaunchShape& s, bool* table_in_smem);
 

@@ -1271,8 +1271,12 @@ LaunchShape default_shape(int L, int p, int num_sms) {
 // shape has it there: the time of a round is set by the latency of one chain,
 // which a fuller warp does not change (measured: within 5 % for L <= 64 and
 // 128), so the job takes the same time on far fewer warps.
+static LaunchShape full_lane_shape(int L, int p, int num_sms);
 LaunchShape dense_shape(int L, int p, int num_sms) {
-  if (warp_chain_better(L, p, num_sms)) return default_shape(L, p, num_sms);
+  return warp_chain_better(L, p, num_sms) ? default_shape(L, p, num_sms) : full_lane_shape(L, p, num_sms);
+}
+
+static LaunchShape full_lane_shape(int L, int p, int num_sms) {
   LaunchShape def = lane_shape(L, p, num_sms);
   // full warps at L = 100, 128 keep their lattices in global memory: a block
   // of 128 chains then needs only the histogram's shared memory, so blocks
@@ -1286,6 +1290,43 @@ LaunchShape dense_shape(int L, int p, int num_sms) {
       if (shape_supported(L, s) && (!ts || table_fits(L, s, true))) return s;
     }
   return def;
+}
+
+// Time of one attempt of every chain, ns, by launch form: one chain a lane
+// (a chain's serial path, whatever the chains), one a warp (the larger of a
+// window's latency and the schedulers' share of instructions).  Measured alone
+// on 152 SMs; used to compare forms, not to predict times.
+static double lane_ns(int L) {
+  if (L <= 32) return L == 24 || L == 32 ? 29.0 : 33.0;
+  if (L == 48) return 43.0;
+  if (L == 64) return 29.0;
+  if (L == 96) return 45.0;
+  if (L == 128) return 60.0;
+  return 75.0;
+}
+static double warp_ns(int L, int p, int num_sms) {
+  const int wd = (L + 31) / 32, loads = (p + 4 * num_sms - 1) / (4 * num_sms);
+  const double windows = warp_pairs(L, p, num_sms) ? 440.0 * ((L + 63) / 64) : 290.0 * wd;   // ns a row
+  return std::max(windows / L, 2.9 * loads * 32.0 * wd / L);
+}
+
+// Jobs side by side take as long as the longest, so only the jobs that would
+// be longer than that one's faster form with a chain a lane take a warp a
+// chain: a full warp of lanes issues a third of the instructions a site.
+// (The uneven batch, young weights: 90 us a sweep with L = 48 and 64 a warp a
+// chain and the others a lane, 120 with L = 32 a warp too, 166 with all a lane;
+// L = 48 and 64 alone 48 each, together 76: the schedulers are then full.)
+void batch_branch_shapes(int n, const int* L, const int* p, int num_sms, LaunchShape* out) {
+  double longest = 0.0;
+  for (int i = 0; i < n; ++i)
+    longest = std::max(longest, L[i] * L[i] * std::min(lane_ns(L[i]), warp_ns(L[i], p[i], num_sms)));
+  for (int i = 0; i < n; ++i) {
+    if (L[i] * L[i] * lane_ns(L[i]) <= longest || !warp_chain_better(L[i], p[i], num_sms)) {
+      out[i] = full_lane_shape(L[i], p[i], num_sms);
+    } else {
+      out[i] = LaunchShape{kPlaceSmem, 1, 4};
+    }
+  }
 }
 
 // The joint's replay kernels take their own launch shape (their work items
