@@ -1065,11 +1065,11 @@ int mc_thermo(mc_job* job, const double* betas, int n_beta, double* out) {
   for (int b = 0; b < n_beta; ++b)
     if (!(betas[b] > 0.0) || !(betas[b] < 1e300)) return fail(MC_EINVAL, "beta[%d] must be positive and finite", b);
   void* dev = nullptr;
-  MC_CUDA(raw_alloc(job, &dev, sizeof(double) * 5 * n_beta), "thermo buffer");
+  MC_CUDA(raw_alloc(job, &dev, sizeof(double) * mcgpu::thermo_doubles(job->N + 1, n_beta)), "thermo buffer");
   double* db = static_cast<double*>(dev);
   double* dout = db + n_beta;
   cudaError_t e = cudaMemcpyAsync(db, betas, sizeof(double) * n_beta, cudaMemcpyHostToDevice, job->stream);
-  if (e == cudaSuccess) e = mcgpu::k_thermo(job->d, db, n_beta, dout, job->stream);
+  if (e == cudaSuccess) e = mcgpu::k_thermo(job->d, n_beta, db, job->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(out, dout, sizeof(double) * 4 * n_beta, cudaMemcpyDeviceToHost, job->stream);
   raw_free(job, dev);

@@ -166,8 +166,10 @@ cudaError_t k_update_weights(const DevJob& j, cudaStream_t st);
 cudaError_t k_generate_attempts(const DevJob& j, uint64_t t0, int64_t n, bool record, cudaStream_t st);
 cudaError_t k_join_attempts(const DevJob& j, uint64_t t0, int64_t M, uint32_t r, bool naive, bool recorded,
                             cudaStream_t st);
-// E, C, F, S at n inverse temperatures (device arrays betas[n], out[n][4])
-cudaError_t k_thermo(const DevJob& j, const double* betas, int n, double* out, cudaStream_t st);
+// E, C, F, S at n inverse temperatures: device buffer buf of thermo_doubles()
+// doubles, betas in buf[0..n), results in buf[n + 4b ..]
+size_t thermo_doubles(int np1, int n);
+cudaError_t k_thermo(const DevJob& j, int n, double* buf, cudaStream_t st);
 cudaError_t k_generate(const DevJob& j, const LaunchShape& s, uint64_t t0, int64_t S,
                        bool trace, cudaStream_t st);
 cudaError_t k_join(const DevJob& j, const LaunchShape& s, uint64_t t0, int64_t S, uint32_t r,
