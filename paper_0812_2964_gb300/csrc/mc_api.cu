@@ -546,11 +546,13 @@ int attempts_prepare(mc_job* job, int64_t n, uint64_t* t0) {
     job->plv_cap = static_cast<size_t>(entries);
     job->bytes += job->plv_cap * sizeof(int32_t);
   }
-  const size_t lat = static_cast<size_t>(job->p) * job->L * job->wd;
-  MC_CUDA(cudaMemcpyAsync(d.spins0, d.spins, lat * sizeof(uint32_t), cudaMemcpyDeviceToDevice, job->stream),
-          "round-start copy");
-  MC_CUDA(cudaMemcpyAsync(d.m0, d.m, job->p * sizeof(int32_t), cudaMemcpyDeviceToDevice, job->stream),
-          "round-start copy");
+  if (!job->attempts_recorded) {   // for the serial joint's replays
+    const size_t lat = static_cast<size_t>(job->p) * job->L * job->wd;
+    MC_CUDA(cudaMemcpyAsync(d.spins0, d.spins, lat * sizeof(uint32_t), cudaMemcpyDeviceToDevice, job->stream),
+            "round-start copy");
+    MC_CUDA(cudaMemcpyAsync(d.m0, d.m, job->p * sizeof(int32_t), cudaMemcpyDeviceToDevice, job->stream),
+            "round-start copy");
+  }
   *t0 = job->t;
   job->t += static_cast<uint64_t>(n);
   job->last_S = n / job->N;

@@ -1164,33 +1164,162 @@ __device__ __forceinline__ int attempt_one(const DevJob& j, uint32_t* lat, int m
   return m;
 }
 
-__global__ void attempts_kernel(const DevJob j, const uint64_t t0, const int64_t n, int32_t* __restrict__ rec) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= j.p) return;
-  uint32_t* lat = j.spins + static_cast<size_t>(c) * j.L * j.wd;
+// A warp of chains a block: the lattices in shared memory (a column a chain),
+// the threshold table beside them where it fits, the site counted up.  What
+// bounds it is one chain's serial path, two shared-memory loads and the
+// arithmetic around them: 100 attempts of 32 chains at L = 20 take 8 us (60
+// with the lattice and the table in global memory and the site divided out
+// of the attempt's number).
+template <bool TSMEM>
+__global__ void __launch_bounds__(32) attempts_kernel(const DevJob j, const uint64_t t0, const int64_t n,
+                                                      int32_t* __restrict__ rec) {
+  extern __shared__ __align__(16) uint32_t smem[];
+  const int lane = threadIdx.x, c = blockIdx.x * 32 + lane, L = j.L, wd = j.wd, np1 = j.np1;
+  const uint32_t* T = j.T;
+  uint32_t* lat = smem + (TSMEM ? ((5 * np1 + 3) & ~3) : 0) + lane;   // word q of the chain at lat[32 q]
+  if (TSMEM) {
+    for (int i = lane; i < 5 * np1; i += 32) smem[i] = j.T[i];
+    T = smem;
+  }
+  const bool active = c < j.p;
+  uint32_t* g = j.spins + static_cast<size_t>(active ? c : 0) * L * wd;
+  if (active)
+    for (int q = 0; q < L * wd; ++q) lat[32 * q] = g[q];
+  __syncwarp();
+  if (!active) return;
   int m = j.m[c];
+  const int site = static_cast<int>(t0 % static_cast<uint64_t>(j.N));
+  int x = site % L, y = site / L;
   uint4 r = make_uint4(0u, 0u, 0u, 0u);
-  uint64_t blk = ~0ull;
   int32_t* lv = rec ? rec + static_cast<size_t>(c) * n : nullptr;
+  const auto spin = [&](int xx, int yy) { return (lat[32 * (yy * wd + (xx >> 5))] >> (xx & 31)) & 1u; };
   for (int64_t k = 0; k < n; ++k) {
-    m = attempt_one(j, lat, m, t0 + static_cast<uint64_t>(k), static_cast<uint32_t>(c), r, blk);
+    const uint64_t t = t0 + static_cast<uint64_t>(k);
+    if ((t & 3u) == 0u || k == 0)
+      r = philox4x32_10(make_uint4(static_cast<uint32_t>(t >> 2), static_cast<uint32_t>(t >> 34),
+                                   static_cast<uint32_t>(c), kTagFlip),
+                        j.key0, j.key1);
+    const uint32_t sv = spin(x, y);
+    const int a = (spin(x ? x - 1 : L - 1, y) == sv) + (spin(x + 1 == L ? 0 : x + 1, y) == sv) +
+                  (spin(x, y ? y - 1 : L - 1) == sv) + (spin(x, y + 1 == L ? 0 : y + 1) == sv);
+    const uint32_t u = uint4_word(r, static_cast<uint32_t>(t & 3u));
+    if (u <= T[a * np1 + m]) {
+      lat[32 * (y * wd + (x >> 5))] ^= 1u << (x & 31);
+      m += a - 2;
+    }
     atomicAdd(&j.hgen[m], 1ull);
     if (lv) lv[k] = m;
+    if (++x == L) {
+      x = 0;
+      if (++y == L) y = 0;
+    }
   }
+  for (int q = 0; q < L * wd; ++q) g[q] = lat[32 * q];
   j.m[c] = m;
 }
 
-// The joint of such a round (Sec. 2 steps 3-5) from the recorded levels:
-// the chains in joint order, one at a time (the input of each is the level
-// passed on by those before it), the samples of a chain tested in parallel
-// -- sample k passes iff its joint uniform Philox((k-1)>>2, r, chain, 1)
-// word (k-1)&3 is at most thr(W[m_k] - W[x]) -- in blocks of the block's
-// threads, stopping at the first block with a pass; k_i is the smallest
-// passing k.  The samples before it (all M when none passes) go to dpre.
+// The joint of such a round (Sec. 2 steps 3-5) from the recorded levels, by
+// heights (mc_height.cuh): every chain's height from all its samples, a warp
+// a chain; the scan that settles every input; then, a warp a chain again, the
+// first passing sample of the chains that keep some and the count of the
+// discarded ones.  A round of 32 chains of 100 samples takes 15 us (63 one
+// chain after another).  An input the heights cannot settle leaves the whole
+// round to partial_joint_kernel.
+__global__ void __launch_bounds__(128) partial_height_kernel(const DevJob j, const int64_t M, const uint32_t r) {
+  const float* wl = level_weights(j);
+  const int lane = threadIdx.x & 31, nwarps = (gridDim.x * blockDim.x) >> 5;
+  for (int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < j.p; q += nwarps) {
+    const int c = j.perm[q];
+    const int32_t* lv = j.plv + static_cast<size_t>(c) * M;
+    Height h = height_none();
+    for (int64_t k = lane; k < M; k += 32) {
+      const uint4 v = philox4x32_10(make_uint4(static_cast<uint32_t>(k >> 2), r, static_cast<uint32_t>(c), kTagJoint),
+                                    j.key0, j.key1);
+      Height one = height_none();
+      one.m = static_cast<uint32_t>(lv[k]);
+      one.u = uint4_word(v, static_cast<uint32_t>(k & 3));
+      one.best = one.u ? wl[one.m] + height_draw(one.u) : CUDART_INF_F;
+      if (one.best == one.best) h = height_merge(h, one);   // (no number: passes no test)
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      Height b;
+      b.m = __shfl_xor_sync(0xFFFFFFFFu, h.m, o);
+      b.u = __shfl_xor_sync(0xFFFFFFFFu, h.u, o);
+      b.best = __shfl_xor_sync(0xFFFFFFFFu, h.best, o);
+      b.second = __shfl_xor_sync(0xFFFFFFFFu, h.second, o);
+      h = height_merge(h, b);
+    }
+    if (lane == 0) {
+      heights(j)[c] = h;
+      // the whole joint is the scan's: nothing known, from the first position on
+      j.k[c] = -1;
+      j.lastacc[q] = -1;
+      if (q == 0) {
+        j.stats[kStatPending] = j.p;
+        j.stats[kStatFirstPending] = 0;
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(128) partial_finish_kernel(const DevJob j, const int64_t M, const uint32_t r) {
+  if (j.stats[kStatScanned] < j.p) return;   // undecided somewhere: partial_joint_kernel
+  const int lane = threadIdx.x & 31, nwarps = (gridDim.x * blockDim.x) >> 5;
+  for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < j.p; c += nwarps) {
+    const int32_t* lv = j.plv + static_cast<size_t>(c) * M;
+    int64_t kf = j.k[c];   // 0 or 1 are final
+    __syncwarp();
+    if (kf < 0) {
+      const double wx = j.W[j.xused[c]];
+      for (int64_t base = 0; base < M; base += 32) {
+        const int64_t k = base + lane;
+        bool hit = false;
+        if (k < M) {
+          const uint4 v = philox4x32_10(
+              make_uint4(static_cast<uint32_t>(k >> 2), r, static_cast<uint32_t>(c), kTagJoint), j.key0, j.key1);
+          hit = uint4_word(v, static_cast<uint32_t>(k & 3)) <= threshold_det(__dsub_rn(j.W[lv[k]], wx));
+        }
+        const unsigned hits = __ballot_sync(0xFFFFFFFFu, hit);
+        if (hits) {
+          kf = base + __ffs(hits);
+          break;
+        }
+      }
+      if (lane == 0) j.k[c] = kf;
+    }
+    const int64_t nd = kf > 0 ? kf - 1 : M;   // discarded samples
+    for (int64_t k = lane; k < nd; k += 32) atomicAdd(&j.dpre[lv[k]], 1ull);
+  }
+}
+
+// The same joint by the serial rule: the chains in joint order, one at a time
+// (the input of each is the level passed on by those before it), the samples
+// of a chain tested in parallel -- sample k passes iff its joint uniform
+// Philox((k-1)>>2, r, chain, 1) word (k-1)&3 is at most thr(W[m_k] - W[x]) --
+// in blocks of the block's threads, stopping at the first block with a pass;
+// k_i is the smallest passing k.  The samples before it (all M when none
+// passes) go to dpre.  Where the heights have settled the round it only
+// fixes the carry.
 __global__ void __launch_bounds__(1024) partial_joint_kernel(const DevJob j, const int64_t M, const uint32_t r) {
   __shared__ unsigned long long s_k;
   __shared__ int s_carry, s_valid;
   const int t = threadIdx.x, nt = blockDim.x;
+  if (j.stats[kStatScanned] == j.p) {
+    if (t == 0) s_carry = -1;
+    __syncthreads();
+    for (int q = t; q < j.p; q += nt)
+      if (j.k[j.perm[q]] > 0) atomicMax(&s_carry, q);
+    __syncthreads();
+    if (t == 0) {
+      if (s_carry >= 0) {
+        j.stats[kStatCarry] = j.m[j.perm[s_carry]];
+        j.stats[kStatCarryValid] = 1;
+      }
+      j.stats[kStatSearched] = static_cast<long long>(j.p) * M;
+      j.stats[kStatScanned] = 0;
+    }
+    return;
+  }
   if (t == 0) {
     s_valid = static_cast<int>(j.stats[kStatCarryValid]);
     s_carry = static_cast<int>(j.stats[kStatCarry]);
@@ -1246,10 +1375,6 @@ __global__ void __launch_bounds__(1024) partial_joint_kernel(const DevJob j, con
   }
 }
 
-__global__ void clear_searched_kernel(const DevJob j) {
-  if (threadIdx.x == 0) j.stats[kStatSearched] = 0;
-}
-
 // The joint of such a round by the serial rule itself (Sec. 2 steps 3-5),
 // one thread: each chain, in joint order, is regenerated from its round
 // start until its first sample that passes the test against the level
@@ -1303,23 +1428,34 @@ __global__ void serial_joint_kernel(const DevJob j, const uint64_t t0, const int
 }
 
 cudaError_t k_generate_attempts(const DevJob& j, uint64_t t0, int64_t n, bool record, cudaStream_t st) {
-  attempts_kernel<<<blocks_for(j.p, 128), 128, 0, st>>>(j, t0, n, record ? j.plv : nullptr);
+  const size_t lat = 128ull * j.L * j.wd, table = 4ull * ((5 * j.np1 + 3) & ~3);
+  const bool ts = lat + table <= kMaxSmem;
+  auto kern = ts ? attempts_kernel<true> : attempts_kernel<false>;
+  const size_t bytes = lat + (ts ? table : 0);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  if (e != cudaSuccess) return e;
+  kern<<<blocks_for(j.p, 32), 32, bytes, st>>>(j, t0, n, record ? j.plv : nullptr);
   launches_add(1);
   return cudaGetLastError();
 }
 
 cudaError_t k_join_attempts(const DevJob& j, uint64_t t0, int64_t M, uint32_t r, bool naive, bool recorded,
                             cudaStream_t st) {
-  order_kernel<<<1, 1024, 0, st>>>(j);
-  if (naive) {
-    naive_kernel<<<blocks_for(j.p, 256), 256, 0, st>>>(j);
-  } else if (recorded) {
-    clear_searched_kernel<<<1, 32, 0, st>>>(j);
+  if (!naive && recorded) {
+    cudaError_t e = kept_prelude(j, st);
+    if (e != cudaSuccess) return e;
+    const unsigned warps = std::min(2432u, blocks_for(j.p, 4));
+    partial_height_kernel<<<warps, 128, 0, st>>>(j, M, r);
+    if ((e = kept_scan(j, st)) != cudaSuccess) return e;
+    partial_finish_kernel<<<warps, 128, 0, st>>>(j, M, r);
     partial_joint_kernel<<<1, 1024, 0, st>>>(j, M, r);
-    launches_add(1);
-  } else {
-    serial_joint_kernel<<<1, 32, 0, st>>>(j, t0, M, r);
+    launch_finalize(j, M, false, st);
+    launches_add(4);
+    return cudaGetLastError();
   }
+  order_kernel<<<1, 1024, 0, st>>>(j);
+  if (naive) naive_kernel<<<blocks_for(j.p, 256), 256, 0, st>>>(j);
+  else serial_joint_kernel<<<1, 32, 0, st>>>(j, t0, M, r);
   launch_finalize(j, M, false, st);
   launches_add(3);
   return cudaGetLastError();
