@@ -227,6 +227,17 @@ MC_CHAIN_UNIT(chain_kernels_smem_L128);
 #undef MC_CHAIN_UNIT
 // generation with one chain per warp (any L; shape kPlaceSmem with one chain a warp)
 cudaError_t chain_kernels_warp(const DevJob& j, uint64_t t0, int64_t S, bool trace, cudaStream_t st);
+#define MC_WARP_UNIT(name)                                                                                    \
+  cudaError_t name(const DevJob& j, int warps, bool ts, bool pairs, uint64_t t0, int64_t S, bool trace, \
+                   cudaStream_t st)
+MC_WARP_UNIT(chain_kernels_warp_1);
+MC_WARP_UNIT(chain_kernels_warp_2a);
+MC_WARP_UNIT(chain_kernels_warp_2b);
+MC_WARP_UNIT(chain_kernels_warp_3a);
+MC_WARP_UNIT(chain_kernels_warp_3b);
+MC_WARP_UNIT(chain_kernels_warp_4a);
+MC_WARP_UNIT(chain_kernels_warp_4b);
+#undef MC_WARP_UNIT
 // the joint of a recorded round (any L): kernels without lattices or table
 cudaError_t chain_kernels_record(const DevJob& j, int64_t S, uint32_t r, cudaStream_t st);
 // the joint of a round that kept its flips

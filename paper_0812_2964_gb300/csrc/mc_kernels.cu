@@ -1753,6 +1753,21 @@ cudaError_t join_finalize(const DevJob& j, int64_t S, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+cudaError_t chain_kernels_warp(const DevJob& j, uint64_t t0, int64_t S, bool trace, cudaStream_t st) {
+  int dev = 0, sms = 1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  int warps = 1;
+  bool ts = false;
+  warp_chain_shape(j.L, j.p, sms, &warps, &ts);
+  const bool pairs = warp_pairs(j.L, j.p, sms);
+  if (j.wd == 1) return chain_kernels_warp_1(j, warps, ts, pairs, t0, S, trace, st);
+  if (j.wd == 2) return (j.L <= 48 ? chain_kernels_warp_2a : chain_kernels_warp_2b)(j, warps, ts, pairs, t0, S, trace, st);
+  if (j.wd == 3) return (j.L <= 80 ? chain_kernels_warp_3a : chain_kernels_warp_3b)(j, warps, ts, pairs, t0, S, trace, st);
+  return (j.L <= 112 ? chain_kernels_warp_4a : chain_kernels_warp_4b)(j, warps, ts, pairs, t0, S, trace, st);
+}
+
 static cudaError_t dispatch(const DevJob& j, const LaunchShape& s, bool gen, uint64_t t0, int64_t S, bool trace,
                             uint32_t r, cudaStream_t st) {
   if (gen && s.placement == kPlaceSmem && s.cpw == 1) return chain_kernels_warp(j, t0, S, trace, st);

@@ -1,6 +1,7 @@
 // Generation with one chain per warp (Sec. 2 step 2): the sites of a window
 // of the row are resolved together: a lattice word, one site a lane (Words),
-// or 64 sites, two neighbouring ones a lane (TwoWords; warp_pairs).
+// 64 sites, two neighbouring ones a lane (TwoWords; warp_pairs), or several
+// rows of a small lattice (ShortRows).
 //
 // A chain's attempts are serial -- the level after each decides the next
 // one's threshold, and its flip the right neighbour's aligned count -- but
@@ -121,21 +122,24 @@ inline void warp_chain_shape(int L, int p, int num_sms, int* warps, bool* tsmem)
 // in chains per scheduler (p / (4 SMs)); up to 8 are resident.  Measured, ns a
 // site (one a warp / one a lane, rounds of 10 to 200 sweeps, grown weights,
 // 152 SMs):
-//   L = 8     35 / 37 at 300 chains (a row fills 8 of 32 lanes: left to the lanes)
-//   L = 16    19 / 33 at 600, 27 / 33 at 2048, 35 / 33 at 3000
-//   L = 20    16 / 33 at 1200, 25 / 33 at 3000
-//   L = 32    8.9 / 28 at 512 or fewer, 13 / 28 at 2048, 21 / 28 at 4096, 41 / 29 at 5500
+//   L = 8     16 / 37 at 608 or fewer, 25 / 37 at 2432, 33 / 37 at 3600
+//   L = 12    15 / 33 at 64, 24 / 33 at 2432, 28 / 35 at 3040, 46 / 33 at 4800
+//   L = 16    12 / 33 at 512, 18 / 33 at 2432, 31 / 33 at 4800
+//   L = 20    13 / 33 at 512, 27 / 33 at 3600, 35 / 33 at 4800
+//   L = 24    23 / 32 at 3600, 30 / 52 at 4800 (lane groups of 4)
+//   L = 32    8.0 / 28 at 512 or fewer, 12 / 28 at 2048, 19 / 28 at 4096, 41 / 29 at 5500
 //   L = 36    19 / 96 at 2048 (no lane kernel with L fixed at compile time)
-//   L = 64    8.7 / 26 at 1024, 19 / 29 at 4096, 33 / 42 at 5500, 43 / 42 at 8192
+//   L = 64    8.1 / 26 at 1024, 19 / 29 at 4096, 33 / 42 at 5500, 43 / 42 at 8192
 //   L = 76    39 / 80 at 6000, 50 / 80 at 9000
 //   L = 96    13 / 44 at 1280, 19 / 45 at 4096, 40 / 52 at 8192
-//   L = 100   9.0 / 53 at 32, 23 / 76 at 4096, 46 / 169 at 8000
-//   L = 128   9.6 / 53 at 1024, 20 / 64 at 4096, 59 / 69 at 6000, 88 / 75 at 8192
+//   L = 100   8.8 / 53 at 32, 21 / 76 at 4096, 46 / 169 at 8000
+//   L = 128   9.2 / 53 at 1024, 20 / 64 at 4096, 59 / 69 at 6000, 88 / 75 at 8192
 inline bool warp_chain_better(int L, int p, int num_sms) {
   int most = 8;                                               // one wave
-  if (L < 12) most = 0;
-  else if (L <= 16) most = 4;
-  else if (L <= 24) most = 6;
+  if (L < 8) most = 0;
+  else if (L == 8) most = 6;
+  else if (L == 12) most = 5;
+  else if (L == 20) most = 7;
   else if (L == 48 || L == 64 || L == 96) most = 12;          // two waves
   else if (L > 32 && L <= 100) most = 16;
   return p <= most * 4 * num_sms;
@@ -312,12 +316,72 @@ __device__ __forceinline__ int warp_fixed_point2(uint32_t& FE, uint32_t& FO, int
 }
 #undef MC_EVAL2
 #undef MC_EVAL_WRAP
+
+// One site a lane, several short rows a window: F also flips the sites above
+// (a row earlier) and, at the row's end, the site at its start, so the masks
+// are made from F each time.
+#define MC_EVALR(LOAD_)                                              \
+  "{\n\t"                                                            \
+  ".reg .pred p, q, v;\n\t"                                          \
+  ".reg .b32 fu, fr, el, s0, n1, x, a, b, c, at, t, fn;\n\t"         \
+  "setp.ne.u32 v, %16, 0;\n\t"                                       \
+  "EVAL:\n\t"                                                        \
+  "shl.b32 fu, %0, %8;\n\t"                                          \
+  "and.b32 fr, %0, %7;\n\t"                                          \
+  "shl.b32 fr, fr, %9;\n\t"                                          \
+  "shl.b32 el, %0, 1;\n\t"                                           \
+  "lop3.b32 el, el, %7, %6, 0x9A;\n\t"                               \
+  "lop3.b32 s0, %2, fu, fr, 0x96;\n\t"                               \
+  "xor.b32 fu, %3, fu;\n\t"                                          \
+  "xor.b32 fr, %5, fr;\n\t"                                          \
+  "lop3.b32 n1, fu, %4, fr, 0x17;\n\t"                               \
+  "and.b32 x, %0, %10;\n\t"                                          \
+  "and.b32 a, x, s0;\n\t"                                            \
+  "and.b32 b, x, el;\n\t"                                            \
+  "and.b32 c, x, n1;\n\t"                                            \
+  "popc.b32 a, a;\n\t"                                               \
+  "popc.b32 b, b;\n\t"                                               \
+  "popc.b32 c, c;\n\t"                                               \
+  "mov.b32 at, %12;\n\t"                                             \
+  "and.b32 t, s0, %11;\n\t"                                          \
+  "setp.ne.u32 q, t, 0;\n\t"                                         \
+  "@q add.s32 at, at, %13;\n\t"                                      \
+  "and.b32 t, el, %11;\n\t"                                          \
+  "setp.ne.u32 q, t, 0;\n\t"                                         \
+  "@q add.s32 at, at, %13;\n\t"                                      \
+  "and.b32 t, n1, %11;\n\t"                                          \
+  "setp.ne.u32 q, t, 0;\n\t"                                         \
+  "@q mad.lo.s32 at, %13, -2, at;\n\t"                               \
+  "add.s32 a, a, b;\n\t"                                             \
+  "mad.lo.s32 %1, c, -2, a;\n\t"                                     \
+  "mad.lo.s32 at, %1, %14, at;\n\t" LOAD_                            \
+  "setp.le.and.u32 p, %15, t, v;\n\t"                                \
+  "vote.sync.ballot.b32 fn, p, 0xffffffff;\n\t"                      \
+  "setp.ne.u32 q, fn, %0;\n\t"                                       \
+  "mov.b32 %0, fn;\n\t"                                              \
+  "@q bra.uni EVAL;\n\t"                                             \
+  "}"
+template <int L, uint32_t COL0, bool TSMEM>
+__device__ __forceinline__ int warp_fixed_point_rows(uint32_t& F, uint32_t e0, uint32_t eu, uint32_t ed, uint32_t er,
+                                                     uint32_t el, uint32_t before, uint32_t bit, int base, int r1, int scale, uint32_t u, bool valid,
+                                                     const uint32_t* __restrict__ T, uint32_t last) {
+  int d;
+#define MC_EVAL_ARGS                                                                                            \
+  : "+r"(F), "=&r"(d)                                                                                           \
+  : "r"(e0), "r"(eu), "r"(ed), "r"(er), "r"(el), "n"(COL0), "n"(L), "n"(L - 1), "r"(before), "r"(bit),          \
+    "r"(base), "r"(r1), "r"(scale), "r"(u), "r"(static_cast<uint32_t>(valid)), "l"(T), "r"(last)
+  if constexpr (TSMEM) asm volatile(MC_EVALR(MC_LOAD_SHARED("at", "t")) MC_EVAL_ARGS);
+  else asm volatile(MC_EVALR(MC_LOAD_GLOBAL("at", "t", "%17", "%18")) MC_EVAL_ARGS);
+#undef MC_EVAL_ARGS
+  return d;
+}
+#undef MC_EVALR
 #undef MC_LOAD_SHARED
 #undef MC_LOAD_GLOBAL
 
 // What every window needs of the block and the lane.
 struct WarpLane {
-  int L, lane;
+  int lane;
   uint32_t bit, lt, le, before;   // this lane, those before it, and it; `before` is everything for lane 0
   int scale;                      // 4; 0 for lane 0, whose sum is the window's
   int r1, r1z, row2;              // a table row in bytes; 0 for lane 0; row 2 at level 0
@@ -362,26 +426,28 @@ __device__ __forceinline__ void warp_count(uint32_t addr) {
 }
 
 // Rows of WD words, a window a word: lane l holds site l of the word.
-template <int WD>
+// (L at compile time: 10 % off a window.)
+template <int WD, int L>
 struct Words {
   static constexpr int kRowWords = WD, kSitesPerLane = 1;
+  static constexpr int lw = L - 32 * (WD - 1);   // sites of the last word
+  __device__ __forceinline__ static int step() { return 1; }
   uint32_t up[WD], cur[WD];
-  __device__ __forceinline__ void begin(const uint32_t* lat, int L) {
+  __device__ __forceinline__ void begin(const uint32_t* lat) {
 #pragma unroll
     for (int w = 0; w < WD; ++w) {
       up[w] = lat[(L - 1) * WD + w];
       cur[w] = lat[w];
     }
   }
-  __device__ __forceinline__ static void load(uint32_t* lat, const uint32_t* g, int L, int lane) {
+  __device__ __forceinline__ static void load(uint32_t* lat, const uint32_t* g, int lane) {
     for (int i = lane; i < L * WD; i += 32) lat[i] = g[i];
   }
-  __device__ __forceinline__ static void store(uint32_t* g, size_t stride, const uint32_t* lat, int L, int lane) {
+  __device__ __forceinline__ static void store(uint32_t* g, size_t stride, const uint32_t* lat, int lane) {
     for (int i = lane; i < L * WD; i += 32) g[i * stride] = lat[i];
   }
   template <bool TSMEM, int KEEP>
   __device__ __forceinline__ void row(uint32_t* lat, int y, int& m, WarpLane& w, WarpRing& ring) {
-    const int L = w.L, lw = L - 32 * (WD - 1);   // sites of the last word
     const int yp = y + 1 == L ? 0 : y + 1;
     uint32_t dn[WD];
 #pragma unroll
@@ -475,11 +541,13 @@ __device__ __forceinline__ uint32_t bits_spread(uint32_t x) {
 // two words (so that neighbours in the row are the other word, or its
 // neighbour bit).  Against 32 sites a window, one a lane: half the solves and
 // a third fewer evaluations a site (2.1 for 64 sites, 1.6 for 32).
-template <int NW>
+template <int NW, int L>
 struct TwoWords {
   static constexpr int kRowWords = 2 * NW, kSitesPerLane = 2;
+  static constexpr int wd = (L + 31) / 32, nl = L - 64 * (NW - 1), hl = nl / 2;   // sites and lanes of the last window
+  __device__ __forceinline__ static int step() { return 1; }
   uint32_t upE[NW], upO[NW], E[NW], O[NW];
-  __device__ __forceinline__ void begin(const uint32_t* lat, int L) {
+  __device__ __forceinline__ void begin(const uint32_t* lat) {
 #pragma unroll
     for (int v = 0; v < NW; ++v) {
       upE[v] = lat[(L - 1) * 2 * NW + 2 * v];
@@ -488,8 +556,7 @@ struct TwoWords {
       O[v] = lat[2 * v + 1];
     }
   }
-  __device__ __forceinline__ static void load(uint32_t* lat, const uint32_t* g, int L, int lane) {
-    const int wd = (L + 31) / 32;
+  __device__ __forceinline__ static void load(uint32_t* lat, const uint32_t* g, int lane) {
     for (int i = lane; i < L * NW; i += 32) {
       const int y = i / NW, v = i % NW;
       const uint32_t a = g[y * wd + 2 * v], b = 2 * v + 1 < wd ? g[y * wd + 2 * v + 1] : 0u;
@@ -497,8 +564,7 @@ struct TwoWords {
       lat[2 * i + 1] = bits_even(a >> 1) | (bits_even(b >> 1) << 16);
     }
   }
-  __device__ __forceinline__ static void store(uint32_t* g, size_t stride, const uint32_t* lat, int L, int lane) {
-    const int wd = (L + 31) / 32;
+  __device__ __forceinline__ static void store(uint32_t* g, size_t stride, const uint32_t* lat, int lane) {
     for (int i = lane; i < L * wd; i += 32) {
       const int y = i / wd, x = i % wd, at = 2 * (y * NW + x / 2), sh = 16 * (x & 1);
       g[i * stride] = bits_spread(lat[at] >> sh) | (bits_spread(lat[at + 1] >> sh) << 1);
@@ -506,9 +572,7 @@ struct TwoWords {
   }
   template <bool TSMEM, int KEEP>
   __device__ __forceinline__ void row(uint32_t* lat, int y, int& m, WarpLane& w, WarpRing& ring) {
-    const int L = w.L;
     const int yp = y + 1 == L ? 0 : y + 1;
-    const int nl = L - 64 * (NW - 1), hl = nl >> 1;   // sites and lanes of the last window
     uint32_t dnE[NW], dnO[NW];
 #pragma unroll
     for (int v = 0; v < NW; ++v) {
@@ -606,13 +670,88 @@ struct TwoWords {
   }
 };
 
+// Rows of 8, 12 or 16 sites, 32 / L of them a window (a row a window would
+// leave most lanes idle): lane l holds site l of the window in typewriter
+// order, the lattice copy a word a window.  The first mask is solved along
+// each row with every other site taken as flipped (levels and rows above
+// included); 1.2 to 1.6 evaluations follow for grown weights.
+template <int L>
+struct ShortRows {
+  static constexpr int kRowWords = 1, kSitesPerLane = 1;
+  static constexpr int R = 32 / L, nb = R * L, top = nb - L, kWindows = L / R;
+  static_assert(L % R == 0, "whole windows");
+  static constexpr uint32_t sites = nb == 32 ? 0xFFFFFFFFu : (1u << (nb & 31)) - 1u;
+  static constexpr uint32_t col0 = L == 8 ? 0x01010101u : (L == 12 ? 0x001001u : 0x00010001u);   // the rows' first sites
+  uint32_t prev;
+  __device__ __forceinline__ static int step() { return R; }
+  __device__ __forceinline__ void begin(const uint32_t* lat) { prev = lat[kWindows - 1]; }
+  __device__ __forceinline__ static void load(uint32_t* lat, const uint32_t* g, int lane) {
+    for (int v = lane; v < kWindows; v += 32) {
+      uint32_t x = 0u;
+      for (int q = 0; q < R; ++q) x |= g[v * R + q] << (q * L);
+      lat[v] = x;
+    }
+  }
+  __device__ __forceinline__ static void store(uint32_t* g, size_t stride, const uint32_t* lat, int lane) {
+    for (int y = lane; y < L; y += 32) g[y * stride] = (lat[y / R] >> ((y % R) * L)) & ((1u << L) - 1u);
+  }
+  template <bool TSMEM, int KEEP>
+  __device__ __forceinline__ void row(uint32_t* lat, int y, int& m, WarpLane& w, WarpRing& ring) {
+    const int v = y / R;
+    const uint32_t c = lat[v], next = lat[v + 1 == kWindows ? 0 : v + 1];
+    ring.need(nb, w.lane);
+    const uint32_t u = *reinterpret_cast<const uint32_t*>(ring.ring + ring.use_at);
+    ring.step(nb);
+    const bool valid = w.lane < nb;
+    // agreements with the neighbours, F's flips left out: the row above is the window's own but for its
+    // first row, the row below but for its last
+    const uint32_t up = (c << L) | (prev >> top), dn = (c >> L) | (next << top);
+    const uint32_t right = ((c >> 1) & ~(col0 << (L - 1))) | ((c & col0) << (L - 1));
+    const uint32_t left = ((c << 1) & ~col0) | ((c >> (L - 1)) & col0);
+    const uint32_t eu = ~(c ^ up), ed = ~(c ^ dn), er = ~(c ^ right), el = ~(c ^ left);
+    const uint32_t e0 = eu ^ ed ^ er;
+    const int base = 4 * m + w.row2;
+    // the first mask: everything flipped but each site's left neighbour, which is solved
+    constexpr uint32_t fr = (sites & col0) << (L - 1);
+    const uint32_t s1 = e0 ^ (sites << L) ^ fr, eu1 = eu ^ (sites << L), er1 = er ^ fr;
+    const uint32_t n1 = ~((eu1 & ed) | (er1 & (eu1 ^ ed))), el1 = el ^ ((sites << 1) & ~col0);
+    const uint32_t X = sites & w.before;
+    int at = base + w.scale * (__popc(X & s1) + __popc(X & el1) - 2 * __popc(X & n1));
+    if (s1 & w.bit) at += w.r1;
+    if (n1 & w.bit) at -= 2 * w.r1;
+    int at0 = at;   // left neighbour not flipped
+    if (el & w.bit) at0 += w.r1;
+    if (el1 & w.bit) at += w.r1;
+    const uint32_t t0 = warp_threshold<TSMEM>(w.T, at0, w.t_last);
+    const uint32_t t1 = warp_threshold<TSMEM>(w.T, at, w.t_last);
+    const uint32_t G0 = __ballot_sync(0xFFFFFFFFu, valid && u <= t0);
+    const uint32_t G1 = __ballot_sync(0xFFFFFFFFu, valid && u <= t1);
+    uint32_t F = warp_solve(G0, G1, w.le);
+    const int d = warp_fixed_point_rows<L, col0, TSMEM>(F, e0, eu, ed, er, el, w.before, w.bit, base, w.r1, w.scale,
+                                                        u, valid, w.T, w.t_last);
+    const int lvl = m + __shfl_sync(0xFFFFFFFFu, d, (w.lane + 1) & 31);
+    m += __shfl_sync(0xFFFFFFFFu, d, 0);
+    if (valid) warp_count(w.hist_a + 4u * lvl);
+    if constexpr (KEEP == kKeepLevels) {
+      if (valid) st_record1(w.rec, lvl);
+      w.rec += (nb >> 2) * kRecGroupStride;
+    }
+    if constexpr (KEEP == kKeepFlips) {
+      if (w.lane < R) __stcs(w.flip + w.lane, (F >> (w.lane * L)) & ((1u << L) - 1u));
+      w.flip += R;
+    }
+    prev = c ^ F;
+    lat[v] = prev;   // (every lane stores the same word)
+  }
+};
+
 // One block of the round: its warps' chains, first + warp.
-template <class Rows, bool TSMEM, int KEEP>
+template <class Rows, int L, bool TSMEM, int KEEP>
 __device__ __forceinline__ void warp_gen_body(const DevJob& j, const uint64_t t0, const int64_t S,
                                               const int64_t flushF, const int do_trace, const int block) {
   extern __shared__ __align__(16) uint32_t smem[];
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
-  const int L = j.L, np1 = j.np1;
+  constexpr int N = L * L, np1 = N + 1, wd = (L + 31) / 32;
   const WarpPlan pl = warp_plan(L, nthr >> 5, TSMEM);
   uint32_t* hist = smem + pl.hist;
   uint32_t* lat = smem + pl.lat + warp * L * Rows::kRowWords;
@@ -621,15 +760,14 @@ __device__ __forceinline__ void warp_gen_body(const DevJob& j, const uint64_t t0
   for (int i = tid; i < np1; i += nthr) hist[i] = 0u;
   const int chain = block * (nthr >> 5) + warp;
   const bool active = chain < j.p;   // (uniform in a warp)
-  uint32_t* spins = j.spins + static_cast<size_t>(active ? chain : 0) * L * j.wd;
+  uint32_t* spins = j.spins + static_cast<size_t>(active ? chain : 0) * L * wd;
   int m = 0;
   if (active) {
-    Rows::load(lat, spins, L, lane);
+    Rows::load(lat, spins, lane);
     m = j.m[chain];
   }
   __syncthreads();
   WarpLane w;
-  w.L = L;
   w.lane = lane;
   w.bit = 1u << lane;
   w.lt = w.bit - 1u;
@@ -647,7 +785,7 @@ __device__ __forceinline__ void warp_gen_body(const DevJob& j, const uint64_t t0
   if constexpr (KEEP == kKeepFlips) w.flip = j.flips + static_cast<size_t>(active ? chain : 0) * flip_words(L, S);
   if constexpr (KEEP == kKeepLevels) {
     const int k = Rows::kSitesPerLane * lane;   // this lane's first sample in a window
-    w.rec = j.rec + rec_index(active ? chain : 0, 0, S * j.N) + (k >> 2) * kRecGroupStride + (k & 3);
+    w.rec = j.rec + rec_index(active ? chain : 0, 0, S * N) + (k >> 2) * kRecGroupStride + (k & 3);
   }
   WarpRing ring;
   ring.ring = reinterpret_cast<char*>(smem + pl.ring + warp * kRingWords);
@@ -662,17 +800,17 @@ __device__ __forceinline__ void warp_gen_body(const DevJob& j, const uint64_t t0
     if (active) {
       if (j.ckpt && ck_left == 0) {
         // lattice and level at the start of segment s / C, for the joint's replays
-        Rows::store(j.ckpt + static_cast<size_t>(seg) * L * j.wd * j.p + chain, static_cast<size_t>(j.p), lat, L, lane);
+        Rows::store(j.ckpt + static_cast<size_t>(seg) * L * wd * j.p + chain, static_cast<size_t>(j.p), lat, lane);
         if (lane == 0) j.ckm[static_cast<size_t>(seg) * j.p + chain] = m;
       }
       Rows rows;
-      rows.begin(lat, L);
+      rows.begin(lat);
 #pragma unroll 1
-      for (int y = 0; y < L; ++y) {
+      for (int y = 0; y < L; y += Rows::step()) {
         rows.template row<TSMEM, KEEP>(lat, y, m, w, ring);
         __syncwarp();
       }
-      if (do_trace && lane == 0) j.trace[s * j.p + chain] = 4 * m - 2 * j.N;
+      if (do_trace && lane == 0) j.trace[s * j.p + chain] = 4 * m - 2 * N;
     }
     if (ck_left == 0) {
       ck_left = j.ck_C;
@@ -694,7 +832,7 @@ __device__ __forceinline__ void warp_gen_body(const DevJob& j, const uint64_t t0
     }
   }
   if (active) {
-    Rows::store(spins, 1, lat, L, lane);
+    Rows::store(spins, 1, lat, lane);
     if (lane == 0) j.m[chain] = m;
   }
   asm volatile("" ::: "memory");
@@ -703,6 +841,26 @@ __device__ __forceinline__ void warp_gen_body(const DevJob& j, const uint64_t t0
     const uint32_t v = hist[i];
     if (v) atomicAdd(&j.hgen[i], static_cast<unsigned long long>(v));
   }
+}
+
+template <class Rows, int L, bool TSMEM, int KEEP>
+__global__ void __launch_bounds__(32 * kWarpChainBlock, 1)
+    warp_gen_kernel(const DevJob j, const uint64_t t0, const int64_t S, const int64_t flushF, const int do_trace) {
+  warp_gen_body<Rows, L, TSMEM, KEEP>(j, t0, S, flushF, do_trace, blockIdx.x);
+}
+
+template <class Rows, int L>
+inline cudaError_t launch_warp_rows(const DevJob& j, int warps, bool ts, uint64_t t0, int64_t S, bool trace,
+                                    cudaStream_t st) {
+  auto kern = ts ? warp_gen_kernel<Rows, L, true, kKeepNone> : warp_gen_kernel<Rows, L, false, kKeepNone>;
+  if (j.rec) kern = ts ? warp_gen_kernel<Rows, L, true, kKeepLevels> : warp_gen_kernel<Rows, L, false, kKeepLevels>;
+  else if (j.flips) kern = ts ? warp_gen_kernel<Rows, L, true, kKeepFlips> : warp_gen_kernel<Rows, L, false, kKeepFlips>;
+  const size_t bytes = 4ull * warp_plan(L, warps, ts).total;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  if (e != cudaSuccess) return e;
+  kern<<<blocks_for(j.p, warps), 32 * warps, bytes, st>>>(j, t0, S, warp_flush_sweeps(warps, j.N, S), trace ? 1 : 0);
+  launches_add(1);
+  return cudaGetLastError();
 }
 
 #endif  // __CUDACC__

@@ -35,7 +35,7 @@ def _run(L, p, S, W, order, replay):
     return out, held
 
 
-@pytest.mark.parametrize("L,p,S,scale,order", [(8, 9001, 15_000, 6.0, 0), (20, 9000, 2_400, 3.0, 1),
+@pytest.mark.parametrize("L,p,S,scale,order", [(8, 9001, 15_000, 6.0, 0), (12, 1500, 40_000, 2.0, 0), (20, 9000, 2_400, 3.0, 1),
                                                (32, 8200, 1_030, 4.0, 0), (36, 2001, 3_350, 0.2, 0),
                                                (64, 1000, 2_150, 4.0, 0), (76, 700, 2_150, 0.2, 1),
                                                (100, 301, 2_900, 3.0, 0), (128, 160, 3_300, 0.3, 0)])
