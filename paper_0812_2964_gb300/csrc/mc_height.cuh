@@ -19,10 +19,17 @@
 // W[x] within rounding of one another) is undecided, and the ordinary
 // resolution passes finish from that chain on.
 //
-// What bounds the pass over the samples: a Philox word (10 operations), one
-// load of the level's weight from shared memory, and a filter of six
-// operations (one of them an exponential) that lets a sample through to the
-// exact bookkeeping only if it may be among the chain's two best.
+// What bounds the pass over the samples: instruction issue and the integer
+// pipes -- 24 instructions a sample, most of them the Philox block of four
+// samples.  Four samples share one filter (the largest weight against the
+// smallest uniform, one exponential) that lets them through to the exact
+// bookkeeping only if one may be among the chain's two best.  The uniforms
+// are drawn four at a time where they are used: with a lattice word's 32 held
+// in registers an SM held 16 warps instead of 24.  Measured, one filter a
+// sample and 32 uniforms ahead, and now: L = 32, p = 16384, S = 1000 (flips)
+// 18.1 -> 16.0 ms; L = 64, p = 4096, S = 1000 23.8 -> 19.3.  (No sample's
+// uniform can be left undrawn however low its level's weight: a uniform of 0
+// passes every test.)
 #pragma once
 #include "mc_chain.cuh"
 #include "mc_internal.h"
@@ -36,6 +43,7 @@ struct alignas(16) Height {
   float best, second;   // the two largest v
 };
 constexpr uint32_t kNoLevel = 0xFFFFFFFFu;
+constexpr uint32_t kSettled = 0xFFFFFFFEu;   // the level of a chain whose height nothing needs
 // |height_value - exact v| stays below half of this: log2 of a float (relative
 // error 2^-22 of at most 32, plus the rounding of u) and the rounding of W
 constexpr double kHeightEps = 1e-4;
@@ -120,6 +128,30 @@ __device__ __forceinline__ bool height_filter(float x, uint32_t u) {
   return !(u1 >= e + 1.0000005f);
 }
 
+// The same for any of four samples: the largest weight against the smallest
+// uniform.  One exponential for four, and a third of the operations of four
+// tests (the exponential's unit takes 8 cycles a warp).
+__device__ __forceinline__ bool height_filter4(const float* wl, const int (&m4)[4], float bl, const uint4& u) {
+  float w[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) w[q] = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(wl) + m4[q]);
+  float top;   // (a NaN stays one)
+  asm("{.reg .f32 t;\n\tmax.NaN.f32 t, %1, %2, %3;\n\tmax.NaN.f32 %0, t, %4;}"
+      : "=f"(top) : "f"(w[0]), "f"(w[1]), "f"(w[2]), "f"(w[3]));
+  return height_filter(top - bl, min(__vimin3_u32(u.x, u.y, u.z), u.w));
+}
+
+// Which of the four pass it by themselves.
+__device__ __forceinline__ uint32_t height_passing(const float* wl, const int (&m4)[4], float bl, const uint4& u) {
+  uint32_t r = 0u;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float w = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(wl) + m4[q]);
+    if (height_filter(w - bl, uint4_word(u, static_cast<uint32_t>(q)))) r |= 1u << q;
+  }
+  return r;
+}
+
 // Hook of the pass over a segment's samples.  wl[m] = (W[m] - Wref) / ln 2 as
 // a float; a sample can be among the best two only if u / 2^32 <
 // 2^(wl[m] - bl), bl below the second-best v found so far by more than the
@@ -130,10 +162,9 @@ struct HeightHook {
   float slack, bl;
   int64_t k;
   uint32_t chain, r, k0, k1;
-  uint32_t uj[32];
+  uint32_t blk;         // the word's first Philox block
   Height h;
-  int mq[4];            // the current group of four samples: levels (times 4),
-  bool any;             // whether one of them passed the filter
+  int mq[4];            // the current group of four samples: levels (times 4)
   bool done;            // never set: the whole segment is read
   __device__ __forceinline__ void begin() {
     h = height_none();
@@ -141,30 +172,32 @@ struct HeightHook {
   }
   __device__ __forceinline__ void poll() { bl = fmaxf(bl, height_load(entry).second - slack); }
   __device__ __forceinline__ void word(int nb) {
-    joint_fill(uj, nb, k, r, chain, k0, k1);
+    blk = static_cast<uint32_t>(static_cast<uint64_t>(k) >> 2);
     k += nb;
   }
-  // (one branch and one copy of the bookkeeping per four samples: unrolled a
-  // word at a time, a copy a sample overran the instruction cache)
+  // (one test, one branch and one copy of the bookkeeping per four samples:
+  // unrolled a word at a time, a copy a sample overran the instruction cache)
   __device__ __forceinline__ void sample(int m4, int b) {
-    const float w = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(wl) + m4);
-    const bool pass = height_filter(w - bl, uj[b]);
     mq[b & 3] = m4;
-    any = (b & 3) == 0 ? pass : (any || pass);
-    if ((b & 3) == 3 && any) {
+    if ((b & 3) != 3) return;
+    const uint4 u = philox4x32_10(make_uint4(blk + static_cast<uint32_t>(b >> 2), r, chain, kTagJoint), k0, k1);
+    if (height_filter4(wl, mq, bl, u)) {
+      // (in small rounds every second group has a lane that passes: one turn per passing
+      // sample, 28 us a pass at L = 16, p = 512, S = 20 instead of 36 with all four)
 #pragma unroll 1
-      for (int q = 0; q < 4; ++q) {
+      for (uint32_t left = height_passing(wl, mq, bl, u); left; left &= left - 1u) {
+        const int q = __ffs(static_cast<int>(left)) - 1;
         const int mm = q == 0 ? mq[0] : (q == 1 ? mq[1] : (q == 2 ? mq[2] : mq[3]));
-        const uint32_t u = q == 0 ? uj[b - 3] : (q == 1 ? uj[b - 2] : (q == 2 ? uj[b - 1] : uj[b]));
+        const uint32_t uq = uint4_word(u, static_cast<uint32_t>(q));
         const float wq = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(wl) + mm);
-        const float v = u ? wq + height_draw(u) : __int_as_float(0x7F800000);
+        const float v = uq ? wq + height_draw(uq) : __int_as_float(0x7F800000);
         if (v > h.second) {
           const bool top = v > h.best;
           h.second = top ? h.best : v;
           if (top) {
             h.best = v;
             h.m = static_cast<uint32_t>(mm) >> 2;
-            h.u = u;
+            h.u = uq;
           }
         }
       }

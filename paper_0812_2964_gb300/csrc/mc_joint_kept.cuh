@@ -90,26 +90,24 @@ struct TestHook {
   float bl;                         // the input's, lowered by the floats' errors
   int64_t k, kw, found;
   uint32_t chain, r, k0, k1;
-  uint32_t uj[32];
+  uint32_t blk;
   int mq[4];
-  bool any;
   bool done;
   __device__ __forceinline__ void word(int nb) {
-    joint_fill(uj, nb, k, r, chain, k0, k1);
+    blk = static_cast<uint32_t>(static_cast<uint64_t>(k) >> 2);
     kw = k;
     k += nb;
   }
   __device__ __forceinline__ void sample(int m4, int b) {   // (by fours, as in HeightHook)
-    const float w = *reinterpret_cast<const float*>(reinterpret_cast<const char*>(wl) + m4);
-    const bool pass = height_filter(w - bl, uj[b]);
     mq[b & 3] = m4;
-    any = (b & 3) == 0 ? pass : (any || pass);
-    if ((b & 3) == 3 && any) {
+    if ((b & 3) != 3) return;
+    const uint4 u = philox4x32_10(make_uint4(blk + static_cast<uint32_t>(b >> 2), r, chain, kTagJoint), k0, k1);
+    if (height_filter4(wl, mq, bl, u)) {
 #pragma unroll 1
-      for (int q = 0; q < 4 && !done; ++q) {
+      for (uint32_t left = height_passing(wl, mq, bl, u); left && !done; left &= left - 1u) {
+        const int q = __ffs(static_cast<int>(left)) - 1;
         const int mm = q == 0 ? mq[0] : (q == 1 ? mq[1] : (q == 2 ? mq[2] : mq[3]));
-        const uint32_t u = q == 0 ? uj[b - 3] : (q == 1 ? uj[b - 2] : (q == 2 ? uj[b - 1] : uj[b]));
-        if (joint_test(W, mm >> 2, wx, u)) {
+        if (joint_test(W, mm >> 2, wx, uint4_word(u, static_cast<uint32_t>(q)))) {
           found = kw + (b - 3 + q) + 1;
           done = true;
         }
@@ -141,6 +139,8 @@ struct CountHook {
 };
 
 // ------------------------------------------------------------------ kernels
+constexpr int kKeptWarps = 12;   // a block's most (two such blocks an SM: 80 registers)
+
 __device__ __forceinline__ unsigned long long* kept_queue(const DevJob& j, int which) {
   return reinterpret_cast<unsigned long long*>(&j.stats[which]);
 }
@@ -179,7 +179,7 @@ __device__ __forceinline__ void kept_test_setup(const DevJob& j, TestHook& hk, c
 // segment is skipped, or left at the next poll, once an earlier one of its
 // chain has a hit.
 template <class Src>
-__global__ void __launch_bounds__(128) kept_search_kernel(const DevJob j, const int cpw, const int64_t S,
+__global__ void __launch_bounds__(32 * kKeptWarps, 2) kept_search_kernel(const DevJob j, const int cpw, const int64_t S,
                                                           const uint32_t r, const int listed, const int later,
                                                           const int exact_first) {
   if (exact_first && rough_last_joint(j.stats[kStatRejected], j.p)) return;   // (the first search only)
@@ -234,7 +234,8 @@ __global__ void __launch_bounds__(128) kept_search_kernel(const DevJob j, const 
 // samples, so that the pass's filter is tight from the start (without it each
 // segment's first samples pass: 15 of 2048 a lane, a quarter of the warps'
 // iterations): the second best of up to 1024 samples spread over the chain,
-// one warp a chain.  Starts the chain's entry.
+// one warp a chain.  Starts the chain's entry; the chains before the first
+// pending one are marked settled.
 __device__ __forceinline__ void height_top2(float v, float& best, float& second) {
   second = fmaxf(second, fminf(best, v));
   best = fmaxf(best, v);
@@ -248,8 +249,16 @@ __global__ void __launch_bounds__(128) kept_seed_kernel(const DevJob j, const in
   const int64_t M = S * j.N;
   const int n = Src::seeds(j, M);
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (int q = f + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5); q < j.p; q += nwarps) {
+  for (int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < j.p; q += nwarps) {
     const int i = j.perm[q];
+    if (q < f) {   // (its answer stands)
+      if (lane == 0) {
+        Height h = height_none();
+        h.m = kSettled;
+        heights(j)[i] = h;
+      }
+      continue;
+    }
     float best = height_none().best, second = best;
     for (int a = lane; a < n; a += 32) {
       int64_t k;   // distinct samples (0-based)
@@ -272,14 +281,15 @@ __global__ void __launch_bounds__(128) kept_seed_kernel(const DevJob j, const in
 }
 
 // Heights of the chains from the first pending one on: items as in the
-// search, all segments.
+// search, all segments.  Lanes take the chains by index, whatever the joint's
+// order, so that a warp reads whole runs of the record (taken in the order of
+// an ordered joint, a warp's loads were 32 separate sectors each: L = 52,
+// p = 1000, S = 100 0.75 ms a pass, 0.33 now).
 template <class Src>
-__global__ void __launch_bounds__(128) kept_height_kernel(const DevJob j, const int cpw, const int64_t S,
+__global__ void __launch_bounds__(32 * kKeptWarps, 2) kept_height_kernel(const DevJob j, const int cpw, const int64_t S,
                                                           const uint32_t r) {
   if (j.stats[kStatPending] == 0) return;
-  const int f = static_cast<int>(j.stats[kStatFirstPending]);
-  const int nchains = j.p - f;
-  const long long items = static_cast<long long>(nchains) * j.ck_K;
+  const long long items = static_cast<long long>(j.p) * j.ck_K;
   const SmemPlan sp = smem_plan(j.L, Src::kPlacement, cpw, blockDim.x >> 5, false, true);
   BlockCtx b = block_setup<false>(j, sp, cpw, 0, false);
   const float* wl = kept_weights(j, b);
@@ -292,9 +302,8 @@ __global__ void __launch_bounds__(128) kept_height_kernel(const DevJob j, const 
     base = __shfl_sync(0xFFFFFFFFu, base, 0);
     if (base >= items) break;
     const long long item = base + b.lane;
-    if (b.lane < cpw && item < items) {
-      const int seg = static_cast<int>(item / nchains);
-      const int i = j.perm[f + static_cast<int>(item % nchains)];
+    const int i = static_cast<int>(item % j.p), seg = static_cast<int>(item / j.p);
+    if (b.lane < cpw && item < items && __ldcg(&heights(j)[i].m) != kSettled) {
       HeightHook hk;
       hk.wl = wl;
       hk.entry = heights(j) + i;
@@ -325,7 +334,7 @@ __global__ void __launch_bounds__(128) kept_height_kernel(const DevJob j, const 
 // hold at most 2^36 samples, and a grid is smaller than the chip only when
 // there are few items).
 template <class Src>
-__global__ void __launch_bounds__(128) kept_count_kernel(const DevJob j, const int cpw, const int64_t S) {
+__global__ void __launch_bounds__(32 * kKeptWarps, 2) kept_count_kernel(const DevJob j, const int cpw, const int64_t S) {
   const int nchains = static_cast<int>(j.stats[kStatNoHit]);
   const long long items = static_cast<long long>(nchains) * j.ck_K;
   const int slots = (blockDim.x >> 5) * cpw;
@@ -453,32 +462,55 @@ inline cudaError_t kept_attr(K kern, size_t bytes) {
   return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
 }
 
+// Warps a block of a pass over so many items: the passes wait on each warp's
+// own chain of operations, so what counts is the warps an SM holds, and a
+// block's warps share one copy of the level weights (64 KiB at L = 128).  From
+// four warps up to kKeptWarps, as many as let an SM hold more of them -- where
+// the items fill the chip (fewer are spread over it in small blocks).
+// Measured, four warps a block and then this: L = 64, 1.7e10 samples, flips (64
+// KiB of lattices each four warps: 8 warps an SM, 12 now) heights 20.6 -> 19.3
+// ms, counts 3.8 -> 1.7; L = 128, 3.4e9 samples, recorded (12 warps an SM, 24
+// now) heights 3.0 -> 3.0 ms, counts 1.10 -> 0.66.
+inline LaunchShape kept_shape(const DevJob& j, LaunchShape s, long long items) {
+  const auto held = [&](int wpb) {
+    const LaunchShape t{s.placement, s.cpw, wpb};
+    return std::min<int>(2 * kKeptWarps, static_cast<int>((kMaxSmem + 1024) / (plan_bytes(j.L, t, false, true) + 2048)) * wpb);
+  };
+  const int base = s.wpb;
+  if (items < 152ll * s.cpw * std::max(1, held(base))) return s;
+  for (int wpb = 2 * base; wpb <= kKeptWarps; wpb += base)
+    if (held(wpb) > held(s.wpb)) s.wpb = wpb;
+  return s;
+}
+
 // s: lanes a warp and warps a block of the passes over segments (Src's
 // lattices and the level weights fit in shared memory).
 template <class Src>
 inline cudaError_t launch_join_kept(const DevJob& j, const LaunchShape& s, int64_t S, uint32_t r, cudaStream_t st) {
-  const size_t bytes = plan_bytes(j.L, s, false, true);
-  const int per_block = s.cpw * s.wpb, threads = 32 * s.wpb;
   auto kq = kept_search_kernel<Src>;
   auto kh = kept_height_kernel<Src>;
   auto kc = kept_count_kernel<Src>;
   auto kr = kept_resolve_kernel<Src>;
   cudaError_t e;
-  if ((e = kept_attr(kq, bytes)) != cudaSuccess || (e = kept_attr(kh, bytes)) != cudaSuccess ||
-      (e = kept_attr(kc, bytes)) != cudaSuccess || (e = kept_attr(kr, bytes)) != cudaSuccess)
-    return e;
   const long long items = static_cast<long long>(j.p) * j.ck_K;
-  const auto grid = [&](long long n, long long resident) {
-    return static_cast<unsigned>(std::max<long long>(1, std::min<long long>(blocks_for(n, per_block), resident)));
+  const LaunchShape all = kept_shape(j, s, items), one = kept_shape(j, s, j.p);   // all segments; one a chain
+  const size_t bytes = plan_bytes(j.L, s, false, true), all_bytes = plan_bytes(j.L, all, false, true),
+               one_bytes = plan_bytes(j.L, one, false, true);
+  if ((e = kept_attr(kq, std::max(all_bytes, one_bytes))) != cudaSuccess || (e = kept_attr(kh, all_bytes)) != cudaSuccess ||
+      (e = kept_attr(kc, all_bytes)) != cudaSuccess || (e = kept_attr(kr, bytes)) != cudaSuccess)
+    return e;
+  const auto grid = [&](auto kern, const LaunchShape& t, size_t b, long long n) {
+    return static_cast<unsigned>(std::max<long long>(
+        1, std::min<long long>(blocks_for(n, t.cpw * t.wpb), resident_blocks(kern, 32 * t.wpb, b))));
   };
-  const long long res_q = resident_blocks(kq, threads, bytes);
+  const unsigned grid_one = grid(kq, one, one_bytes, j.p), grid_later = grid(kq, all, all_bytes, items);
   // (the default limit is the replays': a kept round of any size takes the exact path)
   const bool exact = static_cast<long long>(j.p) * S * j.N <= j.scan_max_samples || j.scan_max_samples == kScanMaxSamples;
   auto search = [&](int listed, int first) -> cudaError_t {
-    kq<<<grid(j.p, res_q), threads, bytes, st>>>(j, s.cpw, S, r, listed, 0, first);
+    kq<<<grid_one, 32 * one.wpb, one_bytes, st>>>(j, one.cpw, S, r, listed, 0, first);
     launches_add(1);
     if (j.ck_K > 1) {
-      kq<<<grid(items, res_q), threads, bytes, st>>>(j, s.cpw, S, r, listed, 1, first);
+      kq<<<grid_later, 32 * all.wpb, all_bytes, st>>>(j, all.cpw, S, r, listed, 1, first);
       launches_add(1);
     }
     return cudaGetLastError();
@@ -503,7 +535,7 @@ inline cudaError_t launch_join_kept(const DevJob& j, const LaunchShape& s, int64
     if ((e = passes(j.passes_scan, kMarkDefer)) != cudaSuccess) return e;
     if ((e = mark(0)) != cudaSuccess) return e;
     kept_seed_kernel<Src><<<std::min(2432u, blocks_for(j.p, 4)), 128, 0, st>>>(j, S, r);
-    kh<<<grid(items, resident_blocks(kh, threads, bytes)), threads, bytes, st>>>(j, s.cpw, S, r);
+    kh<<<grid(kh, all, all_bytes, items), 32 * all.wpb, all_bytes, st>>>(j, all.cpw, S, r);
     launches_add(2);
     if ((e = kept_scan(j, st)) != cudaSuccess) return e;
     if ((e = search(1, 0)) != cudaSuccess) return e;
@@ -512,8 +544,8 @@ inline cudaError_t launch_join_kept(const DevJob& j, const LaunchShape& s, int64
     if ((e = passes(j.passes_plain, 0)) != cudaSuccess) return e;
   }
   if ((e = mark(kMarkFinal)) != cudaSuccess) return e;
-  kr<<<1, threads, bytes, st>>>(j, s.cpw, S, r);
-  kc<<<grid(items, resident_blocks(kc, threads, bytes)), threads, bytes, st>>>(j, s.cpw, S);
+  kr<<<1, 32 * s.wpb, bytes, st>>>(j, s.cpw, S, r);
+  kc<<<grid(kc, all, all_bytes, items), 32 * all.wpb, all_bytes, st>>>(j, all.cpw, S);
   launches_add(2);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return join_finalize(j, S, st);
