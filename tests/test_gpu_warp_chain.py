@@ -40,3 +40,9 @@ def test_chain_counts(p):
 
 def test_default_shape_is_one_chain_a_warp():
     _run_parity(48, 40, 2, 3, 1, seed=9)
+
+
+@pytest.mark.parametrize("L", [36, 64, 68, 100, 128])
+def test_many_chains_of_long_rows(L):
+    """Past the chain count up to which rows are resolved 64 sites at a time."""
+    _run_parity(L, 1300, 1, 2, 1, seed=11, weights=random_weights(L, 5, 3.0))
