@@ -197,11 +197,11 @@ int mc_set_join_policy(mc_job *job, int64_t scan_max_samples, int passes_before_
  * levels, the count of its discarded prefix) runs one segment per GPU lane,
  * so the segment length bounds the joint's critical path.  The library
  * aims at segments of about `samples` attempts (whole sweeps; 0 restores
- * the default of 2^16, of 2^14 where the round keeps its flips), keeps at least min(32, S) segments and at most
- * 2^24 samples per segment, and takes fewer, longer segments where their
- * checkpoints would exceed 4 GiB.  mc_get_info reports the choice of the
- * last round.  MC_EINVAL for samples < 0, MC_ESTATE while a round is
- * pending. */
+ * the default of 2^16, of 2^14 and at least two sweeps where the round keeps
+ * its flips), keeps at least min(32, S) segments and at most 2^24 samples per
+ * segment, and takes fewer, longer segments where their checkpoints would
+ * exceed 4 GiB.  mc_get_info reports the choice of the last round.
+ * MC_EINVAL for samples < 0, MC_ESTATE while a round is pending. */
 int mc_set_segment_samples(mc_job *job, int64_t samples);
 
 /* Checkpoint / resume (no counterpart in the paper).  mc_save writes the

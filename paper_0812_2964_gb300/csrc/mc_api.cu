@@ -328,8 +328,9 @@ namespace {
 constexpr int64_t kSegmentSamples = int64_t(1) << 16;   // default target
 // ... of rounds that keep their flips: rebuilding a segment's levels is so much
 // shorter than running it again that the first segments of a few hundred
-// chains, one a lane, would be most of a search (0.9 ms at 2^16)
-constexpr int64_t kFlipSegmentSamples = int64_t(1) << 14;
+// chains, one a lane, would be most of a search (0.9 ms at 2^16).  At least two
+// sweeps: a segment's lattice is as large as one sweep's flips.
+int64_t flip_segment_samples(int L) { return std::max<int64_t>(int64_t(1) << 14, 2ll * L * L); }
 constexpr int64_t kCheckpointBytes = int64_t(4) << 30;   // per job
 
 // Bytes of the checkpoint buffers per segment: lattices, levels, prefix work list.
@@ -469,7 +470,7 @@ void ensure_flips(mc_job* job, int64_t n_sweeps, bool allow) {
 // Segments of the job's round: finer ones by default where it keeps its flips.
 void choose_segments(const mc_job* job, int64_t n_sweeps, bool allow_record, int* K, int* C) {
   const bool flips = allow_record && flip_record_words(job->L, job->p, n_sweeps, job->rec_max) > 0;
-  round_segments(job->L, job->p, n_sweeps, job->seg_samples > 0 || !flips ? job->seg_samples : kFlipSegmentSamples, K, C);
+  round_segments(job->L, job->p, n_sweeps, job->seg_samples > 0 || !flips ? job->seg_samples : flip_segment_samples(job->L), K, C);
 }
 
 // The round's record (of levels or flips) for a batch, where there is memory
@@ -1483,7 +1484,7 @@ uint64_t mc_job_device_bytes(int L, int n_chains, int64_t sweeps) {
                p * 8 + p * 4 + p * 4 + p * 4 + p * 20 + np1 + p * 4 + np1 * 4 + p * 8 + mcgpu::kStatCount * 8;
   int K = 0, C = 0;
   const size_t flip_words = flip_record_words(L, n_chains, sweeps, mcgpu::default_record_max(L));
-  round_segments(L, n_chains, sweeps, flip_words ? kFlipSegmentSamples : 0, &K, &C);
+  round_segments(L, n_chains, sweeps, flip_words ? flip_segment_samples(L) : 0, &K, &C);
   (void)lw;
   const uint64_t samples = p * static_cast<uint64_t>(sweeps) * N;   // record of the round, if small
   const uint64_t rec = samples <= static_cast<uint64_t>(mcgpu::default_record_max(L))

@@ -22,7 +22,7 @@ def _run(L, p, S, W, order, replay):
         g.set_round_record(0)
     g.set_join_order(order)
     g.weights = W
-    g.set_segment_samples(1 << 14)      # (the same checkpoints either way)
+    g.set_segment_samples(max(1 << 14, 2 * L * L))      # (the same checkpoints either way)
     out = []
     for _ in range(2):
         g.run_sweeps(S)
