@@ -22,6 +22,7 @@
 #pragma once
 #include "mc_chain_kernels.cuh"
 #include "mc_height.cuh"
+#include "mc_launch.cuh"
 
 namespace mcgpu {
 
@@ -182,6 +183,7 @@ template <class Src>
 __global__ void __launch_bounds__(32 * kKeptWarps, 2) kept_search_kernel(const DevJob j, const int cpw, const int64_t S,
                                                           const uint32_t r, const int listed, const int later,
                                                           const int exact_first) {
+  after_previous();
   if (exact_first && rough_last_joint(j.stats[kStatRejected], j.p)) return;   // (the first search only)
   const int nchains = later ? static_cast<int>(j.stats[kStatNoHit]) : (listed ? static_cast<int>(j.stats[kStatPending]) : j.p);
   const int segs = later ? j.ck_K - 1 : 1;
@@ -242,6 +244,7 @@ __device__ __forceinline__ void height_top2(float v, float& best, float& second)
 }
 template <class Src>
 __global__ void __launch_bounds__(128) kept_seed_kernel(const DevJob j, const int64_t S, const uint32_t r) {
+  after_previous();
   if (j.stats[kStatPending] == 0) return;
   const int f = static_cast<int>(j.stats[kStatFirstPending]);
   const float* wl = level_weights(j);
@@ -288,6 +291,7 @@ __global__ void __launch_bounds__(128) kept_seed_kernel(const DevJob j, const in
 template <class Src>
 __global__ void __launch_bounds__(32 * kKeptWarps, 2) kept_height_kernel(const DevJob j, const int cpw, const int64_t S,
                                                           const uint32_t r) {
+  after_previous();
   if (j.stats[kStatPending] == 0) return;
   const long long items = static_cast<long long>(j.p) * j.ck_K;
   const SmemPlan sp = smem_plan(j.L, Src::kPlacement, cpw, blockDim.x >> 5, false, true);
@@ -335,6 +339,7 @@ __global__ void __launch_bounds__(32 * kKeptWarps, 2) kept_height_kernel(const D
 // there are few items).
 template <class Src>
 __global__ void __launch_bounds__(32 * kKeptWarps, 2) kept_count_kernel(const DevJob j, const int cpw, const int64_t S) {
+  after_previous();
   const int nchains = static_cast<int>(j.stats[kStatNoHit]);
   const long long items = static_cast<long long>(nchains) * j.ck_K;
   const int slots = (blockDim.x >> 5) * cpw;
@@ -375,6 +380,7 @@ __global__ void __launch_bounds__(32 * kKeptWarps, 2) kept_count_kernel(const De
 template <class Src>
 __global__ void __launch_bounds__(128) kept_resolve_kernel(const DevJob j, const int cpw, const int64_t S,
                                                            const uint32_t r) {
+  after_previous();
   if (j.stats[kStatPending] == 0) return;
   const SmemPlan sp = smem_plan(j.L, Src::kPlacement, cpw, blockDim.x >> 5, false, true);
   BlockCtx b = block_setup<false>(j, sp, cpw, 0, false);
@@ -507,10 +513,10 @@ inline cudaError_t launch_join_kept(const DevJob& j, const LaunchShape& s, int64
   // (the default limit is the replays': a kept round of any size takes the exact path)
   const bool exact = static_cast<long long>(j.p) * S * j.N <= j.scan_max_samples || j.scan_max_samples == kScanMaxSamples;
   auto search = [&](int listed, int first) -> cudaError_t {
-    kq<<<grid_one, 32 * one.wpb, one_bytes, st>>>(j, one.cpw, S, r, listed, 0, first);
+    launch_next(kq, grid_one, 32 * one.wpb, one_bytes, st, j, one.cpw, S, r, listed, 0, first);
     launches_add(1);
     if (j.ck_K > 1) {
-      kq<<<grid_later, 32 * all.wpb, all_bytes, st>>>(j, all.cpw, S, r, listed, 1, first);
+      launch_next(kq, grid_later, 32 * all.wpb, all_bytes, st, j, all.cpw, S, r, listed, 1, first);
       launches_add(1);
     }
     return cudaGetLastError();
@@ -534,8 +540,8 @@ inline cudaError_t launch_join_kept(const DevJob& j, const LaunchShape& s, int64
   if (exact) {
     if ((e = passes(j.passes_scan, kMarkDefer)) != cudaSuccess) return e;
     if ((e = mark(0)) != cudaSuccess) return e;
-    kept_seed_kernel<Src><<<std::min(2432u, blocks_for(j.p, 4)), 128, 0, st>>>(j, S, r);
-    kh<<<grid(kh, all, all_bytes, items), 32 * all.wpb, all_bytes, st>>>(j, all.cpw, S, r);
+    launch_next(kept_seed_kernel<Src>, std::min(2432u, blocks_for(j.p, 4)), 128, 0, st, j, S, r);
+    launch_next(kh, grid(kh, all, all_bytes, items), 32 * all.wpb, all_bytes, st, j, all.cpw, S, r);
     launches_add(2);
     if ((e = kept_scan(j, st)) != cudaSuccess) return e;
     if ((e = search(1, 0)) != cudaSuccess) return e;
@@ -544,8 +550,8 @@ inline cudaError_t launch_join_kept(const DevJob& j, const LaunchShape& s, int64
     if ((e = passes(j.passes_plain, 0)) != cudaSuccess) return e;
   }
   if ((e = mark(kMarkFinal)) != cudaSuccess) return e;
-  kr<<<1, 32 * s.wpb, bytes, st>>>(j, s.cpw, S, r);
-  kc<<<grid(kc, all, all_bytes, items), 32 * all.wpb, all_bytes, st>>>(j, all.cpw, S);
+  launch_next(kr, 1, 32 * s.wpb, bytes, st, j, s.cpw, S, r);
+  launch_next(kc, grid(kc, all, all_bytes, items), 32 * all.wpb, all_bytes, st, j, all.cpw, S);
   launches_add(2);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return join_finalize(j, S, st);

@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <math_constants.h>
 
+#include "mc_launch.cuh"
 #include "mc_chain_kernels.cuh"
 #include "mc_height.cuh"
 #include "mc_scan_fsm.cuh"
@@ -74,6 +75,7 @@ __global__ void __launch_bounds__(128) levels_kernel(const DevJob j) {
 
 // T[a][m] = thr(W[m + a - 2] - W[m]); moves outside [0, N] never occur.
 __global__ void table_kernel(const DevJob j) {
+  after_previous();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= 5 * j.np1) return;
   const int a = idx / j.np1, m = idx % j.np1;
@@ -83,6 +85,7 @@ __global__ void table_kernel(const DevJob j) {
 
 // Eq. (new_weight) in logarithms: W -= ln h where h > 0; h cleared.
 __global__ void weights_kernel(const DevJob j) {
+  after_previous();
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= j.np1) return;
   const long long h = j.h[m];
@@ -311,6 +314,7 @@ __global__ void spec_inputs_kernel(const DevJob j) {
 // whose scatter walks the chains in index order a warp at a time (ranks among
 // equal levels inside a warp from __match_any_sync).
 __global__ void __launch_bounds__(1024) order_kernel(const DevJob j) {
+  after_previous();
   const int t = threadIdx.x, nt = blockDim.x;
   if (!j.ordered) {
     for (int q = t; q < j.p; q += nt) j.perm[q] = q;
@@ -390,6 +394,7 @@ __device__ __forceinline__ long long block_sum_scan(long long v, long long* s_wa
 // at a time); h += hgen - dpre, or += dpre where that holds the kept samples
 // (the other blocks).
 __global__ void __launch_bounds__(1024) finalize_kernel(const DevJob j, const int64_t M, const int may_count_kept) {
+  after_previous();
   const int t = threadIdx.x;
   if (blockIdx.x > 0) {
     const bool kept = may_count_kept && j.stats[kStatCountKept];
@@ -425,7 +430,7 @@ __global__ void __launch_bounds__(1024) finalize_kernel(const DevJob j, const in
 }
 
 static void launch_finalize(const DevJob& j, int64_t M, bool may_count_kept, cudaStream_t st) {
-  finalize_kernel<<<1 + blocks_for(j.np1, 1024), 1024, 0, st>>>(j, M, may_count_kept ? 1 : 0);
+  launch_next(finalize_kernel, 1 + blocks_for(j.np1, 1024), 1024, 0, st, j, M, may_count_kept ? 1 : 0);
 }
 
 // Control experiment (no detailed balance at the joints): keep everything.
@@ -808,6 +813,7 @@ __device__ __forceinline__ int block_last_kept(const int f, const int p, const K
 // the speculated inputs (spec_inputs_kernel), nothing found yet, the level
 // weights and the cleared counters.
 __global__ void kept_prelude_kernel(const DevJob j) {
+  after_previous();
   const int t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
   if (t == 0) {
     for (const int s : {kStatSearched, kStatMismatch, kStatPasses, kStatPending, kStatScanned, kStatNoHit,
@@ -841,6 +847,7 @@ __global__ void kept_prelude_kernel(const DevJob j) {
 // With kMarkFinal and nothing pending: the carry, and whether fewer samples
 // are kept than discarded.
 __global__ void __launch_bounds__(1024) kept_mark_kernel(const DevJob j, const int64_t M, const int flags) {
+  after_previous();
   __shared__ int s_count, s_first, s_new;
   __shared__ unsigned long long s_kept;
   const int t = threadIdx.x, nt = blockDim.x;
@@ -1085,16 +1092,20 @@ __device__ __forceinline__ void height_path(const DevJob& j) {
 }
 
 __global__ void __launch_bounds__(1024) height_value_kernel(const DevJob j) {
+  after_previous();
   if (j.stats[kStatPending]) height_values(j, blockIdx.x, gridDim.x);
 }
 __global__ void height_next_kernel(const DevJob j) {
+  after_previous();
   if (j.stats[kStatPending]) height_successors(j, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 __global__ void __launch_bounds__(1024) height_path_kernel(const DevJob j) {
+  after_previous();
   if (j.stats[kStatPending]) height_path(j);
 }
 // the three in one launch
 __global__ void __launch_bounds__(1024) height_scan_kernel(const DevJob j) {
+  after_previous();
   if (j.stats[kStatPending] == 0) return;
   height_values(j, 0, 1);
   __syncthreads();
@@ -1226,6 +1237,7 @@ __global__ void __launch_bounds__(32) attempts_kernel(const DevJob j, const uint
 // chain after another).  An input the heights cannot settle leaves the whole
 // round to partial_joint_kernel.
 __global__ void __launch_bounds__(128) partial_height_kernel(const DevJob j, const int64_t M, const uint32_t r) {
+  after_previous();
   const float* wl = level_weights(j);
   const int lane = threadIdx.x & 31, nwarps = (gridDim.x * blockDim.x) >> 5;
   for (int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < j.p; q += nwarps) {
@@ -1263,6 +1275,7 @@ __global__ void __launch_bounds__(128) partial_height_kernel(const DevJob j, con
 }
 
 __global__ void __launch_bounds__(128) partial_finish_kernel(const DevJob j, const int64_t M, const uint32_t r) {
+  after_previous();
   if (j.stats[kStatScanned] < j.p) return;   // undecided somewhere: partial_joint_kernel
   const int lane = threadIdx.x & 31, nwarps = (gridDim.x * blockDim.x) >> 5;
   for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < j.p; c += nwarps) {
@@ -1301,6 +1314,7 @@ __global__ void __launch_bounds__(128) partial_finish_kernel(const DevJob j, con
 // passes) go to dpre.  Where the heights have settled the round it only
 // fixes the carry.
 __global__ void __launch_bounds__(1024) partial_joint_kernel(const DevJob j, const int64_t M, const uint32_t r) {
+  after_previous();
   __shared__ unsigned long long s_k;
   __shared__ int s_carry, s_valid;
   const int t = threadIdx.x, nt = blockDim.x;
@@ -1445,10 +1459,10 @@ cudaError_t k_join_attempts(const DevJob& j, uint64_t t0, int64_t M, uint32_t r,
     cudaError_t e = kept_prelude(j, st);
     if (e != cudaSuccess) return e;
     const unsigned warps = std::min(2432u, blocks_for(j.p, 4));
-    partial_height_kernel<<<warps, 128, 0, st>>>(j, M, r);
+    launch_next(partial_height_kernel, warps, 128, 0, st, j, M, r);
     if ((e = kept_scan(j, st)) != cudaSuccess) return e;
-    partial_finish_kernel<<<warps, 128, 0, st>>>(j, M, r);
-    partial_joint_kernel<<<1, 1024, 0, st>>>(j, M, r);
+    launch_next(partial_finish_kernel, warps, 128, 0, st, j, M, r);
+    launch_next(partial_joint_kernel, 1, 1024, 0, st, j, M, r);
     launch_finalize(j, M, false, st);
     launches_add(4);
     return cudaGetLastError();
@@ -1683,14 +1697,14 @@ cudaError_t join_scan(const DevJob& j, cudaStream_t st) {
 }
 
 cudaError_t kept_prelude(const DevJob& j, cudaStream_t st) {
-  if (j.ordered) order_kernel<<<1, 1024, 0, st>>>(j);
-  kept_prelude_kernel<<<std::min(304u, blocks_for(std::max(j.p, j.np1), 256)), 256, 0, st>>>(j);
+  if (j.ordered) launch_next(order_kernel, 1, 1024, 0, st, j);
+  launch_next(kept_prelude_kernel, std::min(304u, blocks_for(std::max(j.p, j.np1), 256)), 256, 0, st, j);
   launches_add(j.ordered ? 2 : 1);
   return cudaGetLastError();
 }
 
 cudaError_t kept_mark(const DevJob& j, int64_t S, int flags, cudaStream_t st) {
-  kept_mark_kernel<<<1, 1024, 0, st>>>(j, S * j.N, flags);
+  launch_next(kept_mark_kernel, 1, 1024, 0, st, j, S * j.N, flags);
   launches_add(1);
   return cudaGetLastError();
 }
@@ -1698,13 +1712,13 @@ cudaError_t kept_mark(const DevJob& j, int64_t S, int flags, cudaStream_t st) {
 // (one block does the whole scan where its three parts are short: two launches saved)
 cudaError_t kept_scan(const DevJob& j, cudaStream_t st) {
   if (j.p <= 4096) {
-    height_scan_kernel<<<1, 1024, 0, st>>>(j);
+    launch_next(height_scan_kernel, 1, 1024, 0, st, j);
     launches_add(1);
     return cudaGetLastError();
   }
-  height_value_kernel<<<std::min(152u, blocks_for(j.p, 1024)), 1024, 0, st>>>(j);
-  height_next_kernel<<<std::min(1024u, blocks_for(j.p + 1, 128)), 128, 0, st>>>(j);
-  height_path_kernel<<<1, 1024, 0, st>>>(j);
+  launch_next(height_value_kernel, std::min(152u, blocks_for(j.p, 1024)), 1024, 0, st, j);
+  launch_next(height_next_kernel, std::min(1024u, blocks_for(j.p + 1, 128)), 128, 0, st, j);
+  launch_next(height_path_kernel, 1, 1024, 0, st, j);
   launches_add(3);
   return cudaGetLastError();
 }
@@ -1839,7 +1853,7 @@ cudaError_t k_levels(const DevJob& j, cudaStream_t st) {
 }
 
 cudaError_t k_build_table(const DevJob& j, cudaStream_t st) {
-  table_kernel<<<blocks_for(5ll * j.np1, 256), 256, 0, st>>>(j);
+  launch_next(table_kernel, blocks_for(5ll * j.np1, 256), 256, 0, st, j);
   launches_add(1);
   return cudaGetLastError();
 }
@@ -1864,7 +1878,7 @@ cudaError_t k_thermo(const DevJob& j, int n, double* buf, cudaStream_t st) {
 }
 
 cudaError_t k_update_weights(const DevJob& j, cudaStream_t st) {
-  weights_kernel<<<blocks_for(j.np1, 256), 256, 0, st>>>(j);
+  launch_next(weights_kernel, blocks_for(j.np1, 256), 256, 0, st, j);
   launches_add(1);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
