@@ -46,9 +46,7 @@ bool batch_supported(int L, const LaunchShape& s) {
 }
 
 long long batch_resident_blocks(size_t smem_bytes) {
-  if (cudaFuncSetAttribute(gen_batched_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(smem_bytes)) != cudaSuccess)
-    return 0;
+  if (smem_bytes > kMaxSmem || allow_smem(gen_batched_kernel) != cudaSuccess) return 0;
   return resident_blocks(gen_batched_kernel, 32 * kBatchWarps, smem_bytes);
 }
 
@@ -71,8 +69,7 @@ cudaError_t batch_item(const DevJob& j, const LaunchShape& s, uint64_t t0, int64
 }
 
 cudaError_t k_generate_batched(BatchParams& P, size_t smem_bytes, int total_blocks, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(gen_batched_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem_bytes));
+  const cudaError_t e = allow_smem(gen_batched_kernel);
   if (e != cudaSuccess) return e;
   gen_batched_kernel<<<total_blocks, 32 * kBatchWarps, smem_bytes, st>>>(P);
   launches_add(1);

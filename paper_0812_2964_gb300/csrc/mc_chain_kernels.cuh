@@ -748,7 +748,17 @@ struct GlobF : RunnerFactoryGlob<WD, SL> {
   static constexpr int kPlacement = kPlaceGlobal;
 };
 
-constexpr size_t kMaxSmem = 227 * 1024;
+constexpr size_t kMaxSmem = 227 * 1024;   // a block's most
+
+// Lets a kernel have as much dynamic shared memory as fits beside its own
+// variables.  The limit is the kernel's, not the launch's, and host threads
+// with jobs of different sizes launch the same kernels: it is always set to
+// the same value, so that none lowers it under another's launch.
+cudaError_t allow_smem(const void* kernel);
+template <class... P>
+inline cudaError_t allow_smem(void (*kernel)(P...)) {
+  return allow_smem(reinterpret_cast<const void*>(kernel));
+}
 
 // Blocks of a kernel that fit on the device at once (occupancy API).
 template <class K>
@@ -783,7 +793,7 @@ inline cudaError_t launch_gen_t(const DevJob& j, const LaunchShape& s, uint64_t 
     if (s.cpw <= 8)
       kern = j.rec ? gen_kernel<F, TS, 4, kKeepLevels>
                    : (j.flips ? gen_kernel<F, TS, 4, kKeepFlips> : gen_kernel<F, TS, 4, kKeepNone>);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  const cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   const int per_block = s.cpw * s.wpb;
   const unsigned grid = blocks_for(j.p, per_block);
@@ -809,9 +819,7 @@ inline cudaError_t launch_join_t(const DevJob& j, const LaunchShape& s, uint64_t
   cudaError_t e = join_prelude(j, st);
   if (e != cudaSuccess) return e;
   auto kq = search_kernel<F, TS>;
-  if ((e = cudaFuncSetAttribute(kq, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes))) !=
-      cudaSuccess)
-    return e;
+  if ((e = allow_smem(kq)) != cudaSuccess) return e;
   // persistent grids: the blocks that are resident at once, no more than needed
   const unsigned grid_all = static_cast<unsigned>(
       std::min<long long>(blocks_for(items, per_block), resident_blocks(kq, 32 * s.wpb, bytes)));
@@ -853,9 +861,7 @@ inline cudaError_t launch_join_t(const DevJob& j, const LaunchShape& s, uint64_t
     if ((e = join_summary_init(j, st)) != cudaSuccess) return e;
     if ((e = join_reset_queue(j, st)) != cudaSuccess) return e;
     auto ks = summary_kernel<F, TS>;
-    if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes))) !=
-        cudaSuccess)
-      return e;
+    if ((e = allow_smem(ks)) != cudaSuccess) return e;
     const unsigned grid_sum = static_cast<unsigned>(
         std::min<long long>(blocks_for(items, per_block), resident_blocks(ks, 32 * s.wpb, bytes)));
     ks<<<grid_sum, 32 * s.wpb, bytes, st>>>(j, s.cpw, t0, S, r);
@@ -869,14 +875,10 @@ inline cudaError_t launch_join_t(const DevJob& j, const LaunchShape& s, uint64_t
     if ((e = pass(j.passes_plain, false)) != cudaSuccess) return e;
   }
   auto kr = resolve_kernel<F, TS>;
-  if ((e = cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes))) !=
-      cudaSuccess)
-    return e;
+  if ((e = allow_smem(kr)) != cudaSuccess) return e;
   kr<<<1, 32 * s.wpb, bytes, st>>>(j, s.cpw, t0, S, r);
   auto kp = prefix_kernel<F, TS>;
-  if ((e = cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pbytes))) !=
-      cudaSuccess)
-    return e;
+  if ((e = allow_smem(kp)) != cudaSuccess) return e;
   if ((e = join_prefix_list(j, st)) != cudaSuccess) return e;
   if ((e = join_reset_queue(j, st)) != cudaSuccess) return e;
   const unsigned grid_pre = static_cast<unsigned>(

@@ -463,11 +463,6 @@ __global__ void __launch_bounds__(128) kept_resolve_kernel(const DevJob j, const
 }
 
 // ------------------------------------------------------------------ host side
-template <class K>
-inline cudaError_t kept_attr(K kern, size_t bytes) {
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
-}
-
 // Warps a block of a pass over so many items: the passes wait on each warp's
 // own chain of operations, so what counts is the warps an SM holds, and a
 // block's warps share one copy of the level weights (64 KiB at L = 128).  From
@@ -502,8 +497,8 @@ inline cudaError_t launch_join_kept(const DevJob& j, const LaunchShape& s, int64
   const LaunchShape all = kept_shape(j, s, items), one = kept_shape(j, s, j.p);   // all segments; one a chain
   const size_t bytes = plan_bytes(j.L, s, false, true), all_bytes = plan_bytes(j.L, all, false, true),
                one_bytes = plan_bytes(j.L, one, false, true);
-  if ((e = kept_attr(kq, std::max(all_bytes, one_bytes))) != cudaSuccess || (e = kept_attr(kh, all_bytes)) != cudaSuccess ||
-      (e = kept_attr(kc, all_bytes)) != cudaSuccess || (e = kept_attr(kr, bytes)) != cudaSuccess)
+  if ((e = allow_smem(kq)) != cudaSuccess || (e = allow_smem(kh)) != cudaSuccess || (e = allow_smem(kc)) != cudaSuccess ||
+      (e = allow_smem(kr)) != cudaSuccess)
     return e;
   const auto grid = [&](auto kern, const LaunchShape& t, size_t b, long long n) {
     return static_cast<unsigned>(std::max<long long>(

@@ -4,6 +4,8 @@
 // (Sec. 3.1 Eq. new_weight in logarithms, Sec. 4.2).
 #include <atomic>
 #include <algorithm>
+#include <mutex>
+#include <unordered_map>
 #include <math_constants.h>
 
 #include "mc_launch.cuh"
@@ -17,6 +19,29 @@ namespace mcgpu {
 static std::atomic<uint64_t> g_launches{0};
 uint64_t launches_add(uint64_t n) { return g_launches.fetch_add(n) + n; }
 
+// (set again at each use: another's cudaDeviceReset puts it back to the default)
+cudaError_t allow_smem(const void* kernel) {
+  static std::mutex mu;
+  static std::unordered_map<const void*, int> limits;   // a block's most less the kernel's own variables
+  int bytes = 0;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    const auto it = limits.find(kernel);
+    if (it != limits.end()) bytes = it->second;
+  }
+  if (bytes == 0) {
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess) return e;
+    bytes = static_cast<int>(kMaxSmem - a.sharedSizeBytes);
+    std::lock_guard<std::mutex> lk(mu);
+    try {
+      limits[kernel] = bytes;
+    } catch (...) {   // (no memory: asked for again next time)
+    }
+  }
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
 
 // ------------------------------------------------------------------ init
 // Step 1: C_1 all up, or random: bit (site & 31) of Philox word q & 3 at
@@ -1447,7 +1472,7 @@ cudaError_t k_generate_attempts(const DevJob& j, uint64_t t0, int64_t n, bool re
   const bool ts = lat + table <= kMaxSmem;
   auto kern = ts ? attempts_kernel<true> : attempts_kernel<false>;
   const size_t bytes = lat + (ts ? table : 0);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  const cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   kern<<<blocks_for(j.p, 32), 32, bytes, st>>>(j, t0, n, record ? j.plv : nullptr);
   launches_add(1);
@@ -1870,7 +1895,7 @@ cudaError_t k_thermo(const DevJob& j, int n, double* buf, cudaStream_t st) {
   const bool own = j.np1 <= 1025 && n <= 304;
   const int bytes = (own ? 12 : 8) * j.np1;
   auto kern = own ? thermo_kernel<true> : thermo_kernel<false>;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  const cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   if (!own) thermo_norm_kernel<<<kThermoParts, kThermoThreads, 0, st>>>(j, norm, neg);
   kern<<<n, kThermoThreads, bytes, st>>>(j, buf, norm, neg, buf + n);

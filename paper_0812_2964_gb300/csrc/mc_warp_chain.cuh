@@ -856,7 +856,7 @@ inline cudaError_t launch_warp_rows(const DevJob& j, int warps, bool ts, uint64_
   if (j.rec) kern = ts ? warp_gen_kernel<Rows, L, true, kKeepLevels> : warp_gen_kernel<Rows, L, false, kKeepLevels>;
   else if (j.flips) kern = ts ? warp_gen_kernel<Rows, L, true, kKeepFlips> : warp_gen_kernel<Rows, L, false, kKeepFlips>;
   const size_t bytes = 4ull * warp_plan(L, warps, ts).total;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  const cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   kern<<<blocks_for(j.p, warps), 32 * warps, bytes, st>>>(j, t0, S, warp_flush_sweeps(warps, j.N, S), trace ? 1 : 0);
   launches_add(1);
