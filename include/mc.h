@@ -118,10 +118,12 @@ int mc_run_attempts(mc_job *job, int64_t n_attempts);
  * from checkpoints (performance and memory only: both give the serial
  * rule's result).  The default is 2^33 (16 GiB of record); max_samples < 0
  * restores it, 0 turns the record off.  The record holds p rounded up to a
- * multiple of 32 chains.  At the default, larger rounds of up to 2^36 samples
- * keep their accepted flips instead, one bit a sample (at most 8 GiB; where
- * that cannot be allocated the round is replayed), from which the joint
- * rebuilds the levels; any other limit turns that off too.
+ * multiple of 32 chains.  At the default, larger rounds whose accepted flips
+ * take at most 8 GiB keep those instead -- one bit a sample, every lattice row
+ * padded to whole 32-bit words: up to 2^36 samples where L is a multiple of
+ * 32, 2^34 at L = 8 -- and the joint rebuilds the levels from them (where they
+ * cannot be allocated the round is replayed); any other limit turns that off
+ * too.
  * Fused rounds of mc_batch_run are not recorded.  MC_ESTATE while a round
  * is pending. */
 int mc_set_round_record(mc_job *job, int64_t max_samples);

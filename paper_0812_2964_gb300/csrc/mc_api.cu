@@ -354,11 +354,12 @@ void round_segments(int L, int p, int64_t n_sweeps, int64_t target, int* K, int*
 
 // Words of the flip record of a round, 0 if it keeps none: rounds too large
 // for the record of levels (where that is not limited by mc_set_round_record)
-// up to kFlipMax samples.
+// up to kFlipWordsMax words.
 size_t flip_record_words(int L, int p, int64_t n_sweeps, long long rec_max) {
   const long long samples = static_cast<long long>(p) * n_sweeps * L * L;
-  if (rec_max != mcgpu::default_record_max(L) || samples <= rec_max || samples > mcgpu::kFlipMax) return 0;
-  return static_cast<size_t>(p) * static_cast<size_t>(mcgpu::flip_words(L, n_sweeps));
+  if (rec_max != mcgpu::default_record_max(L) || samples <= rec_max) return 0;
+  const long long per_chain = mcgpu::flip_words(L, n_sweeps);
+  return per_chain <= mcgpu::kFlipWordsMax / p ? static_cast<size_t>(p) * static_cast<size_t>(per_chain) : 0;
 }
 
 // Bytes of the checkpoint buffers for K segments.

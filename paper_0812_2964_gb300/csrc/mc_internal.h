@@ -79,11 +79,12 @@ struct DevJob {
 __host__ __device__ inline int64_t flip_words(int L, int64_t S) {
   return (S * L * ((L + 31) / 32) + 31) / 32 * 32;
 }
-// whole-sweep rounds of more than kRecordMax samples, up to this many, keep
-// their flips (at most 8 GiB): iterations with chains that reject, measured
-// at 1.7e10 samples, L = 32 173 -> 52 ms and L = 64 253 -> 124 ms against
-// replaying from checkpoints
-constexpr long long kFlipMax = 1ll << 36;
+// whole-sweep rounds of more than kRecordMax samples keep their flips where
+// these take at most this many words (8 GiB: 2^36 samples where L is a
+// multiple of 32, fewer where a row's last word is not full, 2^34 at L = 8):
+// iterations with chains that reject, measured at 1.7e10 samples, L = 32
+// 173 -> 52 ms and L = 64 253 -> 124 ms against replaying from checkpoints
+constexpr long long kFlipWordsMax = 1ll << 31;
 
 // Round record layout: chains in tiles of 32; inside a tile, each group of
 // four consecutive samples of the 32 chains lies side by side, so that a warp
