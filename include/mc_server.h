@@ -48,7 +48,7 @@ typedef struct mc_jobstats {
   double t_done;
   int64_t attempts;     /* n_chains * iterations * sweeps * N */
   int64_t joined;       /* kept samples over all iterations */
-  uint64_t device_bytes;/* device memory the job held */
+  uint64_t device_bytes;/* device memory the job held (at most) */
 } mc_jobstats;
 
 typedef struct mc_server_info {
@@ -59,8 +59,11 @@ typedef struct mc_server_info {
   uint64_t admitted, completed;
 } mc_server_info;
 
-/* Device memory a job of this shape holds while resident (what admission
- * charges against the budget), trace off. */
+/* Device memory a job of this shape holds while resident, trace off.  Admission
+ * charges it against the budget, but for the flips that very large rounds
+ * keep (mc_set_round_record): a job has those only while the budget has room
+ * for them beside every job that waits, and its rounds are replayed without
+ * (the same results). */
 uint64_t mc_job_device_bytes(int L, int n_chains, int64_t sweeps);
 
 /* Create a server on the current device with `max_slots` (1..64) slots and
@@ -69,8 +72,8 @@ uint64_t mc_job_device_bytes(int L, int n_chains, int64_t sweeps);
 int mc_server_create(uint64_t budget_bytes, int max_slots, mc_server **out);
 
 /* Queue a job; *id identifies it in mc_server_poll / mc_server_wait.
- * MC_EINVAL for a bad spec, MC_ENOMEM if the job alone exceeds the budget,
- * MC_ESTATE after mc_server_free started. */
+ * MC_EINVAL for a bad spec, MC_ENOMEM if the job alone, without flips,
+ * exceeds the budget, MC_ESTATE after mc_server_free started. */
 int mc_server_submit(mc_server *srv, const mc_jobspec *spec, uint64_t *id);
 
 /* *done = 1 when the job has finished (successfully or not). MC_EINVAL for

@@ -70,6 +70,7 @@ struct mc_job {
   long long rec_max = 0;                         // largest p * M recorded (set by mc_init)
   uint32_t* flip_buf = nullptr; // flips of larger rounds (d.flips points here when used)
   size_t flip_cap = 0;          // words of flip_buf
+  bool no_flips = false;        // set by job_drop_flips
   bool pending = false;
   bool trace_on = false;
   bool trace_valid = false;
@@ -365,22 +366,26 @@ size_t flip_record_words(int L, int p, int64_t n_sweeps, long long rec_max) {
 // Bytes of the checkpoint buffers for K segments.
 size_t segment_bytes(const mc_job* job, int K) { return static_cast<size_t>(K) * bytes_per_segment(job->L, job->p); }
 
+void free_segments(mc_job* job) {
+  DevJob& d = job->d;
+  if (!d.ckpt) return;
+  raw_free(job, d.ckpt);
+  raw_free(job, d.ckm);
+  raw_free(job, d.plist);
+  job->bytes -= segment_bytes(job, d.kcap);
+  d.ckpt = nullptr;
+  d.ckm = nullptr;
+  d.plist = nullptr;
+  d.kcap = 0;
+}
+
 // Checkpoint buffers for at least K segments.
 int ensure_segments(mc_job* job, int K) {
   DevJob& d = job->d;
   if (K <= d.kcap && d.ckpt) return MC_OK;
   const size_t lw = static_cast<size_t>(job->L) * job->wd;
   const size_t p = static_cast<size_t>(job->p);
-  if (d.ckpt) {
-    raw_free(job, d.ckpt);
-    raw_free(job, d.ckm);
-    raw_free(job, d.plist);
-    job->bytes -= segment_bytes(job, d.kcap);
-    d.ckpt = nullptr;
-    d.ckm = nullptr;
-    d.plist = nullptr;
-    d.kcap = 0;
-  }
+  free_segments(job);
   void *a = nullptr, *b = nullptr, *w = nullptr;
   cudaError_t e = raw_alloc(job, &a, static_cast<size_t>(K) * lw * p * 4);
   if (e == cudaSuccess) e = raw_alloc(job, &b, static_cast<size_t>(K) * p * 4);
@@ -443,19 +448,28 @@ int ensure_record(mc_job* job, int64_t M, bool allow) {
   return MC_OK;
 }
 
+void free_flips(mc_job* job) {
+  if (!job->flip_buf) return;
+  raw_free(job, job->flip_buf);
+  job->bytes -= job->flip_cap * sizeof(uint32_t);
+  job->flip_buf = nullptr;
+  job->flip_cap = 0;
+  job->d.flips = nullptr;
+}
+
+// Words of flips that a round of the job would keep.
+size_t job_flip_words(const mc_job* job, int64_t n_sweeps) {
+  return job->no_flips ? 0 : flip_record_words(job->L, job->p, n_sweeps, job->rec_max);
+}
+
 // Buffer for the round's flips; without memory for it the round is replayed.
 void ensure_flips(mc_job* job, int64_t n_sweeps, bool allow) {
   DevJob& d = job->d;
   d.flips = nullptr;
-  const size_t words = allow && !d.rec ? flip_record_words(job->L, job->p, n_sweeps, job->rec_max) : 0;
+  const size_t words = allow && !d.rec ? job_flip_words(job, n_sweeps) : 0;
   if (words == 0) return;
   if (words > job->flip_cap) {
-    if (job->flip_buf) {
-      raw_free(job, job->flip_buf);
-      job->bytes -= job->flip_cap * sizeof(uint32_t);
-      job->flip_buf = nullptr;
-      job->flip_cap = 0;
-    }
+    free_flips(job);
     void* v = nullptr;
     if (raw_alloc(job, &v, words * sizeof(uint32_t)) != cudaSuccess) {
       cudaGetLastError();   // (not an error of the call)
@@ -470,7 +484,7 @@ void ensure_flips(mc_job* job, int64_t n_sweeps, bool allow) {
 
 // Segments of the job's round: finer ones by default where it keeps its flips.
 void choose_segments(const mc_job* job, int64_t n_sweeps, bool allow_record, int* K, int* C) {
-  const bool flips = allow_record && flip_record_words(job->L, job->p, n_sweeps, job->rec_max) > 0;
+  const bool flips = allow_record && job_flip_words(job, n_sweeps) > 0;
   round_segments(job->L, job->p, n_sweeps, job->seg_samples > 0 || !flips ? job->seg_samples : flip_segment_samples(job->L), K, C);
 }
 
@@ -1475,7 +1489,7 @@ int mc_batch_shape(mc_job* job, int* placement, int* chains_per_warp, int* warps
   return mcgpu::batch_supported(job->L, s) ? 1 : 0;
 }
 
-uint64_t mc_job_device_bytes(int L, int n_chains, int64_t sweeps) {
+static uint64_t job_bytes(int L, int n_chains, int64_t sweeps, bool flips) {
   if (L < 4 || L > 128 || (L % 4) != 0 || n_chains < 1 || sweeps < 1) return 0;
   const uint64_t N = static_cast<uint64_t>(L) * L, np1 = N + 1, wd = (L + 31) / 32;
   const uint64_t p = static_cast<uint64_t>(n_chains), lw = static_cast<uint64_t>(L) * wd, lat = p * lw;
@@ -1484,7 +1498,7 @@ uint64_t mc_job_device_bytes(int L, int n_chains, int64_t sweeps) {
   uint64_t b = lat * 4 * 2 + p * 4 * 2 + np1 * 8 + 5 * np1 * 4 + np1 * 8 * 3 + p * 8 + p * 4 + p * np1 * 4 +
                p * 8 + p * 4 + p * 4 + p * 4 + p * 20 + np1 + p * 4 + np1 * 4 + p * 8 + mcgpu::kStatCount * 8;
   int K = 0, C = 0;
-  const size_t flip_words = flip_record_words(L, n_chains, sweeps, mcgpu::default_record_max(L));
+  const size_t flip_words = flips ? flip_record_words(L, n_chains, sweeps, mcgpu::default_record_max(L)) : 0;
   round_segments(L, n_chains, sweeps, flip_words ? flip_segment_samples(L) : 0, &K, &C);
   (void)lw;
   const uint64_t samples = p * static_cast<uint64_t>(sweeps) * N;   // record of the round, if small
@@ -1494,9 +1508,24 @@ uint64_t mc_job_device_bytes(int L, int n_chains, int64_t sweeps) {
   return b + static_cast<uint64_t>(K) * bytes_per_segment(L, n_chains) + rec + 4ull * flip_words;
 }
 
+uint64_t mc_job_device_bytes(int L, int n_chains, int64_t sweeps) { return job_bytes(L, n_chains, sweeps, true); }
+
 int mc_sync(mc_job* job) {
   if (int rc = check_job(job)) return rc;
   return sync(job, "sync");
 }
 
 }  // extern "C"
+
+uint64_t mcgpu::job_bytes_without_flips(int L, int n_chains, int64_t sweeps) {
+  return job_bytes(L, n_chains, sweeps, false);
+}
+
+int mcgpu::job_drop_flips(mc_job* job) {
+  if (job->pending) return fail(MC_ESTATE, "round pending");
+  if (int rc = sync(job, "drop flips")) return rc;
+  job->no_flips = true;
+  free_flips(job);
+  free_segments(job);
+  return MC_OK;
+}

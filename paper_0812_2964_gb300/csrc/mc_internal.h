@@ -5,6 +5,8 @@
 
 #include <cuda_runtime.h>
 
+struct mc_job;
+
 namespace mcgpu {
 
 // Lattice placement of a chain during a sweep.
@@ -243,6 +245,13 @@ MC_WARP_UNIT(chain_kernels_warp_4b);
 cudaError_t chain_kernels_record(const DevJob& j, int64_t S, uint32_t r, cudaStream_t st);
 // the joint of a round that kept its flips
 cudaError_t chain_kernels_flips(const DevJob& j, int64_t S, uint32_t r, cudaStream_t st);
+
+// mc_job_device_bytes of a job whose rounds keep no flips
+uint64_t job_bytes_without_flips(int L, int n_chains, int64_t sweeps);
+// From now on the job's rounds keep no flips (one too large for the record of
+// levels is replayed); what the flips and their finer checkpoints took is
+// given back.  Synchronises; no round may be pending.
+int job_drop_flips(mc_job* job);
 
 // launch shape chosen by default for (L, p)
 LaunchShape default_shape(int L, int p, int num_sms);

@@ -4,6 +4,11 @@
 // job at most two weight iterations ahead of the GPU, and collects jobs
 // as they finish.  Each job is driven only through the mc.h calls on its
 // slot's stream, so its results are those of the same job run alone.
+//
+// The flips that a job with very large rounds keeps for its joint are no part
+// of what it needs (without them the rounds are replayed): they take only
+// room in the budget that no waiting job wants, and are given back, between
+// two iterations, for one that comes later.
 #include <algorithm>
 #include <chrono>
 #include <condition_variable>
@@ -35,7 +40,10 @@ struct Rec {
   int slot = -1;
   int it_enq = 0, it_done = 0;
   double t_submit = 0, t_admit = 0, t_done = 0;
-  uint64_t bytes = 0;
+  uint64_t need = 0, full = 0;    // without and with the flips its rounds would keep
+  uint64_t bytes = 0, most = 0;   // charged now, and at most so far
+  bool flips = false;             // runs with them
+  bool give_up = false;           // asked to give them back
   int status = MC_OK;
   std::string err;
   std::vector<double> W;
@@ -91,6 +99,24 @@ void finish_locked(mc_server* srv, Rec* r) {
   srv->cv_done.notify_all();
 }
 
+// Called with the lock held: a job that waits needs `missing` more bytes.  Where
+// flips of running jobs would make up for it, ask for as many back.
+void ask_flips_back(mc_server* srv, uint64_t missing) {
+  const auto can = [](const Slot& sl) {
+    return sl.rec && sl.rec->job && sl.rec->flips && sl.rec->it_enq < sl.rec->spec.iterations;
+  };
+  uint64_t sum = 0;
+  for (const auto& sl : srv->slots)
+    if (can(sl)) sum += sl.rec->bytes - sl.rec->need;
+  if (sum < missing) return;
+  for (auto& sl : srv->slots) {
+    if (missing == 0) break;
+    if (!can(sl)) continue;
+    sl.rec->give_up = true;
+    missing -= std::min(missing, sl.rec->bytes - sl.rec->need);
+  }
+}
+
 // Without the lock: create the job's device state on its slot's stream.
 int admit_job(mc_server* srv, Rec* r) {
   const mc_jobspec& s = r->spec;
@@ -102,6 +128,7 @@ int admit_job(mc_server* srv, Rec* r) {
     const mcgpu::LaunchShape d = mcgpu::dense_shape(s.L, s.n_chains, srv->num_sms);
     rc = mc_set_launch_shape(j, d.placement, d.cpw, d.wpb);
   }
+  if (rc == MC_OK && !r->flips) rc = mcgpu::job_drop_flips(j);
   if (rc != MC_OK) {
     r->err = mc_last_error();
     if (j) mc_free(j);
@@ -150,6 +177,8 @@ void worker_main(mc_server* srv) {
     bool progressed = false;
     // admission: first fit in arrival order
     std::vector<Rec*> admit;
+    uint64_t waiting = 0;   // what the queue needs
+    for (const Rec* r : srv->queue) waiting += r->need;
     for (auto it = srv->queue.begin(); it != srv->queue.end();) {
       Rec* r = *it;
       int free_slot = -1;
@@ -159,10 +188,14 @@ void worker_main(mc_server* srv) {
           break;
         }
       if (free_slot < 0) break;
-      if (srv->in_use + r->bytes > srv->budget) {
+      r->flips = r->full > r->need && srv->in_use + r->full + (waiting - r->need) <= srv->budget;
+      if (!r->flips && srv->in_use + r->need > srv->budget) {
+        ask_flips_back(srv, srv->in_use + r->need - srv->budget);
         ++it;
         continue;
       }
+      waiting -= r->need;
+      r->bytes = r->most = r->flips ? r->full : r->need;
       r->slot = free_slot;
       r->state = State::Active;
       r->t_admit = srv->now();
@@ -181,6 +214,7 @@ void worker_main(mc_server* srv) {
     lk.unlock();
 
     std::vector<std::pair<Rec*, int>> ended;
+    std::vector<Rec*> given;   // gave their flips back
     for (Rec* r : admit) {
       const int rc = admit_job(srv, r);
       progressed = true;
@@ -201,7 +235,13 @@ void worker_main(mc_server* srv) {
         r->it_done += 1;
         progressed = true;
       }
-      while (rc == MC_OK && r->it_enq < r->spec.iterations && r->it_enq - r->it_done < kAhead) {
+      if (rc == MC_OK && r->give_up && r->it_done == r->it_enq) {   // (nothing of it is queued)
+        r->give_up = false;
+        if (r->it_enq < r->spec.iterations && (rc = mcgpu::job_drop_flips(r->job)) == MC_OK) given.push_back(r);
+        else if (rc != MC_OK) r->err = mc_last_error();
+        progressed = true;
+      }
+      while (rc == MC_OK && !r->give_up && r->it_enq < r->spec.iterations && r->it_enq - r->it_done < kAhead) {
         rc = enqueue_iteration(srv, r);
         if (rc == MC_OK) r->it_enq += 1;
         progressed = true;
@@ -220,6 +260,11 @@ void worker_main(mc_server* srv) {
     }
 
     lk.lock();
+    for (Rec* r : given) {
+      srv->in_use -= r->bytes - r->need;
+      r->bytes = r->need;
+      r->flips = false;
+    }
     for (auto& e : ended) {
       e.first->status = e.second;
       finish_locked(srv, e.first);
@@ -284,10 +329,11 @@ int mc_server_submit(mc_server* srv, const mc_jobspec* spec, uint64_t* id) {
     mcgpu::set_last_error("mc_server_submit: bad job spec");
     return MC_EINVAL;
   }
-  const uint64_t bytes = mc_job_device_bytes(spec->L, spec->n_chains, spec->sweeps);
+  const uint64_t full = mc_job_device_bytes(spec->L, spec->n_chains, spec->sweeps);
+  const uint64_t need = std::min(full, mcgpu::job_bytes_without_flips(spec->L, spec->n_chains, spec->sweeps));
   std::lock_guard<std::mutex> lk(srv->mu);
   if (srv->stopping) return MC_ESTATE;
-  if (bytes > srv->budget) {
+  if (need > srv->budget) {
     mcgpu::set_last_error("mc_server_submit: the job alone exceeds the device-memory budget");
     return MC_ENOMEM;
   }
@@ -295,7 +341,8 @@ int mc_server_submit(mc_server* srv, const mc_jobspec* spec, uint64_t* id) {
   if (!r) return MC_ENOMEM;
   r->id = srv->next_id++;
   r->spec = *spec;
-  r->bytes = bytes;
+  r->need = need;
+  r->full = full;
   r->t_submit = srv->now();
   *id = r->id;
   try {
@@ -343,7 +390,7 @@ int mc_server_wait(mc_server* srv, uint64_t id, double* W_out, int n, mc_jobstat
     stats->t_done = r->t_done;
     stats->attempts = static_cast<int64_t>(r->spec.n_chains) * r->spec.iterations * r->spec.sweeps * N;
     stats->joined = r->joined;
-    stats->device_bytes = r->bytes;
+    stats->device_bytes = r->most;
   }
   const int status = r->status;
   if (status != MC_OK) mcgpu::set_last_error(r->err.c_str());

@@ -1,0 +1,77 @@
+"""Memory that a call can do without does not make it fail: a record that
+cannot be had leaves the round to the replaying joint, with the same
+results.  (Allocation failures are injected on the host, before any CUDA call.)
+"""
+import time
+
+import numpy as np
+import pytest
+
+import paper_0812_2964_gb300 as mc
+from paper_0812_2964_gb300.workloads import random_weights
+
+pytestmark = pytest.mark.gpu
+
+MIB = 2 ** 20
+BIG = (32, 8200, 1030)          # L, chains, sweeps: just too large for the record of levels
+BIG_FLIPS = 4 * 8200 * 1030 * 32
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    mc.build()
+    yield
+    mc.mc_inject_alloc_failure(-1)
+
+
+def _alone(L, p, seed, iters, S, replay=False):
+    g = mc.Job(L, p, seed, 1)
+    if replay:
+        g.set_round_record(0)
+    for _ in range(iters):
+        g.run_sweeps(S)
+        g.join()
+        g.update_weights()
+    W = g.weights
+    g.close()
+    return W
+
+
+# ------------------------------------------------------------------ serving
+def test_server_runs_a_large_round_without_room_for_its_flips():
+    L, p, S = BIG
+    budget = mc.mc_job_device_bytes(L, p, S) - BIG_FLIPS
+    with mc.Server(budget, max_slots=2) as srv:
+        W, st = srv.wait(srv.submit(L, p, 81, 2, S))
+        assert srv.info()["peak_bytes"] <= budget
+    assert st["status"] == mc.MC_OK and st["device_bytes"] <= budget
+    assert np.array_equal(W, _alone(L, p, 81, 2, S, replay=True))
+
+
+def test_server_takes_flips_back_for_a_job_that_waits():
+    L, p, S = BIG
+    small = (64, 500, 82, 2, 3)
+    budget = mc.mc_job_device_bytes(L, p, S) + MIB       # room for the large job whole, not for both
+    assert mc.mc_job_device_bytes(64, 500, 3) > MIB
+    with mc.Server(budget, max_slots=2) as srv:
+        a = srv.submit(L, p, 83, 12, S)
+        deadline = time.monotonic() + 60
+        while srv.info()["bytes_in_use"] < mc.mc_job_device_bytes(L, p, S) and time.monotonic() < deadline:
+            time.sleep(0.001)
+        assert srv.info()["bytes_in_use"] == mc.mc_job_device_bytes(L, p, S)
+        b = srv.submit(*small)
+        Wb, stb = srv.wait(b)
+        Wa, sta = srv.wait(a)
+        assert srv.info()["peak_bytes"] <= budget and srv.info()["bytes_in_use"] == 0
+    assert stb["t_admit"] < sta["t_done"]                # it did not wait for the large job's end
+    assert np.array_equal(Wb, _alone(*small))
+    assert np.array_equal(Wa, _alone(L, p, 83, 12, S, replay=True))
+
+
+def test_server_keeps_flips_where_there_is_room():
+    L, p, S = BIG
+    need = mc.mc_job_device_bytes(L, p, S)
+    with mc.Server(2 * need, max_slots=2) as srv:
+        W, st = srv.wait(srv.submit(L, p, 84, 2, S))
+    assert st["device_bytes"] == need
+    assert np.array_equal(W, _alone(L, p, 84, 2, S))
