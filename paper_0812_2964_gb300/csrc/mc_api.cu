@@ -488,6 +488,20 @@ void choose_segments(const mc_job* job, int64_t n_sweeps, bool allow_record, int
   round_segments(job->L, job->p, n_sweeps, job->seg_samples > 0 || !flips ? job->seg_samples : flip_segment_samples(job->L), K, C);
 }
 
+// Checkpoint buffers for a round that may keep its samples if *keep.  Where
+// there is no memory for the finer segments of one that keeps its flips, *keep
+// is cleared and the round takes a replayed one's.
+int prepare_segments(mc_job* job, int64_t n_sweeps, bool* keep, int* K, int* C) {
+  choose_segments(job, n_sweeps, *keep, K, C);
+  const int rc = ensure_segments(job, *K);
+  if (rc != MC_ENOMEM || !*keep || job_flip_words(job, n_sweeps) == 0) return rc;
+  cudaGetLastError();   // (not an error of the call)
+  g_err.clear();
+  *keep = false;
+  choose_segments(job, n_sweeps, false, K, C);
+  return ensure_segments(job, *K);
+}
+
 // The round's record (of levels or flips) for a batch, where there is memory
 // for it; false: the round is replayed.
 bool ensure_kept(mc_job* job, int64_t n_sweeps) {
@@ -514,8 +528,7 @@ int round_prepare(mc_job* job, int64_t n_sweeps, uint64_t* t0, bool allow_record
   if (job->trace_on)
     if (int rc = ensure_trace(job, n_sweeps)) return rc;
   int K = 0, C = 0;
-  choose_segments(job, n_sweeps, allow_record, &K, &C);
-  if (int rc = ensure_segments(job, K)) return rc;
+  if (int rc = prepare_segments(job, n_sweeps, &allow_record, &K, &C)) return rc;
   if (int rc = ensure_record(job, M, allow_record)) return rc;
   ensure_flips(job, n_sweeps, allow_record);
   DevJob& d = job->d;

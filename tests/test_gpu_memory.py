@@ -37,6 +37,31 @@ def _alone(L, p, seed, iters, S, replay=False):
     return W
 
 
+# ------------------------------------------------------------------ one job
+@pytest.mark.parametrize("after", [0, 1, 2, 3])
+def test_flip_rounds_fall_back_to_replays(after):
+    # 0..2: the checkpoints that rebuilding from flips wants, 3: the flips themselves
+    L, p, S = BIG
+    W = random_weights(L, 3, 1.0)
+    out = []
+    for replay in (False, True):
+        g = mc.Job(L, p, 71, 1)
+        g.weights = W
+        if replay:
+            g.set_round_record(0)
+        else:
+            mc.mc_inject_alloc_failure(after)
+        g.run_sweeps(S)
+        mc.mc_inject_alloc_failure(-1)
+        kept = g.join()
+        out.append((kept, g.hist, g.k, g.energies))
+        if not replay:
+            assert g.info()["device_bytes"] < mc.mc_job_device_bytes(L, p, S)    # (the flips are not there)
+        g.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
 # ------------------------------------------------------------------ serving
 def test_server_runs_a_large_round_without_room_for_its_flips():
     L, p, S = BIG
