@@ -761,12 +761,19 @@ static int mc_batch_run_impl(mc_job** jobs, int n_jobs, int iterations, int64_t 
   for (int i = 0; i < n_jobs; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return jobs[a]->N > jobs[b]->N; });
   int rc = MC_OK;
-  for (int i = 0; i < n_jobs && rc == MC_OK; ++i) {  // no allocation inside a capture
+  // No allocation inside a capture: first what every job cannot do without,
+  // then what its rounds may keep, where there is memory left.
+  for (int i = 0; i < n_jobs && rc == MC_OK; ++i) {
     if (jobs[i]->trace_on) rc = ensure_trace(jobs[i], n_sweeps);
+    bool keep = false;
     int K = 0, C = 0;
-    choose_segments(jobs[i], n_sweeps, !fused[i], &K, &C);
-    if (rc == MC_OK) rc = ensure_segments(jobs[i], K);
-    keeps[i] = !fused[i] && rc == MC_OK && ensure_kept(jobs[i], n_sweeps);
+    if (rc == MC_OK) rc = prepare_segments(jobs[i], n_sweeps, &keep, &K, &C);
+  }
+  for (int i = 0; i < n_jobs && rc == MC_OK; ++i) {
+    bool keep = !fused[i];
+    int K = 0, C = 0;
+    if (keep) rc = prepare_segments(jobs[i], n_sweeps, &keep, &K, &C);
+    keeps[i] = keep && rc == MC_OK && ensure_kept(jobs[i], n_sweeps);
   }
   std::vector<cudaEvent_t> done(n_jobs, nullptr);
   cudaEvent_t fork = nullptr;

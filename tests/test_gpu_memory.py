@@ -62,6 +62,40 @@ def test_flip_rounds_fall_back_to_replays(after):
         assert np.array_equal(a, b)
 
 
+# ------------------------------------------------------------------ batches
+BATCH = [(8, 40, 11), (16, 70, 12), (20, 50, 13)]      # L, chains, seed
+
+
+@pytest.mark.parametrize("mode", [0, 2])
+@pytest.mark.parametrize("after", [9, 10, 11])
+def test_batch_records_come_after_what_every_job_needs(mode, after):
+    # three checkpoint buffers a job first, then a record a job: a record that fails is done without
+    live0 = mc.mc_live_allocations()
+    js = [mc.Job(L, p, seed, 1) for L, p, seed in BATCH]
+    mc.mc_inject_alloc_failure(after)
+    mc.mc_batch_run(js, 2, 5, mode)
+    mc.mc_inject_alloc_failure(-1)
+    for j, (L, p, seed) in zip(js, BATCH):
+        assert np.array_equal(j.weights, _alone(L, p, seed, 2, 5))
+        j.close()
+    assert mc.mc_live_allocations() == live0
+
+
+@pytest.mark.parametrize("mode", [0, 2])
+@pytest.mark.parametrize("after", [3, 5, 8])
+def test_batch_reports_what_it_cannot_do_without(mode, after):
+    js = [mc.Job(L, p, seed, 1) for L, p, seed in BATCH]
+    mc.mc_inject_alloc_failure(after)
+    with pytest.raises(mc.McError) as e:
+        mc.mc_batch_run(js, 2, 5, mode)
+    mc.mc_inject_alloc_failure(-1)
+    assert e.value.code == mc.MC_ENOMEM
+    mc.mc_batch_run(js, 2, 5, mode)                      # and the next call works
+    for j, (L, p, seed) in zip(js, BATCH):
+        assert np.array_equal(j.weights, _alone(L, p, seed, 2, 5))
+        j.close()
+
+
 # ------------------------------------------------------------------ serving
 def test_server_runs_a_large_round_without_room_for_its_flips():
     L, p, S = BIG
