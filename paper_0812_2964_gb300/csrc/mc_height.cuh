@@ -54,7 +54,20 @@ __device__ __forceinline__ Height* heights(const DevJob& j) { return reinterpret
 
 // The levels' weights (W[m] - Wref) / ln 2, built at the start of the joint
 // in the scratch of the energy ordering; Wref is the weight of a level that
-// the round met.
+// the round met.  A grown job's lie within 2^15 of it; the floats of weights
+// further away than kWeightSpan (levels masked by a huge value) would be too
+// coarse, or infinite.  As a sample's weight they are replaced by bounds from
+// above, infinity or kWeightLow, as the input's by bounds from below: the
+// filters then let such samples through, the second-best v stays an upper
+// estimate, and the answers are the exact test's, or undecided.
+constexpr float kWeightSpan = 1048576.0f;
+constexpr float kWeightLow = 1.0f - kWeightSpan;   // (1 above: more than the rounding of sums with it)
+__device__ __forceinline__ float level_weight(float v) {
+  return v > kWeightSpan ? __int_as_float(0x7F800000) : (v >= -kWeightSpan ? v : kWeightLow);
+}
+__device__ __forceinline__ float input_weight(float level) {
+  return level == kWeightLow ? __int_as_float(static_cast<int>(0xFF800000)) : fminf(level, kWeightSpan);
+}
 __device__ __forceinline__ float* level_weights(const DevJob& j) { return reinterpret_cast<float*>(j.lvcnt); }
 __device__ __forceinline__ double reference_weight(const DevJob& j) { return j.W[j.m[0]]; }
 

@@ -160,7 +160,7 @@ __device__ __forceinline__ void kept_test_setup(const DevJob& j, TestHook& hk, c
   hk.wl = wl;
   hk.W = j.W;
   hk.wx = j.W[x];
-  hk.bl = level_weights(j)[x] - slack;
+  hk.bl = input_weight(level_weights(j)[x]) - slack;
   hk.k = k;
   hk.kw = k;
   hk.found = 0;

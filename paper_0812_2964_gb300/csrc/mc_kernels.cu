@@ -859,8 +859,8 @@ __global__ void kept_prelude_kernel(const DevJob j) {
   float big = 0.0f;
   for (int m = t; m < j.np1; m += nt) {
     const float v = static_cast<float>((j.W[m] - wref) * 1.4426950408889634);
-    wl[m] = v;
-    if (fabsf(v) < CUDART_INF_F) big = fmaxf(big, fabsf(v));
+    wl[m] = level_weight(v);
+    if (fabsf(v) <= kWeightSpan) big = fmaxf(big, fabsf(v));
   }
   // (0 before: finalize_kernel clears it)
   if (big > 0.0f) atomicMax(&j.stats[kStatWeightMax], static_cast<long long>(__float_as_int(big)));

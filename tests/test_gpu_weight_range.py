@@ -1,0 +1,116 @@
+"""Weights far outside a grown job's range: the joints of kept rounds give what
+the replaying joint gives when weights mask levels with huge values, when a
+level no chain visits carries one, and when whole ranges are lifted."""
+import numpy as np
+import pytest
+
+import paper_0812_2964_gb300 as mc
+from paper_0812_2964_gb300.workloads import random_weights
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    mc.build()
+
+
+def _rows(up):
+    """bool [p][L][L], L <= 32 -> the job's words."""
+    p, L, _ = up.shape
+    return (up.astype(np.uint32) << np.arange(L, dtype=np.uint32)).sum(2, dtype=np.uint32).reshape(-1)
+
+
+def _same(a, b):
+    for x, y in zip(a, b):
+        for u, v in zip(x, y):
+            assert np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("mask", [-1e30, -1e300, -8.9e307])
+def test_masked_levels(mask):
+    # two masks, the deeper one on the antiferromagnetic side: chains that start below the first and above the
+    # second stay there (every move among equal weights is taken: one wall sweeps through the lattice, at most
+    # 9 of 64 levels from the end), and the round's input is a masked level while chain 0 is not
+    L, p = 8, 96
+    N = L * L
+    W = random_weights(L, 5, 0.5)
+    W[:12], W[53:] = mask, 2 * mask
+    stripes = np.add.outer(np.arange(L), np.arange(L)) % 2 == 0
+    up = np.ones((p, L, L), bool)
+    up[p // 2:-1] = stripes
+    mixed = np.random.default_rng(1).random((L, L)) < 0.5
+
+    def run(replay):
+        g = mc.Job(L, p, 9, 0)
+        if replay:
+            g.set_round_record(0)
+        g.weights = W
+        g.spin_words = _rows(up)
+        out = []
+        for r in range(4):
+            g.run_sweeps(3)
+            kept = g.join()
+            out.append((kept, g.hist, g.k, g.energies, g.info()["carry_energy"], g.info()["last_rejected"]))
+            if r == 0:                                   # half the chains rejected: the next joint is by heights
+                assert g.info()["last_rejected"] == p // 2 - 1
+                words = g.spin_words.reshape(p, L).copy()
+                words[0] = _rows(mixed[None])
+                g.spin_words = words.reshape(-1)
+                g.set_join_order(1)
+        g.close()
+        return out
+
+    _same(run(False), run(True))
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("extra", [7.2e5, -7.2e5, 1e8, -1e12, 3e38, -1e300, np.inf, -np.inf])
+def test_a_level_nobody_visits(extra, order):
+    # level 1 does not exist on the lattice: whatever its weight, the joint is that of the other levels
+    L, p, S = 12, 1500, 4
+    W = random_weights(L, 6, 5.0)
+
+    def run(replay, w1):
+        g = mc.Job(L, p, 10, 1)
+        if replay:
+            g.set_round_record(0)
+        w = W.copy()
+        w[1] = w1
+        g.weights = w
+        g.set_join_order(order)
+        out = []
+        for _ in range(4):
+            g.run_sweeps(S)
+            out.append((g.join(), g.hist, g.k, g.offsets, g.energies, g.info()["carry_energy"]))
+        g.close()
+        return out
+
+    want = run(True, extra)
+    _same(run(False, extra), want)
+    _same(run(True, 0.0), want)
+
+
+@pytest.mark.parametrize("attempts", [False, True])
+@pytest.mark.parametrize("lift", [1e6, 1e9, -1e9])
+def test_levels_lifted_out_of_the_filters_range(lift, attempts):
+    # half the levels far above (below) the level that the heights are measured against, with the usual
+    # differences among themselves: answers come from the exact test alone
+    L, p = 12, 700
+    W = random_weights(L, 7, 4.0)
+    W[L * L // 2:] += lift
+
+    def run(fast):
+        g = mc.Job(L, p, 11, 1)
+        if not fast:
+            g.set_round_record(0)
+            g.set_partial_record(0)
+        g.weights = W
+        out = []
+        for _ in range(4):
+            g.run_attempts(70) if attempts else g.run_sweeps(2)
+            out.append((g.join(), g.hist, g.k, g.offsets, g.energies, g.info()["carry_energy"]))
+        g.close()
+        return out
+
+    _same(run(True), run(False))
