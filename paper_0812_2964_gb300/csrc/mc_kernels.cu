@@ -968,13 +968,13 @@ __device__ __forceinline__ void height_values(const DevJob& j, int block, int bl
   const int f = static_cast<int>(j.stats[kStatFirstPending]);
   const int t = threadIdx.x;
   const double wref = reference_weight(j);
-  const float slack = height_slack(j);
+  const float error = height_error(j);
   for (int base = block * 1024; base < j.p; base += blocks * 1024) {
     const int q = base + t;
     double v = -CUDART_INF;
     if (q >= f && q < j.p) {
       const Height h = heights(j)[j.perm[q]];
-      v = fmax(height_value(j, h), height_second(h, wref, slack));
+      v = fmax(height_value(j, h), height_second(h, wref, error));
     }
     if (q < j.p) hs.val[q] = v;
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
@@ -995,7 +995,7 @@ __device__ __forceinline__ void height_values(const DevJob& j, int block, int bl
 // First position from q on whose chain keeps samples for an input level of
 // weight wx; p if none; p + 1 + q' if that is undecided at q'.
 __device__ __forceinline__ int height_next(const DevJob& j, const HeightScratch& hs, int q, double wx, double wref,
-                                           float slack) {
+                                           float error) {
   const double low = wx - (kHeightEps + 1e-13 * fabs(wx));
   while (q < j.p) {
     if ((q & 1023) == 0 && hs.max1024[q >> 10] < low) {
@@ -1007,7 +1007,7 @@ __device__ __forceinline__ int height_next(const DevJob& j, const HeightScratch&
       continue;
     }
     if (!(hs.val[q] < low)) {
-      const int a = height_accepts(j, heights(j)[j.perm[q]], wx, wref, slack);
+      const int a = height_accepts(j, heights(j)[j.perm[q]], wx, wref, error);
       if (a) return a == 1 ? q : j.p + 1 + q;
     }
     ++q;
@@ -1027,14 +1027,14 @@ __device__ __forceinline__ void height_successors(const DevJob& j, int t, int nt
   const HeightScratch hs = height_scratch(j);
   const int f = static_cast<int>(j.stats[kStatFirstPending]);
   const double wref = reference_weight(j);
-  const float slack = height_slack(j);
+  const float error = height_error(j);
   for (int q = f + t; q <= j.p; q += nt) {
     int nx;
     if (q < j.p) {
-      nx = height_next(j, hs, q + 1, j.W[j.m[j.perm[q]]], wref, slack);
+      nx = height_next(j, hs, q + 1, j.W[j.m[j.perm[q]]], wref, error);
     } else {
       const int x = height_input(j, f);
-      nx = x < 0 ? f : height_next(j, hs, f, j.W[x], wref, slack);
+      nx = x < 0 ? f : height_next(j, hs, f, j.W[x], wref, error);
     }
     hs.next[q] = nx;
   }

@@ -114,3 +114,21 @@ def test_levels_lifted_out_of_the_filters_range(lift, attempts):
         return out
 
     _same(run(True), run(False))
+
+
+def test_rough_joints_of_many_chains_are_settled_by_the_heights():
+    # every input of a joint after a rough one is the heights' answer: none is left to the pass that
+    # searches whole chains (the scan counts the chains it settled)
+    L, p = 8, 1 << 17
+    g = mc.Job(L, p, 12, 1)
+    g.weights = random_weights(L, 8, 8.0)
+    settled = []
+    for r in range(9):
+        g.run_sweeps(1)
+        g.join()
+        info = g.info()
+        assert info["last_rejected"] > p // 16
+        if r:
+            settled.append(info["last_scanned"])
+    g.close()
+    assert settled == [p] * 8
