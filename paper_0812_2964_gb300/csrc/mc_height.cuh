@@ -103,7 +103,7 @@ __device__ __forceinline__ float height_slack(const DevJob& j) { return 0.01f + 
 // Error of a second-best v: the logarithm's (within 1e-5 at up to 32, sums
 // included) and the weights'.  Where the line lies between the second best and
 // this above it, the answer is undecided and the scan ends there, so it is no
-// wider than that: with height_slack one chain in some 5 10^5 was, and what was
+// wider than that: with height_slack one chain in some 2 10^6 was, and what was
 // left of its joint (L = 8, 2^17 chains, one sweep) took 4.5 s instead of 2 ms.
 __device__ __forceinline__ float height_error(const DevJob& j) { return 1e-4f + weight_error(j); }
 

@@ -208,6 +208,7 @@ enum MarkFlags : int {
 cudaError_t kept_prelude(const DevJob& j, cudaStream_t st);
 cudaError_t kept_mark(const DevJob& j, int64_t S, int flags, cudaStream_t st);
 cudaError_t kept_scan(const DevJob& j, cudaStream_t st);
+cudaError_t kept_mark_scan(const DevJob& j, int64_t S, int flags, cudaStream_t st);   // the one, then the other
 
 // per-unit launchers of the templated chain kernels (mc_inst_*.cu)
 #define MC_CHAIN_UNIT(name)                                                                              \

@@ -540,7 +540,11 @@ inline cudaError_t launch_join_kept(const DevJob& j, const LaunchShape& s, int64
     launches_add(2);
     if ((e = kept_scan(j, st)) != cudaSuccess) return e;
     if ((e = search(1, 0)) != cudaSuccess) return e;
-    if ((e = passes(j.passes_scan, 0)) != cudaSuccess) return e;
+    if (j.passes_scan > 0) {   // the first pass goes on from an undecided chain, now searched
+      if ((e = kept_mark_scan(j, S, kMarkListed, st)) != cudaSuccess) return e;
+      if ((e = search(1, 0)) != cudaSuccess) return e;
+    }
+    if ((e = passes(j.passes_scan - 1, 0)) != cudaSuccess) return e;
   } else {
     if ((e = passes(j.passes_plain, 0)) != cudaSuccess) return e;
   }

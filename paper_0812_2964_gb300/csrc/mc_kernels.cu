@@ -871,8 +871,7 @@ __global__ void kept_prelude_kernel(const DevJob j) {
 // the one their k was found for go to work[], with the new input in xused.
 // With kMarkFinal and nothing pending: the carry, and whether fewer samples
 // are kept than discarded.
-__global__ void __launch_bounds__(1024) kept_mark_kernel(const DevJob j, const int64_t M, const int flags) {
-  after_previous();
+__device__ __forceinline__ void kept_mark_body(const DevJob& j, const int64_t M, const int flags) {
   __shared__ int s_count, s_first, s_new;
   __shared__ unsigned long long s_kept;
   const int t = threadIdx.x, nt = blockDim.x;
@@ -938,6 +937,11 @@ __global__ void __launch_bounds__(1024) kept_mark_kernel(const DevJob j, const i
   }
   __syncthreads();
   if ((flags & kMarkFinal) && s_count == 0) kept_list_counted(j);
+}
+
+__global__ void __launch_bounds__(1024) kept_mark_kernel(const DevJob j, const int64_t M, const int flags) {
+  after_previous();
+  kept_mark_body(j, M, flags);
 }
 
 // Scratch of the scan in tj (its rows are rebuilt for the chains searched
@@ -1101,6 +1105,11 @@ __device__ __forceinline__ void height_path(const DevJob& j) {
             }
             ++scanned;
           }
+        } else if (q == stop_at) {               // undecided: searched under its input, which is exact
+          j.xused[ch] = last >= 0 ? j.m[j.perm[last]] : x0;
+          j.k[ch] = -1;
+          j.kmin[ch] = kNoHit;
+          j.work[atomicAdd(&s_count, 1)] = ch;
         } else if (kc < 0) {
           j.work[atomicAdd(&s_count, 1)] = ch;   // stopped early: chains still waiting for a search keep their inputs
         }
@@ -1109,7 +1118,7 @@ __device__ __forceinline__ void height_path(const DevJob& j) {
   __syncthreads();
   if (t == 0) {
     j.stats[kStatPending] = s_count;
-    j.stats[kStatScanned] = s_scanned;
+    j.stats[kStatScanned] += s_scanned;
     j.stats[kStatNoHit] = 0;
     j.stats[kStatQueueA] = 0;
     j.stats[kStatQueueB] = 0;
@@ -1129,14 +1138,23 @@ __global__ void __launch_bounds__(1024) height_path_kernel(const DevJob j) {
   if (j.stats[kStatPending]) height_path(j);
 }
 // the three in one launch
-__global__ void __launch_bounds__(1024) height_scan_kernel(const DevJob j) {
-  after_previous();
+__device__ __forceinline__ void height_scan_body(const DevJob& j) {
   if (j.stats[kStatPending] == 0) return;
   height_values(j, 0, 1);
   __syncthreads();
   height_successors(j, threadIdx.x, blockDim.x);
   __syncthreads();
   height_path(j);
+}
+__global__ void __launch_bounds__(1024) height_scan_kernel(const DevJob j) {
+  after_previous();
+  height_scan_body(j);
+}
+__global__ void __launch_bounds__(1024) kept_mark_scan_kernel(const DevJob j, const int64_t M, const int flags) {
+  after_previous();
+  kept_mark_body(j, M, flags);
+  __syncthreads();
+  height_scan_body(j);
 }
 
 __global__ void tj_list_kernel(const DevJob j) {
@@ -1736,8 +1754,19 @@ cudaError_t kept_mark(const DevJob& j, int64_t S, int flags, cudaStream_t st) {
 }
 
 // (one block does the whole scan where its three parts are short: two launches saved)
+constexpr int kScanOneBlock = 4096;
+cudaError_t kept_mark_scan(const DevJob& j, int64_t S, int flags, cudaStream_t st) {
+  if (j.p <= kScanOneBlock) {
+    launch_next(kept_mark_scan_kernel, 1, 1024, 0, st, j, S * j.N, flags);
+    launches_add(1);
+    return cudaGetLastError();
+  }
+  const cudaError_t e = kept_mark(j, S, flags, st);
+  return e == cudaSuccess ? kept_scan(j, st) : e;
+}
+
 cudaError_t kept_scan(const DevJob& j, cudaStream_t st) {
-  if (j.p <= 4096) {
+  if (j.p <= kScanOneBlock) {
     launch_next(height_scan_kernel, 1, 1024, 0, st, j);
     launches_add(1);
     return cudaGetLastError();

@@ -132,3 +132,24 @@ def test_rough_joints_of_many_chains_are_settled_by_the_heights():
             settled.append(info["last_scanned"])
     g.close()
     assert settled == [p] * 8
+
+
+def test_an_undecided_chain_does_not_end_the_scan():
+    # the weight of a level nobody visits widens the error bound (to 0.01): of the same joints some then have an
+    # undecided chain, which is searched and the scan goes on behind it -- no pass searches whole chains
+    L, p = 8, 1 << 17
+    out, passes = [], []
+    for w1 in (0.0, 28_000.0):
+        g = mc.Job(L, p, 12, 1)
+        w = random_weights(L, 8, 8.0)
+        w[1] = w1
+        g.weights = w
+        rounds = []
+        for _ in range(9):
+            g.run_sweeps(1)
+            rounds.append((g.join(), g.hist, g.k, g.energies, g.info()["carry_energy"]))
+            passes.append(g.info()["last_passes"])
+        out.append(rounds)
+        g.close()
+    _same(*out)
+    assert max(passes) <= 5
