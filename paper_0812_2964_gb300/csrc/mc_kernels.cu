@@ -139,6 +139,13 @@ __global__ void weights_kernel(const DevJob j) {
 // three exponentials a level and beta); 10000 at L = 128 2.4 ms (21).
 constexpr int kThermoThreads = 256;
 constexpr int kThermoParts = 32;          // blocks of the sum over e^{-W}
+// -W as a float: -inf marks a level that was not visited (or has no weight at
+// all), so one too far below for a float is no number -- which passes every
+// test of the FP32 look and leaves the level to FP64.
+__device__ __forceinline__ float thermo_exponent(double w) {
+  const float n = static_cast<float>(-w);
+  return n == -CUDART_INF_F && w < CUDART_INF ? CUDART_NAN_F : n;
+}
 constexpr float kThermoReach = 752.0f;    // e^{-745.2} is the smallest double; the rest covers the FP32 exponents
 
 template <class Op>
@@ -170,12 +177,12 @@ __global__ void __launch_bounds__(kThermoThreads) thermo_norm_kernel(const DevJo
   for (int m = lo + threadIdx.x; m < hi; m += kThermoThreads) {
     const bool on = j.visited[m];
     if (on) bm = fmax(bm, -j.W[m]);
-    neg[m] = on ? static_cast<float>(-j.W[m]) : -CUDART_INF_F;
+    neg[m] = on ? thermo_exponent(j.W[m]) : -CUDART_INF_F;
   }
   const double B = block_tree(bm, sh, MaxOp());
   double sg = 0.0;
   for (int m = lo + threadIdx.x; m < hi; m += kThermoThreads)
-    if (j.visited[m]) sg += exp(-j.W[m] - B);
+    if (j.visited[m] && j.W[m] != CUDART_INF) sg += exp(-j.W[m] - B);   // (a part may hold nothing else)
   const double SG = block_tree(sg, sh, AddOp());
   if (threadIdx.x == 0) {
     out[2 * blockIdx.x] = B;
@@ -205,7 +212,7 @@ __global__ void __launch_bounds__(kThermoThreads) thermo_kernel(const DevJob j, 
     for (int m = t; m < np1; m += kThermoThreads) {
       const bool on = j.visited[m];
       if (on) bm = fmax(bm, -j.W[m]);
-      mine[m] = on ? static_cast<float>(-j.W[m]) : -CUDART_INF_F;
+      mine[m] = on ? thermo_exponent(j.W[m]) : -CUDART_INF_F;
     }
     B = block_tree(bm, sh, MaxOp());
     double sg = 0.0;

@@ -1,9 +1,11 @@
 """Weights far outside a grown job's range: the joints of kept rounds give what
 the replaying joint gives when weights mask levels with huge values, when a
-level no chain visits carries one, and when whole ranges are lifted."""
+level no chain visits carries one, and when whole ranges are lifted; the
+averages of weights that are all huge are the oracle's."""
 import numpy as np
 import pytest
 
+import oracle
 import paper_0812_2964_gb300 as mc
 from paper_0812_2964_gb300.workloads import random_weights
 
@@ -13,6 +15,7 @@ pytestmark = pytest.mark.gpu
 @pytest.fixture(scope="module", autouse=True)
 def _built():
     mc.build()
+    oracle.build()
 
 
 def _rows(up):
@@ -153,3 +156,44 @@ def test_an_undecided_chain_does_not_end_the_scan():
         g.close()
     _same(*out)
     assert max(passes) <= 5
+
+
+@pytest.mark.parametrize("L,n", [(8, 5), (16, 305), (36, 7)])
+@pytest.mark.parametrize("base", [1e39, -1e39, 3.3e38, 1e300])
+def test_thermo_of_huge_weights(L, n, base):
+    N = L * L
+    W = np.full(N + 1, base)
+    W[1::3] = base * (1 + 2.0 ** -50)
+    vis = np.ones(N + 1, np.uint8)
+    vis[::5] = 0
+    betas = np.linspace(0.05, 1.0, n)
+    g = mc.Job(L, 2, 1, 1)
+    g.weights = W
+    g.visited = vis
+    a, b = g.thermo(betas), oracle.thermo(L, W, vis, betas)
+    g.close()
+    assert np.isfinite(b).all()
+    assert np.allclose(a[:, 0], b[:, 0], rtol=1e-10, atol=1e-10 * N)
+    assert np.allclose(a[:, 1], b[:, 1], rtol=1e-9, atol=1e-9 * N)
+    assert np.allclose(a[:, 2], b[:, 2], rtol=1e-10)
+    assert np.allclose(a[:, 3], b[:, 3], rtol=0, atol=1e-10 * max(N, abs(base)))
+
+
+@pytest.mark.parametrize("L,n", [(12, 9), (36, 9), (64, 300)])
+def test_thermo_of_infinite_weights(L, n):
+    # a whole stretch of visited levels without any share: it adds nothing
+    N = L * L
+    W = random_weights(L, 4, 2.0)
+    W[N // 2:3 * N // 4] = np.inf
+    vis = np.ones(N + 1, np.uint8)
+    betas = np.linspace(0.05, 1.0, n)
+    g = mc.Job(L, 2, 1, 1)
+    g.weights = W
+    g.visited = vis
+    a, b = g.thermo(betas), oracle.thermo(L, W, vis, betas)
+    g.close()
+    assert np.isfinite(b).all()
+    assert np.allclose(a[:, 0], b[:, 0], rtol=1e-10, atol=1e-10 * N)
+    assert np.allclose(a[:, 1], b[:, 1], rtol=1e-9, atol=1e-9 * N)
+    assert np.allclose(a[:, 2], b[:, 2], rtol=1e-10)
+    assert np.allclose(a[:, 3], b[:, 3], rtol=0, atol=1e-10 * N)
