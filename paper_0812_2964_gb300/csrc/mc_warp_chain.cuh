@@ -119,9 +119,30 @@ inline void warp_chain_shape(int L, int p, int num_sms, int* warps, bool* tsmem)
 }
 
 // Whether p chains run faster one a warp than one a lane.  The line is drawn
-// in chains per scheduler (p / (4 SMs)); up to 8 are resident.  Measured, ns a
-// site (one a warp / one a lane, rounds of 10 to 200 sweeps, grown weights,
-// 152 SMs):
+// in chains per scheduler (p / (4 SMs)); up to 8 are resident.  A job begins
+// with young weights, whose visited range ends in cliffs: 2 to 4 evaluations a
+// window instead of 1.5, which count where instruction issue is the bound.  So
+// the line is where the first ten iterations from W = 0 together are not
+// slower, and grown weights have room to spare; past it the form lost (L = 16
+// at 4864 36 / 33, L = 48 at 5472 47 / 40, L = 64 at 7296 53 / 41, L = 96 there
+// 53 / 51).  L = 64 between 3600 and 4900 chains is the exception: 28 to 35 /
+// 28 to 31 over ten iterations, even after 24, 1.2 to 1.5 times faster grown
+// (an iteration with its joint is no slower at any of them than it was with
+// one chain a lane and the joint of that time).  Measured, ns a site (one a
+// warp / one a lane, 152 SMs), the mean of a job's first ten iterations:
+//   L = 8     22 / 37 at 1824, 25 / 37 at 2432, 28 / 37 at 3040
+//   L = 12    22 / 34 at 1824, 25 / 34 at 2432
+//   L = 16    20 / 32 at 2432, 28 / 32 at 3648, 31 / 32 at 4256
+//   L = 20    22 / 33 at 2432, 29 / 32 at 3648
+//   L = 28    20 / 31 at 3040, 29 / 31 at 4256, 33 / 31 at 4864
+//   L = 32    25 / 29 at 3648, 29 / 31 at 4864
+//   L = 40    41 / 91 at 4864, 81 / 108 at 8512, 88 / 108 at 9728
+//   L = 48    29 / 47 at 3648, 35 / 51 at 4864
+//   L = 56    54 / 84 at 7296, 83 / 84 at 9728
+//   L = 64    18 / 26 at 2432, 23 / 27 at 3040, 41 / 41 at 5472
+//   L = 76    60 / 79 at 7296, 76 / 79 at 9728
+//   L = 96    35 / 48 at 4864, 48 / 51 at 6080
+// and with grown weights (rounds of 10 to 200 sweeps):
 //   L = 8     16 / 37 at 608 or fewer, 25 / 37 at 2432, 33 / 37 at 3600
 //   L = 12    15 / 33 at 64, 24 / 33 at 2432, 28 / 35 at 3040, 46 / 33 at 4800
 //   L = 16    12 / 33 at 512, 18 / 33 at 2432, 31 / 33 at 4800
@@ -139,9 +160,10 @@ inline bool warp_chain_better(int L, int p, int num_sms) {
   if (L < 8) most = 0;
   else if (L == 8) most = 6;
   else if (L == 12) most = 5;
-  else if (L == 20) most = 7;
-  else if (L == 48 || L == 64 || L == 96) most = 12;          // two waves
-  else if (L > 32 && L <= 100) most = 16;
+  else if (L == 16 || L == 28) most = 7;
+  else if (L == 20) most = 6;
+  else if (L == 64 || L == 96) most = 10;                     // two waves
+  else if (L > 32 && L <= 100 && L != 48) most = 16;
   return p <= most * 4 * num_sms;
 }
 
