@@ -292,7 +292,7 @@ def batch_record(torch, mc, S, steps, warmup, tune, rank=0):
             j.set_trace(True)
             if tune:
                 j.autotune(probe_sweeps=max(1, min(S, 2_000_000 // j.N)))
-        if mode > 0:
+        if mode == 1:
             # shapes of the fused launch from the autotuner (whole-batch probes)
             mc.mc_batch_autotune(jobs, max(1, min(S, 100)))
         mc.mc_batch_run(jobs, warmup, S, mode)
@@ -305,8 +305,12 @@ def batch_record(torch, mc, S, steps, warmup, tune, rank=0):
         launches = mc.mc_kernel_launches() - l0
         kept = sum(j.info()["total_joined"] for j in jobs) - kept0
         attempts = sum(j.p * S * j.N for j in jobs) * steps
-        shapes = ([list(mc.mc_batch_shape(j)[:3]) for j in jobs] if mode > 0 else
-                  [[j.info()[k] for k in ("placement", "chains_per_warp", "warps_per_block")] for j in jobs])
+        if mode == 1:
+            shapes = [list(mc.mc_batch_shape(j)[:3]) for j in jobs]
+        elif mode == 2 and not tune:
+            shapes = "chosen by the library for the set of jobs"
+        else:
+            shapes = [[j.info()[k] for k in ("placement", "chains_per_warp", "warps_per_block")] for j in jobs]
         out[mode] = {"mode": modes[mode], "value": kept / el, "seconds": el, "kept": kept,
                      "raw_attempts_per_s": attempts / el, "gpu_launches": launches, "shapes": shapes}
         for j in jobs:
@@ -315,7 +319,7 @@ def batch_record(torch, mc, S, steps, warmup, tune, rank=0):
             "config": {"workload": "batch_uneven", "groups": [list(g) for g in BATCH_GROUPS],
                        "sweeps_per_iteration": S, "iterations_timed": steps,
                        "fused_shapes": "mc_batch_autotune (whole-batch probes of min(S, 100) sweeps)",
-                       "per_job_shapes": "mc_autotune" if tune else "library default",
+                       "per_job_shapes": "mc_autotune" if tune else "library default (mode 2: for the set of jobs)",
                        "timing": "host wall clock around the synchronising call"},
             "modes": out, "fused_vs_per_job": out[1]["value"] / out[0]["value"],
             "graph_vs_per_job": out[2]["value"] / out[0]["value"], "wall_s": time.perf_counter() - t_wall}

@@ -104,11 +104,10 @@ int mc_run_sweeps(mc_job *job, int64_t n_sweeps);
  * continues across rounds.  Whole sweeps from a sweep boundary take the
  * mc_run_sweeps path; any other round (and any mc_run_sweeps while the
  * chains are inside a sweep) runs one thread per chain on its lattice in
- * global memory (meant for short rounds) and records the level of every
+ * shared memory (meant for short rounds) and records the level of every
  * sample (p * n_attempts int32, see mc_set_partial_record), from which
- * mc_join applies the serial rule chain by chain, each chain's samples
- * tested in parallel; rounds too large to record are joined by replaying
- * each chain in one thread.  No trace is recorded for such a round, and
+ * mc_join settles all chains' inputs at once; rounds too large to record are
+ * joined by replaying each chain in one thread.  No trace is recorded for such a round, and
  * mc_batch_run refuses jobs inside a sweep.  1 <= n_attempts < 2^34.
  * Asynchronous; MC_ESTATE if the previous round has not been joined. */
 int mc_run_attempts(mc_job *job, int64_t n_attempts);
@@ -304,7 +303,8 @@ int mc_set_launch_shape(mc_job *job, int placement, int chains_per_warp, int war
  * side by side, each with its own launches -- the shape it was given, else
  * one chosen for the set of jobs -- and a job's joint beside the others'
  * generation.  Rounds of modes 0 and 2 keep their samples for the joint as
- * mc_run_sweeps's do, where there is memory for it.  The
+ * mc_run_sweeps's do (see mc_set_round_record: up to 16 GiB a job, held until
+ * mc_free), where there is memory for it beside what all jobs need.  The
  * chains, and so every result, are the same in all modes.  Synchronises.
  * No round may be pending on any job.  The paper has no counterpart: a
  * scheduling form of running independent weight estimations together. */
@@ -350,7 +350,8 @@ int mc_sync(mc_job *job);
  * while they run (a host function inside a stream, a process whose device
  * memory is fully reserved up front, a pool that forbids foreign
  * allocations).
- *   d_spins   [n_chains][L][ceil(L/32)] uint32, read and overwritten;
+ *   d_spins   [n_chains][L][ceil(L/32)] uint32, read and overwritten
+ *             (bits past site L - 1 of a row zero);
  *   d_levels  [n_chains] int32, level m = (E + 2N)/4 of each lattice, updated;
  *   d_weights [N+1] double, W = ln w (read);
  *   d_hist    [N+1] int64, zeroed, then the number of this round's samples

@@ -720,7 +720,7 @@ static LaunchShape batch_rule_shape(int L, int p) {
 // Results are identical in all modes.
 static int mc_batch_run_impl(mc_job** jobs, int n_jobs, int iterations, int64_t n_sweeps, int mode) {
   if (!jobs || n_jobs < 1) return fail(MC_EINVAL, "no jobs");
-  if (mode < 0 || mode > 2) return fail(MC_EINVAL, "mode=%d: 0 per-job, 1 fused, 2 fused + graph", mode);
+  if (mode < 0 || mode > 2) return fail(MC_EINVAL, "mode=%d: 0 per-job, 1 fused, 2 a graph branch per job", mode);
   if (iterations < 1) return fail(MC_EINVAL, "iterations=%d", iterations);
   if (mode > 0 && n_jobs > mcgpu::kMaxBatch) return fail(MC_EINVAL, "at most %d jobs per fused batch", mcgpu::kMaxBatch);
   for (int i = 0; i < n_jobs; ++i) {
@@ -1268,6 +1268,7 @@ static int mc_autotune_impl(mc_job* job, int64_t probe_sweeps, int use_cache, in
       for (int c : cpws) {
         LaunchShape s{pl, std::min(32, std::max(1, c)), w};
         if (!mcgpu::shape_supported(job->L, s)) continue;
+        if (pl == mcgpu::kPlaceSmem && s.cpw == 1) s.wpb = 4;   // (one chain a warp: the library sizes the blocks)
         bool dup = false;
         for (const auto& q : cands) dup = dup || (q.placement == s.placement && q.cpw == s.cpw && q.wpb == s.wpb);
         if (!dup) cands.push_back(s);

@@ -163,9 +163,9 @@ cudaError_t k_levels(const DevJob& j, cudaStream_t st);
 cudaError_t k_build_table(const DevJob& j, cudaStream_t st);
 cudaError_t k_update_weights(const DevJob& j, cudaStream_t st);
 // rounds that are not whole sweeps: n attempts per chain from attempt t0
-// (levels recorded in j.plv when `record`), and their joint by the serial
-// rule (M attempts per chain): over the recorded levels, one chain at a time
-// with its samples tested in parallel, else by replay in one thread
+// (levels recorded in j.plv when `record`), and their joint (M attempts per
+// chain): from the recorded levels by heights, one chain after another where
+// an answer is undecided; else by replay in one thread
 cudaError_t k_generate_attempts(const DevJob& j, uint64_t t0, int64_t n, bool record, cudaStream_t st);
 cudaError_t k_join_attempts(const DevJob& j, uint64_t t0, int64_t M, uint32_t r, bool naive, bool recorded,
                             cudaStream_t st);

@@ -541,11 +541,8 @@ __global__ void __launch_bounds__(1024) mark_kernel(const DevJob j, const int de
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    // (a recorded round's summary reads the record and the scan mostly
-    // looks its answers up: whenever a sixteenth of the chains wait, it is
-    // the shorter way)
     const bool deferred = defer && s_count > j.p / 16 &&
-                          (j.rec != nullptr || static_cast<long long>(s_count) * 11 < static_cast<long long>(j.seg_len));
+                          static_cast<long long>(s_count) * 11 < static_cast<long long>(j.seg_len);
     j.stats[kStatPending] = deferred ? 0 : s_count;
     j.stats[kStatFirstPending] = s_first;
     if (s_new) {
