@@ -182,12 +182,12 @@ int mc_set_weights(mc_job *job, const double *w, int n);
 
 /* How the joint resolves wrong speculations (performance only: every
  * policy gives the serial rule's result).  Rounds of at most
- * scan_max_samples samples (all chains; < 0: the default 2e10, no limit for
- * rounds that keep their levels or flips) run
+ * scan_max_samples samples (all chains; < 0: the default 2e10) run
  * passes_before_scan speculative passes, then the summary replay and the
  * exact scan if chains are still pending, then passes_before_scan passes
- * more; larger rounds run passes_without_scan passes; whatever is left goes
- * to the one-block fallback.  Passes in 0..64 (defaults 2 and 10).
+ * more; larger rounds run passes_without_scan passes, and those that keep
+ * their levels or flips, at the default limit, then the exact scan too;
+ * whatever is left goes to the one-block fallback.  Passes in 0..64 (defaults 2 and 10).
  * MC_ESTATE while a round is pending. */
 int mc_set_join_policy(mc_job *job, int64_t scan_max_samples, int passes_before_scan, int passes_without_scan);
 

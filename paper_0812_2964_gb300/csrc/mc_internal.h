@@ -124,12 +124,17 @@ constexpr long long kPartialLevelsMax = 1ll << 26;
 // kmin[] value of a chain with no accepted sample found (yet)
 constexpr unsigned long long kNoHit = 0x7FFFFFFFFFFFFFFFull;
 
-// Whether the job's previous joint rejected so many chains that this one
-// skips its speculative first search (where the caller allows it): with more
-// than p/16 of them, the speculated inputs fail for as many chains and the
-// joint takes the exact path anyway, and the speculative search would have
-// read every rejecting chain whole
-__host__ __device__ inline bool rough_last_joint(long long rejected, int p) { return rejected > p / 16; }
+// Whether the job's previous joint rejected so many chains that a kept round's
+// skips its speculative first search: with more than p/16 of them (p/4 where
+// the levels are rebuilt from flips, and the heights of all chains cost the
+// more), the speculated inputs fail for as many chains and the joint takes the
+// exact path anyway, and the speculative search would have read every
+// rejecting chain whole.  (Flips, p/16 and p/4, joint: L = 64, 1024 chains of
+// 4000 sweeps after one that rejected 132 28 -> 9 ms, 17 replayed; L = 96, 4096
+// of 300 after 326 42 -> 12, 20 replayed.)
+__host__ __device__ inline bool rough_last_joint(const DevJob& j, long long rejected) {
+  return rejected > j.p / (j.flips ? 4 : 16);
+}
 
 enum StatIndex : int {
   kStatCarry = 0,        // level passed on to the next round's chain 0
@@ -204,6 +209,7 @@ enum MarkFlags : int {
   kMarkDefer = 2,       // a speculative pass ahead of the exact path: leave many pending chains to it
   kMarkExactFirst = 4,  // the first search was skipped if the previous joint was rough
   kMarkFinal = 8,       // nothing follows but the fallback: fix the carry and what to count
+  kMarkDeferLate = 16,  // as kMarkDefer, from a quarter of the chains on instead of a sixteenth
 };
 cudaError_t kept_prelude(const DevJob& j, cudaStream_t st);
 cudaError_t kept_mark(const DevJob& j, int64_t S, int flags, cudaStream_t st);

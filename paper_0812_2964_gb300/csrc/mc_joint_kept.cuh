@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(32 * kKeptWarps, 2) kept_search_kernel(const D
                                                           const uint32_t r, const int listed, const int later,
                                                           const int exact_first) {
   after_previous();
-  if (exact_first && rough_last_joint(j.stats[kStatRejected], j.p)) return;   // (the first search only)
+  if (exact_first && rough_last_joint(j, j.stats[kStatRejected])) return;   // (the first search only)
   const int nchains = later ? static_cast<int>(j.stats[kStatNoHit]) : (listed ? static_cast<int>(j.stats[kStatPending]) : j.p);
   const int segs = later ? j.ck_K - 1 : 1;
   const long long items = static_cast<long long>(nchains) * segs;
@@ -505,7 +505,7 @@ inline cudaError_t launch_join_kept(const DevJob& j, const LaunchShape& s, int64
         1, std::min<long long>(blocks_for(n, t.cpw * t.wpb), resident_blocks(kern, 32 * t.wpb, b))));
   };
   const unsigned grid_one = grid(kq, one, one_bytes, j.p), grid_later = grid(kq, all, all_bytes, items);
-  // (the default limit is the replays': a kept round of any size takes the exact path)
+  // (the default limit is the replays': a kept round of any size may take the exact path)
   const bool exact = static_cast<long long>(j.p) * S * j.N <= j.scan_max_samples || j.scan_max_samples == kScanMaxSamples;
   auto search = [&](int listed, int first) -> cudaError_t {
     launch_next(kq, grid_one, 32 * one.wpb, one_bytes, st, j, one.cpw, S, r, listed, 0, first);
@@ -533,7 +533,12 @@ inline cudaError_t launch_join_kept(const DevJob& j, const LaunchShape& s, int64
   if ((e = kept_prelude(j, st)) != cudaSuccess) return e;
   if ((e = search(0, exact ? 1 : 0)) != cudaSuccess) return e;
   if (exact) {
-    if ((e = passes(j.passes_scan, kMarkDefer)) != cudaSuccess) return e;
+    // Passes before the heights: a pass reads the pending chains only, and past the replays' limit the heights
+    // of all chains cost more than the passes that replays take there (L = 64, 4096 chains of 4000 sweeps, 279
+    // rejected: 131 ms with two passes, 53 with up to ten, 50 replayed; L = 128, 1024 of 3000, 160 rejected:
+    // 436, 240, 200)
+    const bool large = static_cast<long long>(j.p) * S * j.N > j.scan_max_samples;
+    if ((e = passes(large ? j.passes_plain : j.passes_scan, large ? kMarkDeferLate : kMarkDefer)) != cudaSuccess) return e;
     if ((e = mark(0)) != cudaSuccess) return e;
     launch_next(kept_seed_kernel<Src>, std::min(2432u, blocks_for(j.p, 4)), 128, 0, st, j, S, r);
     launch_next(kh, grid(kh, all, all_bytes, items), 32 * all.wpb, all_bytes, st, j, all.cpw, S, r);

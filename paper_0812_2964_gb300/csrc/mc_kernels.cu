@@ -885,7 +885,7 @@ __device__ __forceinline__ void kept_mark_body(const DevJob& j, const int64_t M,
     s_new = 0;
     s_kept = 0ull;
   }
-  const bool unsearched = (flags & kMarkExactFirst) && rough_last_joint(j.stats[kStatRejected], j.p);
+  const bool unsearched = (flags & kMarkExactFirst) && rough_last_joint(j, j.stats[kStatRejected]);
   const int n = (flags & kMarkListed) ? static_cast<int>(j.stats[kStatPending]) : j.p;
   for (int q = t; q < n; q += nt) {
     const int i = (flags & kMarkListed) ? j.work[q] : q;
@@ -920,7 +920,7 @@ __device__ __forceinline__ void kept_mark_body(const DevJob& j, const int64_t M,
   if (kept && (t & 31) == 0) atomicAdd(&s_kept, kept);
   __syncthreads();
   if (t == 0) {
-    const bool deferred = (flags & kMarkDefer) && s_count > j.p / 16;
+    const bool deferred = ((flags & kMarkDefer) && s_count > j.p / 16) || ((flags & kMarkDeferLate) && s_count > j.p / 4);
     j.stats[kStatPending] = deferred ? 0 : s_count;
     j.stats[kStatFirstPending] = s_first;
     if (s_new) {

@@ -99,3 +99,32 @@ def test_graph_batch_of_kept_and_replayed_rounds_on_a_users_stream():
         assert np.array_equal(j.spin_words, k.spin_words)
         j.close()
         k.close()
+
+
+def test_a_few_rejections_do_not_send_a_flip_round_to_the_heights():
+    # young weights: once between a sixteenth and a quarter of the chains are rejected, the next joint still
+    # searches first (the scan then settles what the passes left, not every chain), with the replayed results
+    L, p, S = 64, 2048, 1_100
+    assert LIMIT < p * S * L * L < 1.2 * LIMIT
+    rounds = []
+    for replay in (False, True):
+        g = mc.Job(L, p, 3, 1)
+        if replay:
+            g.set_round_record(0)
+        out, before = [], 0
+        for _ in range(6):
+            g.run_sweeps(S)
+            kept = g.join()
+            info = g.info()
+            out.append((kept, g.hist, g.k, info["carry_energy"]))
+            if not replay and p // 16 < before <= p // 4:
+                assert info["last_scanned"] < p
+                out.append("smooth enough")
+            before = info["last_rejected"]
+            g.update_weights()
+        g.close()
+        rounds.append(out)
+    assert "smooth enough" in [x for x in rounds[0] if isinstance(x, str)]
+    for a, b in zip([x for x in rounds[0] if not isinstance(x, str)], rounds[1]):
+        for u, v in zip(a, b):
+            assert np.array_equal(u, v)
