@@ -148,17 +148,28 @@ __device__ __forceinline__ float thermo_exponent(double w) {
 }
 constexpr float kThermoReach = 752.0f;    // e^{-745.2} is the smallest double; the rest covers the FP32 exponents
 
-template <class Op>
-__device__ __forceinline__ double block_tree(double v, double* sh, const Op& op) {
-  const int t = threadIdx.x;
-  for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-  if ((t & 31) == 0) sh[t >> 5] = v;
-  __syncthreads();
-  v = sh[0];
-  for (int w = 1; w < kThermoThreads / 32; ++w) v = op(v, sh[w]);
-  __syncthreads();
-  return v;
-}
+// Sums (or maxima) over the block: every thread's value in shared memory, one
+// warp a quantity takes 8 each and folds them.  12 FP64 instructions a warp and
+// quantity in all; with every warp folding its own and all threads the warps'
+// it was 96, and small lattices, whose blocks do little else, took 107 us for
+// 1000 betas at L = 8 (71 now; 75 before the FP32 look).  (Two in a row need no
+// barrier between them but their own: the values are free once the results are
+// there.)
+struct BlockFold {
+  double v[2][kThermoThreads];
+  double r[2];
+  __device__ __forceinline__ void put(int which, double x) { v[which][threadIdx.x] = x; }
+  // by warp `which` of the block, after a barrier
+  template <class Op>
+  __device__ __forceinline__ double fold(int which, const Op& op) {
+    const int lane = threadIdx.x & 31;
+    double x = v[which][lane];
+    for (int w = 1; w < kThermoThreads / 32; ++w) x = op(x, v[which][lane + 32 * w]);
+    for (int o = 16; o > 0; o >>= 1) x = op(x, __shfl_xor_sync(0xFFFFFFFFu, x, o));
+    if (lane == 0) r[which] = x;
+    return x;
+  }
+};
 struct AddOp {
   __device__ double operator()(double a, double b) const { return a + b; }
 };
@@ -170,7 +181,8 @@ struct MaxOp {
 // relative to that; and -W as a float (-inf: not visited).
 __global__ void __launch_bounds__(kThermoThreads) thermo_norm_kernel(const DevJob j, double* __restrict__ out,
                                                                      float* __restrict__ neg) {
-  __shared__ double sh[kThermoThreads / 32];
+  __shared__ BlockFold f;
+  const int warp = threadIdx.x >> 5;
   const int per = (j.np1 + kThermoParts - 1) / kThermoParts;
   const int lo = blockIdx.x * per, hi = min(j.np1, lo + per);
   double bm = -CUDART_INF;
@@ -179,14 +191,22 @@ __global__ void __launch_bounds__(kThermoThreads) thermo_norm_kernel(const DevJo
     if (on) bm = fmax(bm, -j.W[m]);
     neg[m] = on ? thermo_exponent(j.W[m]) : -CUDART_INF_F;
   }
-  const double B = block_tree(bm, sh, MaxOp());
+  f.put(0, bm);
+  __syncthreads();
+  if (warp == 0) f.fold(0, MaxOp());
+  __syncthreads();
+  const double B = f.r[0];
   double sg = 0.0;
   for (int m = lo + threadIdx.x; m < hi; m += kThermoThreads)
     if (j.visited[m] && j.W[m] != CUDART_INF) sg += exp(-j.W[m] - B);   // (a part may hold nothing else)
-  const double SG = block_tree(sg, sh, AddOp());
-  if (threadIdx.x == 0) {
-    out[2 * blockIdx.x] = B;
-    out[2 * blockIdx.x + 1] = SG;
+  f.put(1, sg);
+  __syncthreads();
+  if (warp == 0) {
+    const double SG = f.fold(1, AddOp());
+    if (threadIdx.x == 0) {
+      out[2 * blockIdx.x] = B;
+      out[2 * blockIdx.x + 1] = SG;
+    }
   }
 }
 
@@ -198,37 +218,28 @@ __global__ void __launch_bounds__(kThermoThreads) thermo_kernel(const DevJob j, 
                                                                 const float* __restrict__ neg_in,
                                                                 double* __restrict__ out) {
   extern __shared__ double terms[];   // [np1], then (OWN) -W as floats
-  __shared__ double sh[kThermoThreads / 32];
-  __shared__ float shf[kThermoThreads / 32];
+  __shared__ BlockFold f;
+  __shared__ float s_am[kThermoThreads / 32], s_big[kThermoThreads / 32];
   __shared__ int s_lo, s_hi;
-  const int t = threadIdx.x, np1 = j.np1, N = j.N;
+  const int t = threadIdx.x, warp = t >> 5, np1 = j.np1, N = j.N;
   const double beta = betas[blockIdx.x];
   const float bf = static_cast<float>(beta);
-  const float* neg = neg_in;
-  double B = 0.0, SG = 0.0;
-  if constexpr (OWN) {
-    float* mine = reinterpret_cast<float*>(terms + np1);
-    double bm = -CUDART_INF;
-    for (int m = t; m < np1; m += kThermoThreads) {
-      const bool on = j.visited[m];
-      if (on) bm = fmax(bm, -j.W[m]);
-      mine[m] = on ? thermo_exponent(j.W[m]) : -CUDART_INF_F;
-    }
-    B = block_tree(bm, sh, MaxOp());
-    double sg = 0.0;
-    for (int m = t; m < np1; m += kThermoThreads)
-      if (j.visited[m]) sg += exp(-j.W[m] - B);
-    SG = block_tree(sg, sh, AddOp());
-    neg = mine;   // (each thread reads its own entries, but for the range below)
-  }
-  if (t == 0) {
-    s_lo = np1;
-    s_hi = 0;
-  }
+  float* mine = reinterpret_cast<float*>(terms + np1);
+  const float* neg = OWN ? mine : neg_in;   // (each thread reads its own entries, but for the range below)
   // largest exponent, in FP32; its rounding, relative to the largest of either part
   float am = -CUDART_INF_F, big = 0.0f;
+  double bm = -CUDART_INF;
   for (int m = t; m < np1; m += kThermoThreads) {
-    const float n = neg[m], e = bf * static_cast<float>(4 * m - 2 * N);
+    float n;
+    if constexpr (OWN) {
+      const bool on = j.visited[m];
+      if (on) bm = fmax(bm, -j.W[m]);
+      n = on ? thermo_exponent(j.W[m]) : -CUDART_INF_F;
+      mine[m] = n;
+    } else {
+      n = neg[m];
+    }
+    const float e = bf * static_cast<float>(4 * m - 2 * N);
     if (n != -CUDART_INF_F) {
       am = fmaxf(am, n - e);
       big = fmaxf(big, fmaxf(fabsf(n), fabsf(e)));
@@ -239,26 +250,40 @@ __global__ void __launch_bounds__(kThermoThreads) thermo_kernel(const DevJob j, 
     big = fmaxf(big, __shfl_xor_sync(0xFFFFFFFFu, big, o));
   }
   if ((t & 31) == 0) {
-    shf[t >> 5] = am;
-    sh[t >> 5] = big;
+    s_am[warp] = am;
+    s_big[warp] = big;
   }
+  if (t == 0) {
+    s_lo = np1;
+    s_hi = 0;
+  }
+  if constexpr (OWN) f.put(0, bm);
   __syncthreads();
   for (int w = 0; w < kThermoThreads / 32; ++w) {
-    am = fmaxf(am, shf[w]);
-    big = fmaxf(big, static_cast<float>(sh[w]));
+    am = fmaxf(am, s_am[w]);
+    big = fmaxf(big, s_big[w]);
+  }
+  double B = 0.0, SG = 0.0;
+  if constexpr (OWN) {
+    if (warp == 0) f.fold(0, MaxOp());
+    __syncthreads();
+    B = f.r[0];
   }
   const float low = am - kThermoReach - big * 0x1p-20f, top = am - 0.5f - big * 0x1p-20f;
   // the levels within reach lie in [lo, hi); the exact largest exponent, among those that may hold it
   int lo = np1, hi = 0;
-  double xm = -CUDART_INF;
+  double xm = -CUDART_INF, sg = 0.0;
   for (int m = t; m < np1; m += kThermoThreads) {
     const float n = neg[m];
     const int E = 4 * m - 2 * N;
     const float x = n - bf * static_cast<float>(E);
-    if (n != -CUDART_INF_F && !(x < low)) {
-      lo = min(lo, m);
-      hi = m + 1;
-      if (!(x < top)) xm = fmax(xm, -j.W[m] - beta * static_cast<double>(E));
+    if (n != -CUDART_INF_F) {
+      if (!(x < low)) {
+        lo = min(lo, m);
+        hi = m + 1;
+        if (!(x < top)) xm = fmax(xm, -j.W[m] - beta * static_cast<double>(E));
+      }
+      if constexpr (OWN) sg += exp(-j.W[m] - B);
     }
   }
   lo = __reduce_min_sync(0xFFFFFFFFu, lo);
@@ -267,8 +292,15 @@ __global__ void __launch_bounds__(kThermoThreads) thermo_kernel(const DevJob j, 
     atomicMin(&s_lo, lo);
     atomicMax(&s_hi, hi);
   }
+  f.put(0, xm);
+  if constexpr (OWN) f.put(1, sg);
   __syncthreads();
-  const double A = block_tree(xm, sh, MaxOp());
+  if (warp == 0) f.fold(0, MaxOp());
+  if constexpr (OWN)
+    if (warp == 1) f.fold(1, AddOp());
+  __syncthreads();
+  const double A = f.r[0];
+  if constexpr (OWN) SG = f.r[1];
   lo = s_lo;
   hi = s_hi;
   double z = 0.0, e1 = 0.0;
@@ -283,9 +315,13 @@ __global__ void __launch_bounds__(kThermoThreads) thermo_kernel(const DevJob j, 
     }
     terms[m] = w;
   }
-  const double Z = block_tree(z, sh, AddOp());
-  const double E1 = block_tree(e1, sh, AddOp());
-  const double Eav = E1 / Z;
+  f.put(0, z);
+  f.put(1, e1);
+  __syncthreads();
+  if (warp == 0) f.fold(0, AddOp());
+  if (warp == 1) f.fold(1, AddOp());
+  __syncthreads();
+  const double Z = f.r[0], Eav = f.r[1] / Z;
   double v = 0.0;
   for (int m = lo + t; m < hi; m += kThermoThreads) {
     const double w = terms[m];
@@ -294,8 +330,10 @@ __global__ void __launch_bounds__(kThermoThreads) thermo_kernel(const DevJob j, 
       v += d * d * w;
     }
   }
-  const double V = block_tree(v, sh, AddOp());
+  f.put(0, v);
+  __syncthreads();
   if (t < 32) {
+    const double V = f.fold(0, AddOp());
     if constexpr (!OWN) {   // ln sum e^{-W} from its parts
       static_assert(kThermoParts == 32, "a lane a part");
       const double b = norm[2 * t], g = norm[2 * t + 1];
