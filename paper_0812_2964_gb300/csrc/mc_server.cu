@@ -128,7 +128,7 @@ int admit_job(mc_server* srv, Rec* r) {
     const mcgpu::LaunchShape d = mcgpu::dense_shape(s.L, s.n_chains, srv->num_sms);
     rc = mc_set_launch_shape(j, d.placement, d.cpw, d.wpb);
   }
-  if (rc == MC_OK && !r->flips) rc = mcgpu::job_drop_flips(j);
+  if (rc == MC_OK && !r->flips && r->full > r->need) rc = mcgpu::job_drop_flips(j);
   if (rc != MC_OK) {
     r->err = mc_last_error();
     if (j) mc_free(j);
